@@ -29,6 +29,7 @@
 #include "activations.cuh"
 #include "forge_common.cuh"
 #include "linear_pair.cuh"
+#include "linear_split.cuh"
 #include "sm100_ptx.cuh"
 #include "tmap.cuh"
 
@@ -399,27 +400,6 @@ int launch_linear(const void* x, const void* w, const void* b, const void* resid
     return finish_launch(1);
 }
 
-template <int ACT, bool F16>
-int launch_layout(int w_layout, const void* x, const void* w, const void* b, const void* r, void* y, int M, int N,
-                  int K, cudaStream_t s) {
-    // This kernel gets the problems with a single row tile (M <= 128): they stream W once and are bound by HBM, so
-    // what counts is how many SMs pull on it.  When 192-column tiles would leave many SMs without one (and W is
-    // large enough for that to matter: small problems are bound by latency, which more and narrower tiles only
-    // add to), narrower tiles with deeper rings spread the same bytes over more of them: the widest of 192, 128
-    // and 64 columns that gives at least three quarters of the SMs a tile, else 64.
-    const int sms = sm_count();
-    const long long w_bytes = 2LL * N * K;
-    if ((N + 191) / 192 < (3 * sms) / 4 && w_bytes >= (16LL << 20)) {
-        if ((N + 127) / 128 >= (3 * sms) / 4)
-            return w_layout == FORGE_W_NK ? launch_linear<128, 5, ACT, true, false, F16>(x, w, b, r, y, M, N, K, s)
-                                          : launch_linear<128, 5, ACT, false, false, F16>(x, w, b, r, y, M, N, K, s);
-        return w_layout == FORGE_W_NK ? launch_linear<64, 8, ACT, true, false, F16>(x, w, b, r, y, M, N, K, s)
-                                      : launch_linear<64, 8, ACT, false, false, F16>(x, w, b, r, y, M, N, K, s);
-    }
-    return w_layout == FORGE_W_NK ? launch_linear<192, 4, ACT, true, false, F16>(x, w, b, r, y, M, N, K, s)
-                                  : launch_linear<192, 4, ACT, false, false, F16>(x, w, b, r, y, M, N, K, s);
-}
-
 template <bool F16>
 int linear_act_impl(const void* x, const void* w, const void* b, const void* residual, void* y,
                     int M, int N, int K, int act, int w_layout, void* stream) {
@@ -431,15 +411,15 @@ int linear_act_impl(const void* x, const void* w, const void* b, const void* res
         return FORGE_ERR_INVALID_ARG;
     if ((K % 8) != 0 || (N % 8) != 0) return FORGE_ERR_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // large outputs run on CTA pairs (see linear_pair.cu); shapes with few tiles stay on the one-CTA kernel
-    if (linear_pair_pays(M, N, sm_count())) return linear_pair(F16, x, w, b, residual, y, M, N, K, act, w_layout, s);
-    switch (act) {
-        case FORGE_ACT_GELU_TANH: return launch_layout<FORGE_ACT_GELU_TANH, F16>(w_layout, x, w, b, residual, y, M, N, K, s);
-        case FORGE_ACT_GELU_ERF: return launch_layout<FORGE_ACT_GELU_ERF, F16>(w_layout, x, w, b, residual, y, M, N, K, s);
-        case FORGE_ACT_RELU: return launch_layout<FORGE_ACT_RELU, F16>(w_layout, x, w, b, residual, y, M, N, K, s);
-        case FORGE_ACT_SILU: return launch_layout<FORGE_ACT_SILU, F16>(w_layout, x, w, b, residual, y, M, N, K, s);
-        default: return launch_layout<FORGE_ACT_NONE, F16>(w_layout, x, w, b, residual, y, M, N, K, s);
-    }
+    const int sms = sm_count();
+    if (sms <= 0) return FORGE_ERR_CUDA;
+    // few tiles: K split over clusters (linear_split.cu); large outputs: CTA pairs (linear_pair.cu)
+    SplitPlan plan;
+    bool split = true;
+    if (M <= kBM) plan = linear_split_plan_row(false, M, N, K, sms);
+    else split = linear_split_plan_rows(M, N, K, sms, &plan);
+    return split ? linear_split(plan, F16, x, w, b, residual, y, M, N, K, act, w_layout, s)
+                 : linear_pair(F16, x, w, b, residual, y, M, N, K, act, w_layout, s);
 }
 
 }  // namespace
@@ -470,11 +450,11 @@ extern "C" int forge_linear_swiglu(const void* x, const void* w_gate, const void
     if (!aligned16(x) || !aligned16(w_gate) || !aligned16(w_up) || !aligned16(y)) return FORGE_ERR_INVALID_ARG;
     if ((K % 8) != 0 || (N % 8) != 0) return FORGE_ERR_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // more than one row tile: CTA pairs (see linear_pair.cu)
-    if (M > 128 && sm_count() >= 2) return linear_pair_swiglu(x, w_gate, w_up, y, M, N, K, w_layout, s);
-    return w_layout == FORGE_W_NK
-               ? launch_linear<256, 3, FORGE_ACT_SILU, true, true>(x, w_gate, nullptr, nullptr, y, M, N, K, s, w_up)
-               : launch_linear<256, 3, FORGE_ACT_SILU, false, true>(x, w_gate, nullptr, nullptr, y, M, N, K, s, w_up);
+    const int sms = sm_count();
+    if (sms <= 0) return FORGE_ERR_CUDA;
+    // more than one row tile: CTA pairs (linear_pair.cu); else the weight-streaming kernel (linear_split.cu)
+    if (M > kBM && sms >= 2) return linear_pair_swiglu(x, w_gate, w_up, y, M, N, K, w_layout, s);
+    return linear_split_swiglu(linear_split_plan_row(true, M, N, K, sms), x, w_gate, w_up, y, M, N, K, w_layout, s);
 }
 
 extern "C" int forge_linear_act_w8a16(const void* x, const void* w_int8, const float* scale, const void* b,

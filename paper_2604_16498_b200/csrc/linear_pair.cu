@@ -379,19 +379,6 @@ int dispatch_act(int act, const void* x, const void* w, const void* b, const voi
 
 }  // namespace
 
-bool linear_pair_pays(int M, int N, int sms) {
-    // Efficiency of a persistent schedule = how full its last round is, times how well the tensor cores are fed:
-    // about 0.61 for the one-CTA kernel (operand reads out of L2), about 0.95 for the pair kernel.
-    auto fill = [](long long tiles, long long workers) {
-        const long long rounds = (tiles + workers - 1) / workers;
-        return (double)tiles / (double)(rounds * workers);
-    };
-    const long long t1 = (long long)((M + 127) / 128) * ((N + 191) / 192);
-    const long long t2 = (long long)((M + 255) / 256) * ((N + 255) / 256);
-    // with a single row tile the second CTA of every pair would work on padding only
-    return sms >= 2 && M > 128 && 0.95 * fill(t2, sms / 2) > 0.61 * fill(t1, sms);
-}
-
 int linear_pair_swiglu(const void* x, const void* w_gate, const void* w_up, void* y, int M, int N, int K, int w_layout,
                        cudaStream_t s) {
     return w_layout == FORGE_W_NK
