@@ -47,4 +47,21 @@ __device__ __forceinline__ float activate(float z) {
     return z;
 }
 
+// The activation chosen at run time, for epilogues that are not worth an instantiation each.
+template <int ACT, int N>
+__device__ __forceinline__ void activate_all(float (&z)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) z[i] = activate<ACT>(z[i]);
+}
+template <int N>
+__device__ __forceinline__ void activate_all(int act, float (&z)[N]) {
+    switch (act) {
+        case FORGE_ACT_GELU_TANH: activate_all<FORGE_ACT_GELU_TANH>(z); break;
+        case FORGE_ACT_GELU_ERF: activate_all<FORGE_ACT_GELU_ERF>(z); break;
+        case FORGE_ACT_RELU: activate_all<FORGE_ACT_RELU>(z); break;
+        case FORGE_ACT_SILU: activate_all<FORGE_ACT_SILU>(z); break;
+        default: break;
+    }
+}
+
 }  // namespace forge

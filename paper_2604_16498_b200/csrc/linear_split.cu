@@ -74,21 +74,6 @@ __device__ __forceinline__ float widen16(uint16_t bits) {
     else return __uint_as_float(static_cast<uint32_t>(bits) << 16);
 }
 
-template <int ACT>
-__device__ __forceinline__ void activate8(float (&z)[8]) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) z[i] = activate<ACT>(z[i]);
-}
-__device__ __forceinline__ void activate8(int act, float (&z)[8]) {
-    switch (act) {
-        case FORGE_ACT_GELU_TANH: activate8<FORGE_ACT_GELU_TANH>(z); break;
-        case FORGE_ACT_GELU_ERF: activate8<FORGE_ACT_GELU_ERF>(z); break;
-        case FORGE_ACT_RELU: activate8<FORGE_ACT_RELU>(z); break;
-        case FORGE_ACT_SILU: activate8<FORGE_ACT_SILU>(z); break;
-        default: break;
-    }
-}
-
 // GATED: tmap_w = gate weights, tmap_w2 = up weights; no bias, residual or activation other than SiLU on the gate.
 template <bool W_NK, bool F16, bool GATED>
 __global__ void __launch_bounds__(kThreads, 2)
@@ -313,7 +298,7 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     } else {
 #pragma unroll
                         for (int k = 0; k < 8; ++k) z[0][k] += s_bias[g * 8 + k];
-                        activate8(p.act, z[0]);
+                        activate_all(p.act, z[0]);
                         const uint32_t rw[4] = {r16.x, r16.y, r16.z, r16.w};
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {

@@ -23,9 +23,9 @@ bool encode_tmap_bf16_sw128(CUtensorMap* map, const void* base, int rank, const 
 bool encode_tmap_bf16_plain(CUtensorMap* map, const void* base, int rank, const uint64_t* dims,
                             const uint64_t* strides_bytes, const uint32_t* box);
 
-// Encodes a tiled tensor map over bytes without swizzle (the tile lands row by row).  box[0] must be a
-// multiple of 16 bytes.  Same conventions and return value as above.
-bool encode_tmap_u8_plain(CUtensorMap* map, const void* base, int rank, const uint64_t* dims,
-                          const uint64_t* strides_bytes, const uint32_t* box);
+// Encodes a tiled tensor map over bytes whose rows of box[0] = 64 bytes land with 64-byte swizzle (16-byte piece c of
+// row r at c ^ (r / 2 % 4)).  Same conventions and return value as above.
+bool encode_tmap_u8_sw64(CUtensorMap* map, const void* base, int rank, const uint64_t* dims,
+                         const uint64_t* strides_bytes, const uint32_t* box);
 
 }  // namespace forge
