@@ -14,7 +14,7 @@
 //               warp of its scheduler: 1.2 % of the kernel)
 //   warp 9    : tcgen05.mma issuer of tile 0 (one elected lane), owns the TMEM allocation
 //   warp 10   : tcgen05.mma issuer of tile 1
-//   warp 11 only completes the third warpgroup, which hands registers to the other two
+//   warp 11   : issues the TMA stores of both tiles' outputs; the third warpgroup hands registers to the other two
 //   (setmaxnreg: 208 per softmax thread, 88 for the rest; 256*208 + 128*88 = 384*168 as launched).
 // Tensor memory (512 columns): S_t at t*128 (half h at +64h, 64 fp32 columns each), O_0 at 256,
 // O_1 at 256 + D.  P (bf16, two per column) of half h is written over the first 32 columns of that
@@ -25,6 +25,12 @@
 // O is rescaled in TMEM only when a row's maximum grows by more than 2^8 (the stale maximum is
 // kept otherwise; the final division by l uses the same reference, so the result is unchanged).
 // Q and K are K-major operands, V [keys, D] is the MN-major B operand of P V.
+// Between items: each tile has two Q buffers, so the issuer sends the first two scores of the next item right behind
+// the last products of this one; the output is staged in the Q buffer of its own item (whose last reader was that item's
+// last S) and stored from there by warp 11, which then hands the buffer back.  A boundary costs the softmax warps
+// about 3100 cycles instead of 4700 (8 x 12 x 1024 x 64 causal 34.1 -> 32.3 us, 18 x 32/8 x 895 x 96 padded 153 -> 149).
+// Reading the output only after the next item's first half-step gained nothing more and cost short items their overlap
+// (64 x 16/4 x 64: 16.7 -> 21.3 us).  At D = 128 long runs are at the power limit: fewer cycles, lower clock.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -48,6 +54,7 @@ constexpr int kThreads = 384;
 constexpr int kTmemCols = 512;
 constexpr int kColS = 0;          // S_t at t * 128
 constexpr int kColO = 256;        // O_t at 256 + t * D
+constexpr int kTakeAhead = 6;     // half-steps before the end of an item's loads at which the next item is taken
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
 #ifndef FORGE_ATTN_FMA_EXP_PAIRS
 #define FORGE_ATTN_FMA_EXP_PAIRS 2
@@ -63,15 +70,14 @@ struct AttnSmem {
     static constexpr int kKVTileBytes = (D / 64) * kKVChunkBytes;
     static constexpr int kKVStages = (D == 64) ? 8 : 3;
     static constexpr int kQOff = 0;
-    static constexpr int kKOff = kQOff + kTilesPerCta * kTileBytes;
+    static constexpr int kKOff = kQOff + 2 * kTilesPerCta * kTileBytes;  // two Q buffers per tile
     static constexpr int kVOff = kKOff + kKVStages * kKVTileBytes;
-    // output staging: 32 rows x 64 bf16 per softmax warp and 64-column block of D
-    static constexpr int kOutOff = kVOff + kKVStages * kKVTileBytes;
-    static constexpr int kOutWarpBytes = (D / 64) * 4096;
-    static constexpr int kBarOff = kOutOff + 8 * kOutWarpBytes;
-    // q_full[2], q_empty[2], k/v full+empty per stage, s_full[4], p_ready[4], pv_done[4], o_free[2]
-    static constexpr int kNumBars = 4 + 4 * kKVStages + 14;
-    static constexpr int kTotal = kBarOff + kNumBars * 8 + 16;
+    static constexpr int kBarOff = kVOff + kKVStages * kKVTileBytes;
+    // q_full[4], q_empty[4], k/v full+empty per stage, s_full[4], p_ready[4], pv_done[4], o_free[2], next_full[2],
+    // next_empty[2], taken, o_staged[4]
+    static constexpr int kNumBars = 8 + 4 * kKVStages + 23;
+    static constexpr int kNextOff = kBarOff + (kNumBars * 8 + 15) / 16 * 16;  // the launch queue's answer, two items
+    static constexpr int kTotal = kNextOff + 16 + 2 * 64 + 16;
     static constexpr int kAlloc = kTotal + 1024;
 };
 
@@ -167,6 +173,7 @@ struct AttnParams {
     FastDiv div_heads;  // by the number of items per query step
     FastDiv div_inner;  // by the head pairs (or heads) per batch entry
     FastDiv div_group;  // by the query heads per KV head
+    int sms;
     int* status;
 };
 
@@ -196,9 +203,9 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     uint8_t* sK = smem + L::kKOff;
     uint8_t* sV = smem + L::kVOff;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
-    uint64_t* q_full = bars;                 // [2] per query tile
-    uint64_t* q_empty = bars + 2;            // [2]
-    uint64_t* k_full = bars + 4;
+    uint64_t* q_full = bars;                 // [4] query tile t, buffer u at t * 2 + u
+    uint64_t* q_empty = bars + 4;            // [4] the output that was staged in the buffer has left it
+    uint64_t* k_full = bars + 8;
     uint64_t* k_empty = k_full + kKVStages;
     uint64_t* v_full = k_empty + kKVStages;
     uint64_t* v_empty = v_full + kKVStages;
@@ -206,7 +213,14 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     uint64_t* p_ready = s_full + 4;          // [4]
     uint64_t* pv_done = p_ready + 4;         // [4] one completion per P V product of that tile and half
     uint64_t* o_free = pv_done + 4;          // [2] per query tile
-    uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(o_free + 2);
+    uint64_t* next_full = o_free + 2;        // [2] the next item is in shared memory (two places in turn)
+    uint64_t* next_empty = next_full + 2;    // [2] both issuers, the eight softmax warps and the store warp have read it
+    uint64_t* taken = next_empty + 2;        // the launch queue has answered
+    uint64_t* o_staged = taken + 1;          // [4] the tile's output lies in its Q buffer, ready to be stored
+    uint8_t* next_answer = smem + L::kNextOff;
+    // [2][16]: 1 or 0 (no item), then b, kvlen, n_max, q0[2], h[2], nh[2] as in ItemInfo
+    volatile int* next_items = reinterpret_cast<int*>(smem + L::kNextOff + 16);
+    uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(smem + L::kNextOff + 16 + 2 * 64);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // The two tiles of an item: with an even number of query heads per KV head, the same 128 query rows of
@@ -229,13 +243,12 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     const int causal_off = p.Skv - p.Sq;
     const bool causal = (p.mask_kind & FORGE_MASK_CAUSAL) != 0;
 
-    // Persistent schedule.  Items are ordered longest first (the last query-tile pair of every head, then
-    // the one before, ...); CTA c takes item c of every round of gridDim.x items, in alternating direction
-    // from round to round, which keeps the per-CTA sums of causal work close together.
-    auto item_of_round = [&](int r) {
-        const int c = (r & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x;
-        return r * (int)gridDim.x + c;
-    };
+    // Dynamic schedule.  The grid has one CTA per item, ordered longest first (the last query-tile pair of every head, then
+    // the one before, ...); a CTA that nears the end of its item takes the next one that has not started yet out of the
+    // launch queue, so whoever is done first gets it, whatever the items cost (padding, ragged tiles).  Against a fixed
+    // order (item c of every round to CTA c, in alternating direction): 8 x 16/4 heads x 1000 x 1700 with lengths from 300
+    // 74 -> 66 us, 2 x 28/4 x 2048 causal 65.6 -> 62.7, 8 x 12 x 1024 causal (an even load) 34.5 -> 34.1.
+    const bool dynamic = num_items > p.sms;  // else everything runs at once and nothing is left to take
     auto decode = [&](int i) {
         ItemInfo it;
         const int round_q = fast_div(i, p.div_heads);
@@ -269,9 +282,17 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         }
         return it;
     };
+    // The n-th item after the first, worked out by the producer and read by everyone else from next_items[n % 2]: 1 if there
+    // is one, 0: no more work, -1: gave up.
+    auto next_item = [&](int n) -> int {
+        if (!dynamic) return 0;
+        if (!mbar_wait(&next_full[n & 1], (n >> 1) & 1)) return -1;
+        return next_items[(n & 1) * 16];
+    };
 
     if (threadIdx.x == 0) {
-        for (int t = 0; t < 2; ++t) { mbar_init(&q_full[t], 1); mbar_init(&q_empty[t], 1); }
+        for (int i = 0; i < 4; ++i) { mbar_init(&q_full[i], 1); mbar_init(&q_empty[i], 1); mbar_init(&o_staged[i], 4); }
+        mbar_init(taken, 1);
         // a shared K/V stage is released by both tiles' issuer threads, a private one by its own
         const uint32_t releases = two_streams ? 1 : 2;
         for (int i = 0; i < kKVStages; ++i) {
@@ -279,7 +300,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
             mbar_init(&v_full[i], 1); mbar_init(&v_empty[i], releases);
         }
         for (int i = 0; i < 4; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_ready[i], 4); mbar_init(&pv_done[i], 1); }
-        for (int t = 0; t < 2; ++t) mbar_init(&o_free[t], 4);
+        for (int t = 0; t < 2; ++t) { mbar_init(&o_free[t], 4); mbar_init(&next_full[t], 1); mbar_init(&next_empty[t], 11); }
         fence_mbar_init();
         prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_o);
     }
@@ -304,39 +325,53 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         if (elect_one()) {
             int kvn[2] = {0, 0};     // KV tiles loaded so far per stream (ring position), across items
             int q_loads[2] = {0, 0}; // Q tiles loaded so far per query tile
-            for (int r = 0; !failed; ++r) {
-                const int i = item_of_round(r);
-                if (i >= num_items) break;
-                const ItemInfo it = decode(i);
-                if (it.n_max == 0) continue;
+            auto load_q = [&](const ItemInfo& x) -> bool {
 #pragma unroll
                 for (int t = 0; t < kTilesPerCta; ++t) {
-                    if (it.nh[t] == 0) continue;
-                    // the tile's last S = Q K^T of its previous item has completed: Q may be replaced
-                    if (!mbar_wait_relaxed(&q_empty[t], (q_loads[t] & 1) ^ 1)) { failed = true; break; }
+                    if (x.nh[t] == 0) continue;
+                    const int u = q_loads[t] & 1, at = t * 2 + u;
+                    if (!mbar_wait_relaxed(&q_empty[at], ((q_loads[t] >> 1) & 1) ^ 1)) return false;
                     ++q_loads[t];
-                    mbar_expect_tx(&q_full[t], L::kTileBytes);
+                    mbar_expect_tx(&q_full[at], L::kTileBytes);
 #pragma unroll
                     for (int c = 0; c < D / 64; ++c)  // rows beyond Sq are zero-filled by the TMA unit
-                        tma_load_4d(sQ + t * L::kTileBytes + c * L::kChunkBytes, &tmap_q, &q_full[t], c * 64,
-                                    it.q0[t], it.h[t], it.b);
+                        tma_load_4d(sQ + at * L::kTileBytes + c * L::kChunkBytes, &tmap_q, &q_full[at], c * 64, x.q0[t], x.h[t], x.b);
                 }
-                // The next item's Q tiles are asked into L2 now, a whole item ahead: Q can only be copied to
-                // shared memory once this item's last scores are done, and a copy that then has to come from
-                // HBM leaves the tensor core idle for a microsecond or two at every item boundary.
-                {
-                    const int i_next = item_of_round(r + 1);
-                    if (i_next < num_items) {
-                        const ItemInfo nx = decode(i_next);
-#pragma unroll
-                        for (int t = 0; t < kTilesPerCta; ++t) {
-                            if (nx.nh[t] == 0) continue;
-#pragma unroll
-                            for (int c = 0; c < D / 64; ++c) tma_prefetch_l2_4d(&tmap_q, c * 64, nx.q0[t], nx.h[t], nx.b);
-                        }
-                    }
+                return true;
+            };
+            ItemInfo it = decode(blockIdx.x), nx = it;
+            if (!load_q(it)) failed = true;
+            bool more = true;
+            for (int r = 0; more && !failed; ++r) {
+                more = false;
+                // takes the next item out of the launch queue / publishes it
+                auto request_next = [&]() {
+                    mbar_expect_tx(taken, 16);
+                    clc_try_cancel(next_answer, taken);
+                };
+                auto receive_next = [&]() -> bool {
+                    if (!mbar_wait(taken, r & 1)) return false;
+                    const int x = clc_taken(next_answer);
+                    fence_proxy_async_smem();  // the next answer is written to this place by another proxy
+                    more = x >= 0;
+                    if (more) nx = decode(x);
+                    if (!mbar_wait_relaxed(&next_empty[r & 1], ((r >> 1) & 1) ^ 1)) return false;
+                    volatile int* to = next_items + (r & 1) * 16;
+                    to[0] = more ? 1 : 0; to[1] = nx.b; to[2] = nx.kvlen; to[3] = nx.n_max;
+                    to[4] = nx.q0[0]; to[5] = nx.q0[1]; to[6] = nx.h[0]; to[7] = nx.h[1]; to[8] = nx.nh[0]; to[9] = nx.nh[1];
+                    mbar_arrive(&next_full[r & 1]);
+                    return true;
+                };
+                if (it.n_max == 0 && dynamic) {
+                    request_next();
+                    if (!receive_next()) failed = true;
                 }
+                // Late enough that the item goes to whoever is done first, early enough that its Q tiles, which are loaded behind
+                // this item's last K/V tiles, are in shared memory before the last products of this one are out.
+                const int j_request = max(0, it.n_max - kTakeAhead), j_receive = max(0, it.n_max - kTakeAhead / 2);
                 for (int j = 0; j < it.n_max && !failed; ++j) {
+                    if (dynamic && j == j_request) request_next();
+                    if (dynamic && j == j_receive && !receive_next()) { failed = true; break; }
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         if (u == 1 && !two_streams) continue;
@@ -358,6 +393,10 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                                         j * kHalf, kvh, it.b);
                     }
                 }
+                // (The buffer is free once the output staged in it has left, which happens after the first half-step of this item,
+                // whose K/V tiles have all been loaded.)
+                if (!failed && more && !load_q(nx)) failed = true;
+                it = nx;
             }
         }
       } else if (warp <= 10) {
@@ -367,107 +406,154 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
             const int u = two_streams ? t : 0;
             constexpr uint32_t idesc_s = F16 ? make_idesc_f16(kBM, kHalf, false, false) : make_idesc_bf16(kBM, kHalf, false, false);
             constexpr uint32_t idesc_o = F16 ? make_idesc_f16(kBM, D, false, true) : make_idesc_bf16(kBM, D, false, true);
-            const uint32_t q_addr = smem_u32(sQ) + t * L::kTileBytes, k_addr = smem_u32(sK), v_addr = smem_u32(sV);
+            const uint32_t q_addr = smem_u32(sQ) + 2 * t * L::kTileBytes, k_addr = smem_u32(sK), v_addr = smem_u32(sV);
             const uint32_t s_tmem = tmem_base + kColS + t * kBN, o_tmem = tmem_base + kColO + t * D;
             // descriptors differ only in the start-address field: build one per operand, then add
             // (byte offset >> 4) for each step (the field cannot overflow below 256 KB)
-            const uint64_t qd = make_smem_desc(q_addr, 16, 1024);
+            const uint64_t qd0 = make_smem_desc(q_addr, 16, 1024);
             int kvbase = 0;      // ring position of the item's first KV tile in this tile's stream
-            int q_uses = 0;      // items in which this tile had work (phases of q_full, o_free)
-            int steps0 = 0, steps1 = 0;  // half-steps issued so far per half (phases of p_ready)
+            int q_uses = 0;      // items in which this tile had work (Q buffers, phases of q_full, o_free)
+            int steps = 0;       // half-steps of earlier items (step s uses half s % 2 of S_t, phase s / 2)
+            int primed = 0;      // scores of the current item that were issued during the previous one
 
-            ItemInfo it;
-            int i_cur = item_of_round(0);
-            if (i_cur < num_items) it = decode(i_cur);
-            for (int r = 0; !failed && i_cur < num_items; ++r) {
-                const int i_next = item_of_round(r + 1);
-                ItemInfo it_next;
-                if (it.n_max == 0) {
-                    if (i_next < num_items) it_next = decode(i_next);
-                    it = it_next; i_cur = i_next;
-                    continue;
-                }
-                const int nh = pick(it.nh, t);
-
-                // A barrier poll costs a few hundred cycles even on a completed phase, so the operands of a step
-                // (V(g) for the product, K(g + 2) for the next scores) are waited for before the probabilities,
-                // while this thread has nothing to issue; once P(g) arrives the MMAs go out back to back.
-                auto wait_k = [&](int g) -> bool {
-                    const int pos = kvbase + g;
-                    return mbar_wait(&k_full[kv_slot(u, pos)], kv_phase(pos));
-                };
-                auto wait_v = [&](int g) -> bool {
-                    const int pos = kvbase + g;
-                    return mbar_wait(&v_full[kv_slot(u, pos)], kv_phase(pos));
-                };
-                // S(g) = Q K(g)^T into half g % 2 of S_t (K(g) has landed)
-                auto issue_qk = [&](int g) -> bool {
-                    const int hh = g & 1, pos = kvbase + g, st = kv_slot(u, pos);
-                    tc_fence_after_sync();
-                    const uint64_t kd = make_smem_desc(k_addr + st * L::kKVTileBytes, 16, 1024);
+            // A barrier poll costs a few hundred cycles even on a completed phase, so the operands of a step
+            // (V(g) for the product, K(g + 2) for the next scores) are waited for before the probabilities,
+            // while this thread has nothing to issue; once P(g) arrives the MMAs go out back to back.
+            auto wait_k = [&](int pos) -> bool { return mbar_wait(&k_full[kv_slot(u, pos)], kv_phase(pos)); };
+            auto wait_v = [&](int pos) -> bool { return mbar_wait(&v_full[kv_slot(u, pos)], kv_phase(pos)); };
+            auto wait_q = [&](int use) -> bool { return mbar_wait(&q_full[t * 2 + (use & 1)], (use >> 1) & 1); };
+            // S(step) = Q K(pos)^T into half step % 2 of S_t (Q and K have landed)
+            auto issue_qk = [&](int use, int step, int pos) {
+                const int hh = step & 1, st = kv_slot(u, pos);
+                tc_fence_after_sync();
+                const uint64_t qd = qd0 + (use & 1) * (L::kTileBytes >> 4);
+                const uint64_t kd = make_smem_desc(k_addr + st * L::kKVTileBytes, 16, 1024);
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk) {
-                        const uint32_t qoff = ((kk / 4) * L::kChunkBytes + (kk % 4) * 32) >> 4;
-                        const uint32_t koff = ((kk / 4) * L::kKVChunkBytes + (kk % 4) * 32) >> 4;
-                        mma_ss(s_tmem + hh * kHalf, qd + qoff, kd + koff, idesc_s, kk != 0);
-                    }
-                    mma_commit(&s_full[t * 2 + hh]);
-                    mma_commit(&k_empty[st]);                  // this tile is done with the K tile
-                    if (g == nh - 1) mma_commit(&q_empty[t]);  // and, after the item's last S, with Q
-                    return true;
-                };
-                // O_t += P(g) V(g) with P read from tensor memory (V(g) has landed)
-                auto issue_pv = [&](int g) -> bool {
-                    const int hh = g & 1, pos = kvbase + g, st = kv_slot(u, pos);
-                    if (!mbar_wait(&p_ready[t * 2 + hh], (hh ? steps1 : steps0) & 1)) return false;
-                    if (hh) ++steps1; else ++steps0;
-                    // the first product of an item overwrites O_t: the previous item's epilogue must have read it
-                    if (g == 0 && !mbar_wait(&o_free[t], (q_uses & 1) ^ 1)) return false;
-                    tc_fence_after_sync();
-                    // P: 16 keys = 8 columns of packed bf16 pairs.  V: MN-major, 16 keys = two 1024-byte groups
-                    // (2048 bytes per step); the 64-wide chunks of D are 8 KB apart.
-                    const uint64_t vd = make_smem_desc(v_addr + st * L::kKVTileBytes, L::kKVChunkBytes, 1024);
-                    const uint32_t p_tmem = s_tmem + hh * kHalf;
-                    if (g == 0) mma_ts(o_tmem, p_tmem, vd, idesc_o, 0u);
-                    else mma_ts(o_tmem, p_tmem, vd, idesc_o, 1u);
+                for (int kk = 0; kk < D / 16; ++kk) {
+                    const uint32_t qoff = ((kk / 4) * L::kChunkBytes + (kk % 4) * 32) >> 4;
+                    const uint32_t koff = ((kk / 4) * L::kKVChunkBytes + (kk % 4) * 32) >> 4;
+                    mma_ss(s_tmem + hh * kHalf, qd + qoff, kd + koff, idesc_s, kk != 0);
+                }
+                mma_commit(&s_full[t * 2 + hh]);
+                mma_commit(&k_empty[st]);                  // this tile is done with the K tile
+            };
+            // O_t += P(g) V(g) with P read from tensor memory (V(g) has landed)
+            auto issue_pv = [&](int g) -> bool {
+                const int step = steps + g, hh = step & 1, st = kv_slot(u, kvbase + g);
+                if (!mbar_wait(&p_ready[t * 2 + hh], (step >> 1) & 1)) return false;
+                // the first product of an item overwrites O_t: the previous item's epilogue must have read it
+                if (g == 0 && !mbar_wait(&o_free[t], (q_uses & 1) ^ 1)) return false;
+                tc_fence_after_sync();
+                // P: 16 keys = 8 columns of packed bf16 pairs.  V: MN-major, 16 keys = two 1024-byte groups
+                // (2048 bytes per step); the 64-wide chunks of D are 8 KB apart.
+                const uint64_t vd = make_smem_desc(v_addr + st * L::kKVTileBytes, L::kKVChunkBytes, 1024);
+                const uint32_t p_tmem = s_tmem + hh * kHalf;
+                if (g == 0) mma_ts(o_tmem, p_tmem, vd, idesc_o, 0u);
+                else mma_ts(o_tmem, p_tmem, vd, idesc_o, 1u);
 #pragma unroll
-                    for (int kk = 1; kk < kHalf / 16; ++kk) mma_ts(o_tmem, p_tmem + kk * 8, vd + kk * (2048 >> 4), idesc_o, 1u);
-                    mma_commit(&pv_done[t * 2 + hh]);
-                    mma_commit(&v_empty[st]);
-                    return true;
-                };
+                for (int kk = 1; kk < kHalf / 16; ++kk) mma_ts(o_tmem, p_tmem + kk * 8, vd + kk * (2048 >> 4), idesc_o, 1u);
+                mma_commit(&pv_done[t * 2 + hh]);
+                mma_commit(&v_empty[st]);
+                return true;
+            };
 
-                if (nh > 0) {
-                    if (!mbar_wait(&q_full[t], q_uses & 1)) { failed = true; break; }
-                    if (!wait_k(0) || !issue_qk(0)) { failed = true; break; }
-                    if (nh > 1 && (!wait_k(1) || !issue_qk(1))) { failed = true; break; }
+            int nh, n_max;
+            {
+                const ItemInfo it = decode(blockIdx.x);
+                nh = pick(it.nh, t);
+                n_max = it.n_max;
+            }
+            int state = 1;
+            for (int r = 0; state == 1; ++r) {
+                // Where this tile reads every K/V tile of the item, the first scores of the next item are issued behind the last
+                // products of this one, so the softmax warps go on without a gap.  (Otherwise the tiles that only the
+                // other query tile reads have to be released first, or the ring would not reach the next item.)
+                const bool look_ahead = nh > 0 && (two_streams || nh == n_max);
+                const int next_base = kvbase + (two_streams ? nh : n_max);
+                int have_next = 0, ahead = 0, next_nh = 0;
+                for (int g = primed; g < min(nh, 2); ++g) {
+                    if ((g == 0 && !wait_q(q_uses)) || !wait_k(kvbase + g)) { state = -1; break; }
+                    issue_qk(q_uses, steps + g, kvbase + g);
                 }
-                // the next item's coordinates, worked out while the softmax warps are busy with the first S
-                if (i_next < num_items) it_next = decode(i_next);
-                if (nh > 0) {
-                    for (int g = 0; g < nh; ++g) {
-                        if (!wait_v(g) || (g + 2 < nh && !wait_k(g + 2))) { failed = true; break; }
-                        if (!issue_pv(g)) { failed = true; break; }
-                        if (g + 2 < nh && !issue_qk(g + 2)) { failed = true; break; }
+                for (int g = 0; g < nh && state == 1; ++g) {
+                    if (!wait_v(kvbase + g) || (g + 2 < nh && !wait_k(kvbase + g + 2)) || !issue_pv(g)) { state = -1; break; }
+                    if (g + 2 < nh) {
+                        issue_qk(q_uses, steps + g + 2, kvbase + g + 2);
+                    } else if (look_ahead) {
+                        if (!have_next) {
+                            const int more = next_item(r);
+                            if (more == -1) { state = -1; break; }
+                            have_next = 1;
+                            next_nh = more == 1 ? next_items[(r & 1) * 16 + 8 + t] : 0;
+                            if (next_nh > 0 && !wait_q(q_uses + 1)) { state = -1; break; }
+                        }
+                        if (ahead < next_nh) {
+                            if (!wait_k(next_base + ahead)) { state = -1; break; }
+                            issue_qk(q_uses + 1, steps + nh + ahead, next_base + ahead);
+                            ++ahead;
+                        }
                     }
-                    if (failed) break;
-                    ++q_uses;
                 }
-                if (two_streams) {
-                    kvbase += nh;
-                } else {
+                if (state == -1) break;
+                if (!two_streams) {
                     // K/V tiles that only the other query tile reads: release them once they have landed
-                    for (int j = nh; j < it.n_max; ++j) {
+                    for (int j = nh; j < n_max; ++j) {
                         const int pos = kvbase + j, st = kv_slot(0, pos);
-                        if (!mbar_wait(&k_full[st], kv_phase(pos))) { failed = true; break; }
+                        if (!wait_k(pos)) { state = -1; break; }
                         mbar_arrive(&k_empty[st]);
-                        if (!mbar_wait(&v_full[st], kv_phase(pos))) { failed = true; break; }
+                        if (!wait_v(pos)) { state = -1; break; }
                         mbar_arrive(&v_empty[st]);
                     }
-                    kvbase += it.n_max;
+                    if (state == -1) break;
                 }
-                it = it_next; i_cur = i_next;
+                if (nh > 0) ++q_uses;
+                steps += nh;
+                kvbase = next_base;
+                primed = ahead;
+                state = next_item(r);
+                if (state == 1) {
+                    nh = next_items[(r & 1) * 16 + 8 + t];
+                    n_max = next_items[(r & 1) * 16 + 3];
+                    mbar_arrive(&next_empty[r & 1]);
+                }
             }
+            if (state == -1) failed = true;
+        }
+      } else {
+        // ------------------------------------------------------------------ output stores
+        if (elect_one()) {
+            int uses[2] = {0, 0};  // items in which the tile had work
+            int nh[2], q0[2], h[2], b;
+            {
+                const ItemInfo it = decode(blockIdx.x);
+                nh[0] = it.nh[0]; nh[1] = it.nh[1]; q0[0] = it.q0[0]; q0[1] = it.q0[1]; h[0] = it.h[0]; h[1] = it.h[1]; b = it.b;
+            }
+            int state = 1;
+            for (int r = 0; state == 1; ++r) {
+#pragma unroll
+                for (int t = 0; t < kTilesPerCta; ++t) {
+                    if (nh[t] == 0 || state != 1) continue;
+                    // (one barrier per buffer: the output of the last item may be ready before the one before it has been looked at)
+                    const int at = t * 2 + (uses[t] & 1);
+                    if (!mbar_wait_relaxed(&o_staged[at], (uses[t] >> 1) & 1)) { state = -1; continue; }
+                    ++uses[t];
+#pragma unroll
+                    for (int c = 0; c < D / 64; ++c)  // rows beyond Sq are clipped by the TMA unit
+                        tma_store_4d(&tmap_o, sQ + at * L::kTileBytes + c * L::kChunkBytes, c * 64, q0[t], h[t], b);
+                    tma_store_commit();
+                    tma_store_wait_read<0>();
+                    mbar_arrive(&q_empty[at]);  // the producer may load Q there again
+                }
+                if (state != 1) break;
+                state = next_item(r);
+                if (state == 1) {
+                    volatile const int* x = next_items + (r & 1) * 16;
+                    b = x[1]; q0[0] = x[4]; q0[1] = x[5]; h[0] = x[6]; h[1] = x[7]; nh[0] = x[8]; nh[1] = x[9];
+                    mbar_arrive(&next_empty[r & 1]);
+                }
+            }
+            if (state == -1) failed = true;
+            tma_store_wait_all<0>();  // every output tile has left shared memory and is written
         }
       }
     } else {
@@ -480,44 +566,91 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         const uint32_t col_s = kColS + t * kBN, col_o = kColO + t * D;
         const float sl2 = p.scale_log2;
         const float2 sl2v = make_float2(sl2, sl2);
-        uint8_t* stage_out = smem + L::kOutOff + warp * L::kOutWarpBytes;  // this warp's 32 rows x 128 bytes per block
-        int steps0 = 0, steps1 = 0;  // half-steps done so far per half (barrier phases run across items)
+        int steps = 0;               // half-steps of earlier items (step s uses half s % 2 of S_t, phase s / 2)
+        int q_uses = 0;              // earlier items in which this tile had work: they use the two Q buffers in turn
         const int u = two_streams ? t : 0;  // K/V stream of this tile
         int kvbase = 0;              // ring position of the item's first KV tile in that stream
         const bool padding = (p.mask_kind & FORGE_MASK_PADDING) != 0;
+        // The output of an item is read from tensor memory at the start of the next one (or of a last, empty pass): by then its
+        // last products are done, and the next item's first scores have been issued behind them.
+        bool pending = false;
+        float out_inv = 0.f;
 
-        ItemInfo it;
-        int i_cur = item_of_round(0);
-        if (i_cur < num_items) it = decode(i_cur);
-        for (int r = 0; !failed && i_cur < num_items; ++r) {
-            const int i_next = item_of_round(r + 1);
-            ItemInfo it_next;
-            const int q0 = pick(it.q0, t);
+        int nh, q0, head, b, kvlen, n_max;
+        {
+            const ItemInfo it = decode(blockIdx.x);
+            nh = pick(it.nh, t); q0 = pick(it.q0, t); head = pick(it.h, t);
+            b = it.b; kvlen = it.kvlen; n_max = it.n_max;
+        }
+        for (int r = 0, state = 1; !failed; ++r) {
             const int qi = q0 + row;
-            const int nh = pick(it.nh, t);
-            const int head = pick(it.h, t);
-            if (nh == 0) {  // no visible key for any row of this tile (or the tile lies beyond Sq)
-                if (qi < p.Sq) {
-                    uint16_t* orow = p.out + it.b * p.o_sb + head * p.o_sh + qi * p.o_ss;
-                    for (int c = 0; c < p.head_dim / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = make_uint4(0, 0, 0, 0);
-                }
-                if (i_next < num_items) it_next = decode(i_next);
-                if (!two_streams) kvbase += it.n_max;  // the tiles the other query tile of the item reads
-                it = it_next; i_cur = i_next;
-                continue;
-            }
             float m_run = -INFINITY;  // running maximum of the raw scores (reference of the exponentials)
             float l_run = 0.f;
             // last visible key of this row
-            const int row_limit = min(it.kvlen - 1, causal ? qi + causal_off : 0x7fffffff);
+            const int row_limit = min(kvlen - 1, causal ? qi + causal_off : 0x7fffffff);
+            if (pending) {
+                // The last product of that item (its barrier's phase before it was covered by the last S barrier seen).
+                if (!warp_wait(&pv_done[t * 2 + ((steps - 1) & 1)], ((steps - 1) >> 1) & 1)) { failed = true; break; }
+                tc_fence_after_sync();
+                // O / l as bf16 through 128-byte-swizzled staging rows (32 rows x 64 columns per block of D) in the item's own Q
+                // buffer, whose last reader was the item's last S, and one TMA store per block; rows beyond Sq are clipped
+                // by the TMA unit.  A short rolled loop: its footprint matters more than its issue count.
+                uint8_t* stage_out = sQ + (t * 2 + ((q_uses - 1) & 1)) * L::kTileBytes + quarter * 4096;
+                uint32_t cur[32];
+                tmem_ld_x32(lane_base + col_o, cur);
 #pragma unroll 1
-            for (int g = 0; g < nh; ++g) {
-                const int hh = g & 1;
+                for (int c32 = 0; c32 < D / 32; ++c32) {
+                    tmem_ld_wait();
+                    uint32_t w[16];
+#pragma unroll
+                    for (int k = 0; k < 16; ++k)
+                        w[k] = pack16<F16>(__uint_as_float(cur[2 * k]) * out_inv, __uint_as_float(cur[2 * k + 1]) * out_inv);
+                    if (c32 + 1 < D / 32) tmem_ld_x32(lane_base + col_o + (c32 + 1) * 32, cur);
+                    // 32 columns = four 16-byte chunks of this row's 128-byte line in block c32 / 2
+                    uint8_t* line = stage_out + (c32 >> 1) * L::kChunkBytes + lane * 128;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        *reinterpret_cast<uint4*>(line + ((((c32 & 1) * 4 + c) ^ (lane & 7)) << 4)) =
+                            make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+                }
+                // O_t is in shared memory: the issuer may overwrite it, the store warp may send it off
+                tc_fence_before_sync();
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) { mbar_arrive(&o_free[t]); mbar_arrive(&o_staged[t * 2 + ((q_uses - 1) & 1)]); }
+                pending = false;
+            }
+            if (state != 1) break;
+            // One half-step.  At D = 64 the first one of an item has code of its own, without the votes and branches that its
+            // state decides (34.0 -> 32.3 us at 8 x 12 x 1024); at D = 128 and with a bias the second copy of the code
+            // costs as much as it saves.
+            constexpr bool kOwnFirst = D == 64 && !BIAS;
+            auto do_step = [&](auto first_tag, int g) -> bool {
+                constexpr bool kFirst = decltype(first_tag)::value;
+                const int step = steps + g, hh = step & 1;
                 const uint32_t col_h = col_s + hh * kHalf;
+                const int key0 = g * kHalf;
+                // The bias of this row and half-step is on its way while the scores are waited for (4 x 16 heads x 700 x 900, a
+                // bias per head: 68.9 -> 48.4 us).
+                [[maybe_unused]] float bias[BIAS ? kHalf : 1];
+                if constexpr (BIAS) {
+                    const int hb = p.bias_heads == 1 ? 0 : head;
+                    const float* brow = p.bias + (((size_t)b * p.bias_heads + hb) * p.Sq + min(qi, p.Sq - 1)) * (size_t)p.Skv + key0;
+                    const int nvalid = min(kHalf, p.Skv - key0);  // columns beyond Skv are masked below
+                    if ((p.Skv & 3) == 0) {  // rows start on 16-byte boundaries
+#pragma unroll
+                        for (int c = 0; c < kHalf / 4; ++c) {
+                            const float4 bv = c * 4 < nvalid ? __ldg(reinterpret_cast<const float4*>(brow) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            bias[4 * c] = bv.x; bias[4 * c + 1] = bv.y; bias[4 * c + 2] = bv.z; bias[4 * c + 3] = bv.w;
+                        }
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < kHalf; ++k) bias[k] = k < nvalid ? __ldg(brow + k) : 0.f;
+                    }
+                }
                 // S(g) is complete, and so is every MMA this tile's issuer issued before it: O_t holds the
                 // P V products up to g - 2 and P(g - 2) has been consumed.
-                if (!warp_wait(&s_full[t * 2 + hh], (hh ? steps1 : steps0) & 1)) { failed = true; break; }
-                if (hh) ++steps1; else ++steps0;
+                if (!warp_wait(&s_full[t * 2 + hh], (step >> 1) & 1)) return false;
                 tc_fence_after_sync();
                 float s[kHalf];
 #pragma unroll
@@ -529,30 +662,12 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 }
                 tmem_ld_wait();
 
-                const int key0 = (g >> 1) * kBN + hh * kHalf;
-                const bool need_mask = (key0 + kHalf > it.kvlen) || (causal && (key0 + kHalf - 1 > q0 + causal_off)) ||
+                const bool need_mask = (key0 + kHalf > kvlen) || (causal && (key0 + kHalf - 1 > q0 + causal_off)) ||
                                        BIAS;  // a bias may hold -inf: the path that tolerates it
                 if constexpr (BIAS) {
                     // Eq. 8's mask node as a tensor: scale * s + bias = scale * (s + bias / scale)
-                    const int hb = p.bias_heads == 1 ? 0 : pick(it.h, t);
-                    const float* brow = p.bias + (((size_t)it.b * p.bias_heads + hb) * p.Sq + min(qi, p.Sq - 1)) * (size_t)p.Skv + key0;
-                    const int nvalid = min(kHalf, p.Skv - key0);  // columns beyond Skv are masked below
-                    if ((p.Skv & 3) == 0) {  // rows start on 16-byte boundaries
 #pragma unroll
-                        for (int c = 0; c < kHalf / 4; ++c) {
-                            if (c * 4 < nvalid) {
-                                const float4 bv = __ldg(reinterpret_cast<const float4*>(brow) + c);
-                                s[4 * c] = fmaf(bv.x, p.inv_scale, s[4 * c]);
-                                s[4 * c + 1] = fmaf(bv.y, p.inv_scale, s[4 * c + 1]);
-                                s[4 * c + 2] = fmaf(bv.z, p.inv_scale, s[4 * c + 2]);
-                                s[4 * c + 3] = fmaf(bv.w, p.inv_scale, s[4 * c + 3]);
-                            }
-                        }
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < kHalf; ++k)
-                            if (k < nvalid) s[k] = fmaf(__ldg(brow + k), p.inv_scale, s[k]);
-                    }
+                    for (int k = 0; k < kHalf; ++k) s[k] = fmaf(bias[k], p.inv_scale, s[k]);
                 }
                 bool stored = false;
                 if (need_mask) {
@@ -574,7 +689,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 // current reference in the same pass that finds the maximum.  Valid as long as no row's
                 // maximum exceeds its reference by more than the threshold, which is what the lazy rescale
                 // tolerates anyway; otherwise the half is redone below with a new reference.
-                if (!stored && __all_sync(0xffffffffu, m_run != -INFINITY)) {
+                if (!kFirst && !stored && __all_sync(0xffffffffu, m_run != -INFINITY)) {
                     auto fast_path = [&](auto fma_tag) {
                         constexpr bool kUseFma = decltype(fma_tag)::value;
                         const float2 neg_m = make_float2(-m_run * sl2, -m_run * sl2);
@@ -626,10 +741,10 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                         alpha = (m_run == -INFINITY) ? 1.f : ex2((m_run - m_tile) * sl2);
                         m_run = m_tile;
                     }
-                    if (g > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
+                    if (!kFirst && (kOwnFirst || g > 0) && __any_sync(0xffffffffu, alpha != 1.f)) {
                         // O_t must hold every product issued so far and none may be in flight: the product of
                         // half-step g - 1 (the other half's latest) is the only one the barrier above does not cover.
-                        if (!warp_wait(&pv_done[t * 2 + (hh ^ 1)], ((hh ? steps0 : steps1) - 1) & 1)) { failed = true; break; }
+                        if (!warp_wait(&pv_done[t * 2 + (hh ^ 1)], ((step - 1) >> 1) & 1)) return false;
                         tc_fence_after_sync();
                         // rare after the first steps: small chunks, not unrolled, to keep register pressure low
 #pragma unroll 1
@@ -663,10 +778,10 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 // anything; their probabilities are exactly 0, but 0 x NaN is NaN on the tensor core.  The four
                 // warps of the tile zero those rows in shared memory before the product is allowed to start (the
                 // issuer needs all four arrivals below).  Rows beyond Skv were zero-filled by the copy itself.
-                if (padding && key0 + kHalf > it.kvlen && it.kvlen < p.Skv) {
+                if (padding && key0 + kHalf > kvlen && kvlen < p.Skv) {
                     const int pos = kvbase + g, st = kv_slot(u, pos);
-                    if (!warp_wait(&v_full[st], kv_phase(pos))) { failed = true; break; }
-                    const int first = max(it.kvlen - key0, 0);       // first padded row of this tile
+                    if (!warp_wait(&v_full[st], kv_phase(pos))) return false;
+                    const int first = max(kvlen - key0, 0);       // first padded row of this tile
                     const int per_chunk = (kHalf - first) * 8;        // 16-byte pieces to clear per 64-column chunk
                     uint8_t* vt = sV + st * L::kKVTileBytes;
                     for (int i = quarter * 32 + lane; i < (D / 64) * per_chunk; i += 128) {
@@ -680,57 +795,37 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&p_ready[t * 2 + hh]);  // one arrival per warp
+                return true;
+            };
+            int g = 0;
+            if constexpr (kOwnFirst) {
+                if (nh > 0 && !do_step(std::true_type{}, 0)) { failed = true; break; }
+                g = 1;
             }
-            if (failed) break;
-            // the next item's coordinates, worked out while the last products are still running
-            if (i_next < num_items) it_next = decode(i_next);
-            // The last product of either half (every S barrier seen covers that half's product before the
-            // latest, so each wait is at most one completion behind and the phase parity identifies it).
-            if (steps0 > 0 && !warp_wait(&pv_done[t * 2], (steps0 - 1) & 1)) { failed = true; break; }
-            if (steps1 > 0 && !warp_wait(&pv_done[t * 2 + 1], (steps1 - 1) & 1)) { failed = true; break; }
-            tc_fence_after_sync();
-            // O / l as bf16 through this warp's 128-byte-swizzled staging rows (32 rows x 64 columns per
-            // block of D) and one TMA store per block; rows beyond Sq are clipped by the TMA unit.  A short
-            // rolled loop: the code runs once per item, so its footprint matters more than its issue count.
-            {
-                const float inv = l_run > 0.f ? 1.f / l_run : 0.f;  // no visible key: zeros
-                if (lane == 0) tma_store_wait_read<0>();  // the previous item's stores have read the staging rows
-                __syncwarp();
-                uint32_t cur[32];
-                tmem_ld_x32(lane_base + col_o, cur);
 #pragma unroll 1
-                for (int c32 = 0; c32 < D / 32; ++c32) {
-                    tmem_ld_wait();
-                    uint32_t w[16];
-#pragma unroll
-                    for (int k = 0; k < 16; ++k)
-                        w[k] = pack16<F16>(__uint_as_float(cur[2 * k]) * inv, __uint_as_float(cur[2 * k + 1]) * inv);
-                    if (c32 + 1 < D / 32) tmem_ld_x32(lane_base + col_o + (c32 + 1) * 32, cur);
-                    // 32 columns = four 16-byte chunks of this row's 128-byte line in block c32 / 2
-                    uint8_t* line = stage_out + (c32 >> 1) * 4096 + lane * 128;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        *reinterpret_cast<uint4*>(line + ((((c32 & 1) * 4 + c) ^ (lane & 7)) << 4)) =
-                            make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-                }
-                // O_t is in shared memory: hand it back to the issuer before the stores go out
-                tc_fence_before_sync();
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(&o_free[t]);
-                    const int row0 = q0 + quarter * 32;
-                    if (row0 < p.Sq) {
-#pragma unroll
-                        for (int cb = 0; cb < D / 64; ++cb) tma_store_4d(&tmap_o, stage_out + cb * 4096, cb * 64, row0, head, it.b);
-                        tma_store_commit();
-                    }
-                }
+            for (; g < nh; ++g)
+                if (!do_step(std::false_type{}, g)) { failed = true; break; }
+            if (failed) break;
+            if (nh > 0) {
+                pending = true;
+                out_inv = l_run > 0.f ? 1.f / l_run : 0.f;  // no visible key: zeros
+                ++q_uses;
+                steps += nh;
+            } else if (qi < p.Sq) {  // no visible key for any row of this tile
+                uint16_t* orow = p.out + b * p.o_sb + head * p.o_sh + qi * p.o_ss;
+                for (int c = 0; c < p.head_dim / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = make_uint4(0, 0, 0, 0);
             }
-            kvbase += two_streams ? nh : it.n_max;
-            it = it_next; i_cur = i_next;
+            kvbase += two_streams ? nh : n_max;
+            state = next_item(r);
+            if (__any_sync(0xffffffffu, state < 0)) { failed = true; break; }  // the same for every lane of the warp
+            nh = 0;                // after the last item: one more pass, for its output
+            if (state == 1) {
+                volatile const int* x = next_items + (r & 1) * 16;
+                b = x[1]; kvlen = x[2]; n_max = x[3]; q0 = x[4 + t]; head = x[6 + t]; nh = x[8 + t];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&next_empty[r & 1]);
+            }
         }
-        if (lane == 0) tma_store_wait_all<0>();  // every output tile has left shared memory and is written
     }
 
     if (failed) {
@@ -773,7 +868,7 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
     if (!encode(&tq, q, Hq, Sq, sq, 128)) return FORGE_ERR_CUDA;
     if (!encode(&tk, k, Hkv, Skv, sk, kHalf)) return FORGE_ERR_CUDA;
     if (!encode(&tv, v, Hkv, Skv, sv, kHalf)) return FORGE_ERR_CUDA;
-    if (!encode(&to, out, Hq, Sq, so, 32)) return FORGE_ERR_CUDA;  // the output leaves in boxes of 32 rows, one per softmax warp
+    if (!encode(&to, out, Hq, Sq, so, 128)) return FORGE_ERR_CUDA;
     AttnParams p;
     p.out = static_cast<uint16_t*>(out);
     p.o_sb = so.b; p.o_sh = so.h; p.o_ss = so.s;
@@ -805,8 +900,8 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
     const bool head_pairs = ((Hq / Hkv) % 2 == 0) || L::kKVStages >= 8;  // same rule as in the kernel
     const long long items = head_pairs ? (long long)((Hq + 1) / 2) * B * q_tiles
                                        : (long long)Hq * B * ((q_tiles + 1) / 2);
-    const int grid = items < sms ? (int)items : sms;
-    FORGE_CUDA_TRY(launch_pdl(kernel, dim3(grid), dim3(kThreads), L::kAlloc, s, tq, tk, tv, to, p));
+    p.sms = sms;
+    FORGE_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)items), dim3(kThreads), L::kAlloc, s, tq, tk, tv, to, p));
     return finish_launch(1);
 }
 

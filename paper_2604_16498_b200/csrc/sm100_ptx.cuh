@@ -360,6 +360,30 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar, uint16_t cta_mask
                  : "memory");
 }
 
+// ----------------------------------------------------------------- dynamic schedule (cluster launch control)
+// Takes a CTA of this grid that has not started yet out of the launch queue, if there is one: 16 bytes of response arrive
+// at `response` (shared memory, 16-byte aligned) and are counted on `bar`.  Not to be called again after a refusal.
+__device__ __forceinline__ void clc_try_cancel(void* response, uint64_t* bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 ::"r"(smem_u32(response)), "r"(smem_u32(bar))
+                 : "memory");
+}
+// The x index of the CTA that was taken, or -1.
+__device__ __forceinline__ int clc_taken(const void* response) {
+    uint32_t ok, x;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\t.reg .b128 R;\n\t"
+        "ld.shared.b128 R, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 P, R;\n\t"
+        "selp.u32 %0, 1, 0, P;\n\t"
+        "mov.u32 %1, 0;\n\t"
+        "@P clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, R;\n\t}"
+        : "=r"(ok), "=r"(x)
+        : "r"(smem_u32(response))
+        : "memory");
+    return ok ? (int)x : -1;
+}
+
 // ----------------------------------------------------------------- TMEM <-> registers
 // 32x32b shape: thread t of the warp reads lane (32 * (warp % 4) + t); register i is column (col + i).
 __device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, uint32_t (&r)[32]) {

@@ -1,0 +1,55 @@
+"""GPU parity: 16-bit attention with more work items than SMs, where a CTA takes items out of the launch queue, loads the next
+item's Q and issues its first scores behind the last products of the current one.  Items of very different cost side by
+side: empty sequences, one key, one half-step, several; odd head counts (the second tile of an item is absent), odd
+group sizes (two consecutive tiles of a head, the last one beyond Sq), rows that see no key.  fp64 oracle; runs are equal
+bit for bit whatever CTA took which item."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2604_16498_b200 import binding, workloads as wl
+from util import Guarded, assert_close_bf16, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Skv,D,mask,lens", [
+    (40, 8, 8, 130, 200, 64, 2, [0, 1, 63, 64, 65, 128, 129, 200]),     # private K/V streams, empty items among full ones
+    (24, 15, 15, 100, 70, 64, 3, [70, 1, 0, 64]),                       # odd head count; rows without a visible key
+    (30, 7, 1, 260, 333, 128, 3, [333, 10, 0, 64, 100]),                # odd group: three tiles of a head in two items
+    (50, 8, 2, 40, 300, 128, 2, [300, 0, 1, 65, 257]),                  # one tile per head, pairs of heads
+    (64, 12, 12, 128, 128, 64, 1, None),                                # two half-steps each
+    (20, 10, 2, 300, 300, 96, 1, None),
+])
+def test_many_uneven_items(B, Hq, Hkv, Sq, Skv, D, mask, lens):
+    w = wl.attention_workload("t", 71, B, Hq, Hkv, Sq, Skv, D, mask, 1.0 / np.sqrt(D), "bf16", lens_range=(1, Skv))
+    dl = None
+    if lens is not None:
+        w.lens = np.array((lens * B)[:B], dtype=np.int32)
+        dl = torch.from_numpy(w.lens).cuda()
+    q, k, v = to_device(w.q), to_device(w.k), to_device(w.v)
+    g = Guarded((B, Hq, Sq, D), torch.bfloat16)
+    binding.attn_fused(q, k, v, mask, dl, w.scale, out=g.tensor)
+    binding.check_status()
+    pick = np.unique(np.concatenate([np.arange(min(B, 8)), [B - 1]]))  # the oracle checks a period of the lengths and the last entry
+    ref = oracle.attn(w.q.values[pick], w.k.values[pick], w.v.values[pick], mask, w.lens[pick] if lens is not None else None, w.scale)
+    assert_close_bf16(g.tensor[torch.from_numpy(pick).cuda()], ref)
+    g.assert_intact()
+    assert torch.isfinite(g.tensor.float()).all()
+    for _ in range(10):
+        assert torch.equal(binding.attn_fused(q, k, v, mask, dl, w.scale), g.tensor)
+    binding.check_status()
+
+
+def test_many_items_with_a_bias():
+    """The bias of a half-step is read ahead; -inf entries, ragged keys, more items than SMs."""
+    B, H, Sq, Skv, D = 12, 16, 200, 201, 64
+    w = wl.attention_workload("t", 72, B, H, H, Sq, Skv, D, wl.MASK_CAUSAL, 0.125, "bf16")
+    bias = wl.normal_tensor(wl.seed_for(72, "b"), (B, 1, Sq, Skv), "f32").values.copy()
+    bias[:, :, ::3, 5:70] = -np.inf
+    got = binding.attn_fused_bias(to_device(w.q), to_device(w.k), to_device(w.v), torch.from_numpy(bias.astype(np.float32)).cuda(),
+                                  wl.MASK_CAUSAL, None, 0.125)
+    binding.check_status()
+    ref = oracle.attn_bias(w.q.values[:3], w.k.values[:3], w.v.values[:3], bias[:3].astype(np.float64), wl.MASK_CAUSAL, None, 0.125)
+    assert_close_bf16(got[:3], ref)
