@@ -360,15 +360,21 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                     to[0] = more ? 1 : 0; to[1] = nx.b; to[2] = nx.kvlen; to[3] = nx.n_max;
                     to[4] = nx.q0[0]; to[5] = nx.q0[1]; to[6] = nx.h[0]; to[7] = nx.h[1]; to[8] = nx.nh[0]; to[9] = nx.nh[1];
                     mbar_arrive(&next_full[r & 1]);
+                    // its Q tiles are asked into L2 while their buffer may still be in use
+#pragma unroll
+                    for (int t = 0; t < kTilesPerCta; ++t) {
+                        if (!more || nx.nh[t] == 0) continue;
+#pragma unroll
+                        for (int c = 0; c < D / 64; ++c) tma_prefetch_l2_4d(&tmap_q, c * 64, nx.q0[t], nx.h[t], nx.b);
+                    }
                     return true;
                 };
-                if (it.n_max == 0 && dynamic) {
-                    request_next();
-                    if (!receive_next()) failed = true;
-                }
                 // Late enough that the item goes to whoever is done first, early enough that its Q tiles, which are loaded behind
-                // this item's last K/V tiles, are in shared memory before the last products of this one are out.
-                const int j_request = max(0, it.n_max - kTakeAhead), j_receive = max(0, it.n_max - kTakeAhead / 2);
+                // this item's last K/V tiles, are in shared memory before the last products of this one are out.  The answer
+                // of the launch queue is not waited for before the first K/V tiles are on their way.
+                const int j_request = max(0, it.n_max - kTakeAhead);
+                const int j_receive = it.n_max > kTakeAhead / 2 ? it.n_max - kTakeAhead / 2 : it.n_max;
+                if (dynamic && it.n_max == 0) request_next();
                 for (int j = 0; j < it.n_max && !failed; ++j) {
                     if (dynamic && j == j_request) request_next();
                     if (dynamic && j == j_receive && !receive_next()) { failed = true; break; }
@@ -393,8 +399,8 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                                         j * kHalf, kvh, it.b);
                     }
                 }
-                // (The buffer is free once the output staged in it has left, which happens after the first half-step of this item,
-                // whose K/V tiles have all been loaded.)
+                if (dynamic && !failed && j_receive == it.n_max && !receive_next()) failed = true;
+                // (The buffer is free once the output that was staged in it at the start of this item has left.)
                 if (!failed && more && !load_q(nx)) failed = true;
                 it = nx;
             }
@@ -480,16 +486,15 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                     if (g + 2 < nh) {
                         issue_qk(q_uses, steps + g + 2, kvbase + g + 2);
                     } else if (look_ahead) {
-                        if (!have_next) {
-                            const int more = next_item(r);
-                            if (more == -1) { state = -1; break; }
+                        // only what is there already: the products still to come must not wait for the next item
+                        if (!have_next && dynamic && mbar_test(&next_full[r & 1], (r >> 1) & 1)) {
                             have_next = 1;
-                            next_nh = more == 1 ? next_items[(r & 1) * 16 + 8 + t] : 0;
-                            if (next_nh > 0 && !wait_q(q_uses + 1)) { state = -1; break; }
+                            next_nh = next_items[(r & 1) * 16] ? next_items[(r & 1) * 16 + 8 + t] : 0;
                         }
-                        if (ahead < next_nh) {
-                            if (!wait_k(next_base + ahead)) { state = -1; break; }
-                            issue_qk(q_uses + 1, steps + nh + ahead, next_base + ahead);
+                        const int pos = next_base + ahead, use = q_uses + 1;
+                        if (ahead < next_nh && mbar_test(&q_full[t * 2 + (use & 1)], (use >> 1) & 1) &&
+                            mbar_test(&k_full[kv_slot(u, pos)], kv_phase(pos))) {
+                            issue_qk(use, steps + nh + ahead, pos);
                             ++ahead;
                         }
                     }
