@@ -374,7 +374,9 @@ int launch_split(const SplitPlan& plan, const void* x, const void* w, const void
     // an MMA reads 128 rows of A, also where the X tile is shorter
     if (total < (stages - 1) * stage_bytes + kABytes) total = (stages - 1) * stage_bytes + kABytes;
     total += 1024;  // slack to align the base
-    p.prefetch = plan.two_per_sm;
+    const long long ctas = (long long)((M + kBM - 1) / kBM) * ((N + bno - 1) / bno) * S;
+    if (ctas > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
+    p.prefetch = plan.two_per_sm || ctas * 2 <= sm_count();
     p.status = device_status_word();
     if (!p.status) return FORGE_ERR_CUDA;
 
@@ -395,8 +397,6 @@ int launch_split(const SplitPlan& plan, const void* x, const void* w, const void
     if (!GATED) tmap_w2 = tmap_w;
     auto kernel = linear_split_kernel<W_NK, F16, GATED>;
     FORGE_SET_SMEM_ONCE(kernel, kSmemWhole);
-    const long long ctas = (long long)((M + kBM - 1) / kBM) * ((N + bno - 1) / bno) * S;
-    if (ctas > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
     FORGE_CUDA_TRY(launch_pdl_cluster(kernel, dim3((unsigned)ctas), dim3(kThreads), total, S, s, tmap_x, tmap_w, tmap_w2, p));
     return finish_launch(1);
 }
