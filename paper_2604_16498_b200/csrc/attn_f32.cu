@@ -190,8 +190,11 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
         __syncthreads();  // V has landed (and P is complete)
         if (work) {
             const float* vr = sV + ks * T::KW * D + kg * 4;
+            // A hidden key has a probability of exactly 0, but 0 x NaN is NaN: a warp stops at the last key that any of its 16 rows
+            // sees.  (With 16 rows per CTA the copy stops there already.)
+            const int nk = T::BM > 16 ? min(T::KW, kv_end_warp - key0) : T::KW;
 #pragma unroll 4
-            for (int j = 0; j < T::KW; ++j) {
+            for (int j = 0; j < nk; ++j) {
                 const float4 pv = *reinterpret_cast<const float4*>(sP + j * kPStride + rg * 4);
                 const float pr[4] = {pv.x, pv.y, pv.z, pv.w};
 #pragma unroll

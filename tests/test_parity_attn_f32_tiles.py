@@ -35,3 +35,22 @@ def test_tiles(B, Hq, Hkv, Sq, Skv, D, mask, lens):
     binding.check_status()
     assert_close_f32(g.tensor, ref)
     g.assert_intact()
+
+
+@pytest.mark.parametrize("B,H,Sq,Skv,D", [
+    (1, 2, 100, 100, 64), (1, 2, 70, 133, 128),          # 16-row CTAs
+    (8, 32, 100, 100, 64), (8, 32, 100, 137, 64), (8, 32, 70, 71, 128),  # 64-row CTAs
+])
+def test_a_later_v_row_reaches_no_earlier_tile_of_16_queries(B, H, Sq, Skv, D):
+    """NaN and Inf in V rows that the causal mask hides from every query of a 16-row tile leave that tile as it is, bit for
+    bit, wherever the row lies among the keys that a warp takes at once."""
+    w = wl.attention_workload("t", 62, B, H, H, Sq, Skv, D, wl.MASK_CAUSAL, 1.0 / np.sqrt(D), "f32")
+    q, k, v = to_device(w.q), to_device(w.k), to_device(w.v)
+    clean = binding.attn_fused_f32(q, k, v, wl.MASK_CAUSAL, None, w.scale)
+    for first_hidden in range(16, Sq, 16):        # the tile of queries first_hidden - 16 .. first_hidden - 1
+        dirty = v.clone()
+        dirty[:, :, first_hidden + Skv - Sq::2] = float("nan")
+        dirty[:, :, first_hidden + Skv - Sq + 1::2] = float("inf")
+        out = binding.attn_fused_f32(q, k, dirty, wl.MASK_CAUSAL, None, w.scale)
+        assert torch.equal(out[:, :, :first_hidden], clean[:, :, :first_hidden])
+    binding.check_status()
