@@ -10,7 +10,8 @@
 //   KSPLIT = 8: 16 query rows per CTA, 16 keys of a 128-key tile per warp: shortest chain, most CTAs
 //   KSPLIT = 2: 64 query rows per CTA, 32 keys of a 64-key tile per warp: K and V are copied a quarter as often
 // Thread = rows 4 (lane / 8) .. + 3 of its warp's 16, keys lane % 8 + 8 j; in P V the same rows, head columns
-// 4 (lane % 8) .. + 3 and + 32 h.
+// 4 (lane % 8) .. + 3 and + 32 h.  Q is multiplied by scale * log2(e) on its way to shared memory, so that products which fp32
+// holds only after scaling do not overflow before it.
 // 12 heads, D = 64, causal, cold inputs, against 16-row CTAs of four warps with one row x 8 keys per thread: 1 x 128
 // 12.1 -> 7.0 us, 3 x 200 42.7 -> 18.7 us, 8 x 512 278 -> 122 us; error against fp64 2.1e-7 -> 1.5e-7 (shorter sums).
 #include "forge_common.cuh"
@@ -101,9 +102,32 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
     const float* kb = k + (size_t)(b * Hkv + kvh) * Skv * D;
     const float* vb = v + (size_t)(b * Hkv + kvh) * Skv * D;
 
-    for (int idx = tid; idx < T::BM * (D / 4); idx += kThreads) {
-        const int r = idx / (D / 4), c = idx % (D / 4);
-        cp_async16(sQ + r * LD + c * 4, qb + (q0 + r < Sq ? (size_t)r * D + c * 4 : 0), q0 + r < Sq);
+    // keys at and beyond kv_end are zero-filled, never read (padding may hold anything)
+    auto copy_tile = [&](int j0) {
+        for (int idx = tid; idx < T::BN * (D / 4); idx += kThreads) {
+            const int r = idx / (D / 4), c = idx % (D / 4);
+            cp_async16(sK + r * LD + c * 4, kb + (j0 + r < kv_end ? (size_t)(j0 + r) * D + c * 4 : 0), j0 + r < kv_end);
+        }
+        cp_async_commit();
+        for (int idx = tid; idx < T::BN * (D / 4); idx += kThreads) {
+            const int r = idx / (D / 4), c = idx % (D / 4);
+            cp_async16(sV + r * D + c * 4, vb + (j0 + r < kv_end ? (size_t)(j0 + r) * D + c * 4 : 0), j0 + r < kv_end);
+        }
+        cp_async_commit();
+    };
+    constexpr int kQPieces = T::BM * (D / 4) / kThreads;
+    float4 qpiece[kQPieces];
+#pragma unroll
+    for (int i = 0; i < kQPieces; ++i) {
+        const int idx = i * kThreads + tid, r = idx / (D / 4), c = idx % (D / 4);
+        qpiece[i] = q0 + r < Sq ? *reinterpret_cast<const float4*>(qb + (size_t)r * D + c * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (kv_end > 0) copy_tile(0);
+#pragma unroll
+    for (int i = 0; i < kQPieces; ++i) {
+        const int idx = i * kThreads + tid, r = idx / (D / 4), c = idx % (D / 4);
+        *reinterpret_cast<float4*>(sQ + r * LD + c * 4) =
+            make_float4(qpiece[i].x * scale_log2, qpiece[i].y * scale_log2, qpiece[i].z * scale_log2, qpiece[i].w * scale_log2);
     }
 
     float m_run[4], l_run[4];
@@ -117,18 +141,10 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
     }
 
     for (int j0 = 0; j0 < kv_end; j0 += T::BN) {
-        if (j0 > 0) __syncthreads();  // the previous tile has been consumed
-        // keys at and beyond kv_end are zero-filled, never read (padding may hold anything)
-        for (int idx = tid; idx < T::BN * (D / 4); idx += kThreads) {
-            const int r = idx / (D / 4), c = idx % (D / 4);
-            cp_async16(sK + r * LD + c * 4, kb + (j0 + r < kv_end ? (size_t)(j0 + r) * D + c * 4 : 0), j0 + r < kv_end);
+        if (j0 > 0) {
+            __syncthreads();  // the previous tile has been consumed
+            copy_tile(j0);
         }
-        cp_async_commit();
-        for (int idx = tid; idx < T::BN * (D / 4); idx += kThreads) {
-            const int r = idx / (D / 4), c = idx % (D / 4);
-            cp_async16(sV + r * D + c * 4, vb + (j0 + r < kv_end ? (size_t)(j0 + r) * D + c * 4 : 0), j0 + r < kv_end);
-        }
-        cp_async_commit();
         cp_async_wait<1>();
         __syncthreads();
         const int key0 = j0 + ks * T::KW;
@@ -163,7 +179,7 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
                 float s[NJ], m_tile = -INFINITY;
 #pragma unroll
                 for (int j = 0; j < NJ; ++j) {
-                    s[j] = key0 + kg + 8 * j <= limit ? (s2[i][j].x + s2[i][j].y) * scale_log2 : -INFINITY;
+                    s[j] = key0 + kg + 8 * j <= limit ? s2[i][j].x + s2[i][j].y : -INFINITY;
                     m_tile = fmaxf(m_tile, s[j]);
                 }
 #pragma unroll
@@ -209,7 +225,6 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
             }
         }
     }
-    cp_async_wait<0>();  // also where no tile was read: Q is still on its way
 
     // Merge the KSPLIT warps of every 16 rows.
 #pragma unroll

@@ -54,3 +54,17 @@ def test_a_later_v_row_reaches_no_earlier_tile_of_16_queries(B, H, Sq, Skv, D):
         out = binding.attn_fused_f32(q, k, dirty, wl.MASK_CAUSAL, None, w.scale)
         assert torch.equal(out[:, :, :first_hidden], clean[:, :, :first_hidden])
     binding.check_status()
+
+
+@pytest.mark.parametrize("B,H,S,D", [(1, 2, 40, 64), (1, 2, 40, 128), (8, 32, 100, 64), (8, 32, 100, 128)])
+@pytest.mark.parametrize("factor,scale", [(1e19, 1.2e-38), (1e25, 0.0)])
+def test_products_that_only_the_scale_brings_into_range(B, H, S, D, factor, scale):
+    """q . k is beyond what fp32 holds, (scale * q) . k is not: the scale is applied to q, not to the sum."""
+    w = wl.attention_workload("t", 63, B, H, H, S, S, D, wl.MASK_CAUSAL, 1.0, "f32")
+    q, k, v = to_device(w.q) * factor, to_device(w.k) * factor, to_device(w.v)
+    out = binding.attn_fused_f32(q, k, v, wl.MASK_CAUSAL, None, scale)
+    binding.check_status()
+    eff = scale * factor * factor
+    pick = np.array([0, B - 1])
+    ref = oracle.attn(w.q.values[pick], w.k.values[pick], w.v.values[pick], wl.MASK_CAUSAL, None, eff)
+    assert_close_f32(out[[0, B - 1]], ref)
