@@ -164,6 +164,7 @@ struct AttnParams {
     long long o_sb, o_sh, o_ss;  // element strides of out between batch entries, heads and rows
     const int32_t* lens;
     const float* bias;  // additive bias on the scaled scores [B, bias_heads, Sq, Skv], or nullptr
+    const float* bias_end;  // one past its last element
     int bias_heads;     // 1 (shared by all heads) or Hq
     float inv_scale;    // 1 / scale: the bias is added to the unscaled scores as bias / scale
     int B, Hq, Hkv, Sq, Skv;
@@ -636,21 +637,27 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 const uint32_t col_h = col_s + hh * kHalf;
                 const int key0 = g * kHalf;
                 // The bias of this row and half-step is on its way while the scores are waited for (4 x 16 heads x 700 x 900, a
-                // bias per head: 68.9 -> 48.4 us).
-                [[maybe_unused]] float bias[BIAS ? kHalf : 1];
+                // bias per head: 68.9 -> 48.4 us).  Always in pieces of 16 bytes: where rows start between two of them, from the
+                // piece that holds the row's first element on, and the elements are moved up below.  (One by one, each 32-byte sector
+                // is asked for eight times, and the L1 left beside 224 KB of shared memory does not hold what eight warps ask for:
+                // 4 x 32/8 heads x 3283, D = 96, 2243 -> 889 us; 2317 x 2321, 28/4 heads, D = 64, 163 -> 111.)
+                [[maybe_unused]] float bias[BIAS ? kHalf + 4 : 1];
+                [[maybe_unused]] int lead = 0;  // elements of the first piece that lie before the row's first
                 if constexpr (BIAS) {
                     const int hb = p.bias_heads == 1 ? 0 : head;
                     const float* brow = p.bias + (((size_t)b * p.bias_heads + hb) * p.Sq + min(qi, p.Sq - 1)) * (size_t)p.Skv + key0;
-                    const int nvalid = min(kHalf, p.Skv - key0);  // columns beyond Skv are masked below
-                    if ((p.Skv & 3) == 0) {  // rows start on 16-byte boundaries
+                    lead = (int)(reinterpret_cast<uintptr_t>(brow) >> 2) & 3;
+                    const int nvalid = lead + min(kHalf, p.Skv - key0);  // columns beyond Skv are masked below
+                    if (__all_sync(0xffffffffu, brow - lead + ((nvalid + 3) & ~3) <= p.bias_end)) {
+                        const float4* pieces = reinterpret_cast<const float4*>(brow - lead);
 #pragma unroll
-                        for (int c = 0; c < kHalf / 4; ++c) {
-                            const float4 bv = c * 4 < nvalid ? __ldg(reinterpret_cast<const float4*>(brow) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int c = 0; c <= kHalf / 4; ++c) {
+                            const float4 bv = c * 4 < nvalid ? __ldg(pieces + c) : make_float4(0.f, 0.f, 0.f, 0.f);
                             bias[4 * c] = bv.x; bias[4 * c + 1] = bv.y; bias[4 * c + 2] = bv.z; bias[4 * c + 3] = bv.w;
                         }
-                    } else {
+                    } else {  // the last piece of some row would reach beyond the tensor's end
 #pragma unroll
-                        for (int k = 0; k < kHalf; ++k) bias[k] = k < nvalid ? __ldg(brow + k) : 0.f;
+                        for (int k = 0; k < kHalf + 4; ++k) bias[k] = k >= lead && k < nvalid ? __ldg(brow - lead + k) : 0.f;
                     }
                 }
                 // S(g) is complete, and so is every MMA this tile's issuer issued before it: O_t holds the
@@ -671,6 +678,12 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                                        BIAS;  // a bias may hold -inf: the path that tolerates it
                 if constexpr (BIAS) {
                     // Eq. 8's mask node as a tensor: scale * s + bias = scale * (s + bias / scale)
+                    if ((p.Skv & 3) != 0) {
+#pragma unroll
+                        for (int k = 0; k < kHalf + 2; ++k) bias[k] = lead & 1 ? bias[k + 1] : bias[k];
+#pragma unroll
+                        for (int k = 0; k < kHalf; ++k) bias[k] = lead & 2 ? bias[k + 2] : bias[k];
+                    }
 #pragma unroll
                     for (int k = 0; k < kHalf; ++k) s[k] = fmaf(bias[k], p.inv_scale, s[k]);
                 }
@@ -879,6 +892,7 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
     p.o_sb = so.b; p.o_sh = so.h; p.o_ss = so.s;
     p.lens = lens;
     p.bias = bias;
+    p.bias_end = bias ? bias + (size_t)B * bias_heads * Sq * Skv : nullptr;
     p.bias_heads = bias_heads;
     p.inv_scale = scale > 0.f ? 1.f / scale : 0.f;
     p.head_dim = head_dim;

@@ -33,7 +33,7 @@ def _run(w, bias):
 SHAPES = [  # B, Hq, Hkv, Sq, Skv, D, bias heads
     (1, 2, 2, 128, 128, 64, 1),
     (2, 4, 2, 300, 300, 64, 4),     # several tiles, ragged tail, GQA, per-head bias
-    (1, 8, 2, 200, 333, 128, 1),    # Skv not a multiple of 4: scalar bias loads; Sq != Skv
+    (1, 8, 2, 200, 333, 128, 1),    # Skv not a multiple of 4: bias rows off 16-byte boundaries; Sq != Skv
     (2, 3, 3, 130, 260, 128, 3),    # odd group size at D = 128: consecutive tiles of one head
     (1, 3, 3, 70, 200, 64, 3),      # odd group size at D = 64: two K/V streams
 ]
@@ -97,3 +97,12 @@ def test_argument_checks():
     assert e.value.status == binding.ERR_UNSUPPORTED
     with pytest.raises(ValueError):
         binding.attn_fused_bias(q, q, q, torch.zeros((1, 2, 128, 64), device="cuda"), 0, None, 0.125)
+
+
+@pytest.mark.parametrize("Skv", [1, 3, 62, 65, 66, 67, 129, 190])
+@pytest.mark.parametrize("D,heads", [(64, 3), (96, 1), (128, 3)])
+def test_rows_that_start_off_16_byte_boundaries(Skv, D, heads):
+    """Rows of every offset, the last of which ends with the tensor (its last piece of 16 bytes would reach beyond it).  A
+    quarter of the entries is -inf, so a neighbouring row's element in the place of an own one shows."""
+    w = wl.attention_workload("t", 47, 2, 3, 1, 135, Skv, D, wl.MASK_NONE, 1.0 / np.sqrt(D), "bf16")
+    _run(w, _bias(4701 + Skv, (2, heads, 135, Skv), hole_fraction=0.25))
