@@ -14,7 +14,7 @@
 //               warp of its scheduler: 1.2 % of the kernel)
 //   warp 9    : tcgen05.mma issuer of tile 0 (one elected lane), owns the TMEM allocation
 //   warp 10   : tcgen05.mma issuer of tile 1
-//   warp 11   : issues the TMA stores of both tiles' outputs; the third warpgroup hands registers to the other two
+//   warp 11   : issues the TMA stores of both tiles' outputs (but the last ones); the third warpgroup hands registers to the other two
 //   (setmaxnreg: 208 per softmax thread, 88 for the rest; 256*208 + 128*88 = 384*168 as launched).
 // Tensor memory (512 columns): S_t at t*128 (half h at +64h, 64 fp32 columns each), O_0 at 256,
 // O_1 at 256 + D.  P (bf16, two per column) of half h is written over the first 32 columns of that
@@ -29,6 +29,8 @@
 // the last products of this one; the output is staged in the Q buffer of its own item (whose last reader was that item's
 // last S) and stored from there by warp 11, which then hands the buffer back.  A boundary costs the softmax warps
 // about 3100 cycles instead of 4700 (8 x 12 x 1024 x 64 causal 34.1 -> 32.3 us, 18 x 32/8 x 895 x 96 padded 153 -> 149).
+// The CTA's last output is stored by the softmax warps, each its own rows, without the way through warp 11: with one item
+// per CTA that is 0.4 us (6 x 12 heads x 385 causal, D = 128, 12.56 -> 12.15; 8 x 12 x 1024 x 64 32.26 -> 31.8).
 // Reading the output only after the next item's first half-step gained nothing more and cost short items their overlap
 // (64 x 16/4 x 64: 16.7 -> 21.3 us).  At D = 128 long runs are at the power limit: fewer cycles, lower clock.
 #include <cuda_bf16.h>
@@ -195,7 +197,7 @@ template <int D, bool F16, bool BIAS>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                  const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_o,
-                 const AttnParams p) {
+                 const __grid_constant__ CUtensorMap tmap_o32, const AttnParams p) {
     using L = AttnSmem<D>;
     constexpr int kKVStages = L::kKVStages;
     extern __shared__ uint8_t smem_raw[];
@@ -285,10 +287,19 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     };
     // The n-th item after the first, worked out by the producer and read by everyone else from next_items[n % 2]: 1 if there
     // is one, 0: no more work, -1: gave up.
-    auto next_item = [&](int n) -> int {
+    auto next_item = [&](int n, bool relaxed = false) -> int {
         if (!dynamic) return 0;
-        if (!mbar_wait(&next_full[n & 1], (n >> 1) & 1)) return -1;
+        if (!(relaxed ? mbar_wait_relaxed(&next_full[n & 1], (n >> 1) & 1) : mbar_wait(&next_full[n & 1], (n >> 1) & 1))) return -1;
         return next_items[(n & 1) * 16];
+    };
+    // Sends the rows from row r of query tile q0 on (a whole tile or a quarter of one) off, out of Q buffer `at`, where the output is
+    // staged; the map's box has that many rows.  Rows beyond Sq are clipped by the TMA unit.
+    auto store_rows = [&](const CUtensorMap* map, int at, int r, int q0, int head, int b) {
+        if (q0 + r >= p.Sq) return;
+#pragma unroll
+        for (int c = 0; c < D / 64; ++c)
+            tma_store_4d(map, sQ + at * L::kTileBytes + c * L::kChunkBytes + r * 128, c * 64, q0 + r, head, b);
+        tma_store_commit();
     };
 
     if (threadIdx.x == 0) {
@@ -303,7 +314,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         for (int i = 0; i < 4; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_ready[i], 4); mbar_init(&pv_done[i], 1); }
         for (int t = 0; t < 2; ++t) { mbar_init(&o_free[t], 4); mbar_init(&next_full[t], 1); mbar_init(&next_empty[t], 11); }
         fence_mbar_init();
-        prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_o);
+        prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_o); prefetch_tmap(&tmap_o32);
     }
     if (warp == 9) {
         tmem_alloc(tmem_base_slot, kTmemCols);
@@ -534,31 +545,27 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 const ItemInfo it = decode(blockIdx.x);
                 nh[0] = it.nh[0]; nh[1] = it.nh[1]; q0[0] = it.q0[0]; q0[1] = it.q0[1]; h[0] = it.h[0]; h[1] = it.h[1]; b = it.b;
             }
-            int state = 1;
-            for (int r = 0; state == 1; ++r) {
-#pragma unroll
-                for (int t = 0; t < kTilesPerCta; ++t) {
-                    if (nh[t] == 0 || state != 1) continue;
-                    // (one barrier per buffer: the output of the last item may be ready before the one before it has been looked at)
-                    const int at = t * 2 + (uses[t] & 1);
-                    if (!mbar_wait_relaxed(&o_staged[at], (uses[t] >> 1) & 1)) { state = -1; continue; }
-                    ++uses[t];
-#pragma unroll
-                    for (int c = 0; c < D / 64; ++c)  // rows beyond Sq are clipped by the TMA unit
-                        tma_store_4d(&tmap_o, sQ + at * L::kTileBytes + c * L::kChunkBytes, c * 64, q0[t], h[t], b);
-                    tma_store_commit();
-                    tma_store_wait_read<0>();
-                    mbar_arrive(&q_empty[at]);  // the producer may load Q there again
-                }
-                if (state != 1) break;
-                state = next_item(r);
+            for (int r = 0;; ++r) {
+                int state = next_item(r, /*relaxed=*/true);
                 if (state == 1) {
-                    volatile const int* x = next_items + (r & 1) * 16;
-                    b = x[1]; q0[0] = x[4]; q0[1] = x[5]; h[0] = x[6]; h[1] = x[7]; nh[0] = x[8]; nh[1] = x[9];
-                    mbar_arrive(&next_empty[r & 1]);
+#pragma unroll
+                    for (int t = 0; t < kTilesPerCta; ++t) {
+                        if (nh[t] == 0 || state != 1) continue;
+                        // (one barrier per buffer: the output of an item may be ready before the one before it has been looked at)
+                        const int at = t * 2 + (uses[t] & 1);
+                        if (!mbar_wait_relaxed(&o_staged[at], (uses[t] >> 1) & 1)) { state = -1; continue; }
+                        ++uses[t];
+                        store_rows(&tmap_o, at, 0, q0[t], h[t], b);
+                        tma_store_wait_read<0>();
+                        mbar_arrive(&q_empty[at]);  // the producer may load Q there again
+                    }
                 }
+                if (state == -1) failed = true;
+                if (state != 1) break;  // (the output of the last item is stored by the softmax warps)
+                volatile const int* x = next_items + (r & 1) * 16;
+                b = x[1]; q0[0] = x[4]; q0[1] = x[5]; h[0] = x[6]; h[1] = x[7]; nh[0] = x[8]; nh[1] = x[9];
+                mbar_arrive(&next_empty[r & 1]);
             }
-            if (state == -1) failed = true;
             tma_store_wait_all<0>();  // every output tile has left shared memory and is written
         }
       }
@@ -599,8 +606,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 if (!warp_wait(&pv_done[t * 2 + ((steps - 1) & 1)], ((steps - 1) >> 1) & 1)) { failed = true; break; }
                 tc_fence_after_sync();
                 // O / l as bf16 through 128-byte-swizzled staging rows (32 rows x 64 columns per block of D) in the item's own Q
-                // buffer, whose last reader was the item's last S, and one TMA store per block; rows beyond Sq are clipped
-                // by the TMA unit.  A short rolled loop: its footprint matters more than its issue count.
+                // buffer, whose last reader was the item's last S.  A short rolled loop: its footprint matters more than its issue count.
                 uint8_t* stage_out = sQ + (t * 2 + ((q_uses - 1) & 1)) * L::kTileBytes + quarter * 4096;
                 uint32_t cur[32];
                 tmem_ld_x32(lane_base + col_o, cur);
@@ -624,9 +630,15 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) { mbar_arrive(&o_free[t]); mbar_arrive(&o_staged[t * 2 + ((q_uses - 1) & 1)]); }
-                pending = false;
             }
-            if (state != 1) break;
+            if (state != 1) {  // the CTA's last item (q0, head and b are still its own): no waiting for the other three warps
+                if (pending && lane == 0) {
+                    store_rows(&tmap_o32, t * 2 + ((q_uses - 1) & 1), quarter * 32, q0, head, b);
+                    tma_store_wait_all<0>();  // shared memory is not given up before it has been read
+                }
+                break;
+            }
+            pending = false;
             // One half-step.  At D = 64 the first one of an item has code of its own, without the votes and branches that its
             // state decides (34.0 -> 32.3 us at 8 x 12 x 1024); at D = 128 and with a bias the second copy of the code
             // costs as much as it saves.
@@ -882,11 +894,12 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
         const uint64_t strides[3] = {(uint64_t)st.s * 2, (uint64_t)st.h * 2, (uint64_t)st.b * 2};
         return encode_tmap_bf16_sw128(m, base, 4, dims, strides, box);
     };
-    CUtensorMap tq, tk, tv, to;
+    CUtensorMap tq, tk, tv, to, to32;
     if (!encode(&tq, q, Hq, Sq, sq, 128)) return FORGE_ERR_CUDA;
     if (!encode(&tk, k, Hkv, Skv, sk, kHalf)) return FORGE_ERR_CUDA;
     if (!encode(&tv, v, Hkv, Skv, sv, kHalf)) return FORGE_ERR_CUDA;
     if (!encode(&to, out, Hq, Sq, so, 128)) return FORGE_ERR_CUDA;
+    if (!encode(&to32, out, Hq, Sq, so, 32)) return FORGE_ERR_CUDA;  // a softmax warp's rows
     AttnParams p;
     p.out = static_cast<uint16_t*>(out);
     p.o_sb = so.b; p.o_sh = so.h; p.o_ss = so.s;
@@ -920,7 +933,7 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
     const long long items = head_pairs ? (long long)((Hq + 1) / 2) * B * q_tiles
                                        : (long long)Hq * B * ((q_tiles + 1) / 2);
     p.sms = sms;
-    FORGE_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)items), dim3(kThreads), L::kAlloc, s, tq, tk, tv, to, p));
+    FORGE_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)items), dim3(kThreads), L::kAlloc, s, tq, tk, tv, to, to32, p));
     return finish_launch(1);
 }
 
