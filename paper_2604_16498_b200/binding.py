@@ -106,12 +106,24 @@ def load() -> ctypes.CDLL:
     return _lib
 
 
+def _find_raw_stream():
+    """torch.cuda.current_stream() builds a Stream object around the stream's number, which takes 3.2 us, a third of the host
+    time of a small call; these two lookups take a tenth of that.  They are not part of torch's public interface: a torch
+    without them gets the public way."""
+    get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if get is None or dev is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: get(dev())
+
+
+_raw_stream = _find_raw_stream()
+
+
 def _stream() -> int:
-    """The calling thread's current stream on its current device, as a number.  torch.cuda.current_stream() builds a Stream
-    object around it, which takes 3.2 us, a third of the host time of a small call; these lookups take a tenth of that."""
+    """The calling thread's current stream on its current device, as a number."""
     if not torch.cuda.is_initialized():
         torch.cuda.init()
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream()
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> int:
