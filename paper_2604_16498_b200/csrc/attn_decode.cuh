@@ -68,8 +68,12 @@ constexpr int kPiecesPerLane = 1;          // no merge walks through more than 3
 //             which merge theirs in shared memory first; one level over at most 21 CTAs is left.  Against two levels:
 //             2 x 32/8 heads x 20000 33.6 -> 30.9 us, 3 x 32/8 x 6000, D = 64 17.1 -> 14.7, 1 x 32/8 x 32768 33.7 -> 32.8.
 //             (With 256 pieces of 7 heads each one warp merging 38 partials takes 34.0 us, two levels 31.1.)
-//   kTwoLevel the rest.
+//   kTwoLevel the rest, and 7 or 8 heads of 128 per kv head with up to 32 pieces too: there the streaming loop that the compiler
+//             makes without the second level is the slower one (8 x 28/4 heads x 2396..9584: 29.2 us, 28.4 with it;
+//             15 x 28/4 x 3572 23.9 and 23.2; level at 6 heads and fewer).
 enum { kShort = 0, kGrouped = 1, kTwoLevel = 2 };
+template <int D, int G>
+constexpr int kUpTo32Pieces = D == 128 && G >= 7 ? kTwoLevel : kShort;
 constexpr int kMaxGroupedPieces = 20 * kWarps;
 
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
@@ -733,38 +737,47 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
             }
             continue;
         }
-        // ---- several pieces: partial to the workspace, then the arrival count (grouped: to this warp's ring, whose rows have
-        // all been consumed, and the CTA's warps meet below)
+        // ---- several pieces: the partial, head h of the group to o_of(h) and ml_of(h)
+        auto write_partial = [&](auto o_of, auto ml_of) {
+            if (g < G && c == 0) {
+                ml_of(g)[0] = m_run;
+                ml_of(g)[1] = l_run;
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (2 * c + e >= G) continue;
+                float* o = o_of(2 * c + e);
+#pragma unroll
+                for (int hb = 0; hb < NHB; ++hb) {
+                    const int d0 = hb * 64 + g * 8;
+                    *reinterpret_cast<float4*>(o + d0) = make_float4(acc[hb][0][e], acc[hb][1][e], acc[hb][2][e], acc[hb][3][e]);
+                    *reinterpret_cast<float4*>(o + d0 + 4) =
+                        make_float4(acc[hb][0][2 + e], acc[hb][1][2 + e], acc[hb][2][2 + e], acc[hb][3][2 + e]);
+                }
+            }
+        };
         const size_t slot0 = (size_t)head0 * num_splits + it.piece;  // head 0 of the group
-        float* part_o = ws_o + slot0 * D;
-        float* part_ml = ws_ml + slot0 * 2;
-        size_t per_head = num_splits;
-        if (MODE == kGrouped && sched.grouped) {
-            part_o = reinterpret_cast<float*>(ring_raw + (ring - static_cast<uint32_t>(__cvta_generic_to_shared(ring_raw))));
-            part_ml = part_o + G * D;
-            per_head = 1;
-            if (lane == 0) {
-                merge_info[warp][1] = it.piece; merge_info[warp][2] = it.pieces; merge_info[warp][3] = head0;
-                merge_info[warp][0] = it.b * Hkv + it.kvh;
+        if constexpr (MODE == kGrouped) {
+            // to this warp's ring, whose rows have all been consumed (the CTA's warps meet below), or to the workspace
+            float* part_o = ws_o + slot0 * D;
+            float* part_ml = ws_ml + slot0 * 2;
+            size_t per_head = num_splits;
+            if (sched.grouped) {
+                part_o = reinterpret_cast<float*>(ring_raw + (ring - static_cast<uint32_t>(__cvta_generic_to_shared(ring_raw))));
+                part_ml = part_o + G * D;
+                per_head = 1;
+                if (lane == 0) {
+                    merge_info[warp][1] = it.piece; merge_info[warp][2] = it.pieces; merge_info[warp][3] = head0;
+                    merge_info[warp][0] = it.b * Hkv + it.kvh;
+                }
             }
+            write_partial([&](int h) { return part_o + h * per_head * D; }, [&](int h) { return part_ml + h * per_head * 2; });
+            if (sched.grouped) continue;
+        } else {
+            write_partial([&](int h) { return ws_o + (slot0 + (size_t)h * num_splits) * D; },
+                          [&](int h) { return ws_ml + (slot0 + (size_t)h * num_splits) * 2; });
         }
-        if (g < G && c == 0) {
-            part_ml[g * per_head * 2] = m_run;
-            part_ml[g * per_head * 2 + 1] = l_run;
-        }
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            if (2 * c + e >= G) continue;
-            float* o = part_o + (2 * c + e) * per_head * D;
-#pragma unroll
-            for (int hb = 0; hb < NHB; ++hb) {
-                const int d0 = hb * 64 + g * 8;
-                *reinterpret_cast<float4*>(o + d0) = make_float4(acc[hb][0][e], acc[hb][1][e], acc[hb][2][e], acc[hb][3][e]);
-                *reinterpret_cast<float4*>(o + d0 + 4) =
-                    make_float4(acc[hb][0][2 + e], acc[hb][1][2 + e], acc[hb][2][2 + e], acc[hb][3][2 + e]);
-            }
-        }
-        if (MODE == kGrouped && sched.grouped) continue;
+        // to the workspace: then the arrival count
         if (MODE == kTwoLevel && it.pieces > kSingleLevelPieces) {
             arrive_two_level<D, G, F16>(counters, ws_o, ws_ml, out, B, Hkv, it.b, it.kvh, it.piece, it.pieces, head0,
                                         num_splits, head_dim, lane);
@@ -836,13 +849,13 @@ int dispatch_g(int G, const void* q, const void* kc, const void* vc, const int32
                int num_splits, float scale_log2, cudaStream_t s) {
     // no more pieces than this can exist, whatever lens holds
     const long long blocks_max = (Smax + kBlockKeys - 1) / kBlockKeys, most = blocks_max < num_splits ? blocks_max : num_splits;
-    const int mode = most <= kSingleLevelPieces ? kShort
-                     : most <= kMaxGroupedPieces && most * B * Hkv <= (long long)sm_count() * kWarps ? kGrouped : kTwoLevel;
+    const bool few = most <= kSingleLevelPieces;
+    const bool grouped = most <= kMaxGroupedPieces && most * B * Hkv <= (long long)sm_count() * kWarps;
 #define FORGE_DECODE_CASE(g)                                                                                     \
     case g:                                                                                                      \
-        return mode == kShort   ? launch_split<D, g, F16, kShort>(FORGE_DECODE_ARGS)                             \
-               : mode == kGrouped ? launch_split<D, g, F16, kGrouped>(FORGE_DECODE_ARGS)                         \
-                                  : launch_split<D, g, F16, kTwoLevel>(FORGE_DECODE_ARGS)
+        return few       ? launch_split<D, g, F16, kUpTo32Pieces<D, g>>(FORGE_DECODE_ARGS)                       \
+               : grouped ? launch_split<D, g, F16, kGrouped>(FORGE_DECODE_ARGS)                                  \
+                         : launch_split<D, g, F16, kTwoLevel>(FORGE_DECODE_ARGS)
 #define FORGE_DECODE_ARGS \
     q, kc, vc, lens, out, counters, ws_o, ws_ml, B, Hq, Hkv, Smax, head_dim, num_splits, scale_log2, s
     switch (G) {
