@@ -20,6 +20,10 @@
 // the next (persistent CTAs).  Outputs with few tiles split K over clusters as linear_split.cu does: CTA r of S sums
 // its share of the k-blocks, owns a share of the tokens, and is sent the others' partial sums through shared memory.
 //
+// A cluster's CTAs wait for one another, so two clusters must not each hold tensor memory that the other one's CTAs wait for.
+// Beside one of these CTAs (832 threads of 72 registers, all 512 columns) an SM has 5600 registers left, and the CTAs of the other
+// kernels that run in clusters (linear_pair.cu, linear_split.cu) take 23000 and more.
+//
 // Warps: 0 TMA producer, 1 MMA issuer and TMEM owner, then six quads of four warps (128 TMEM lanes): epilogue quads, which
 // take groups of tokens in turn, and three or four converter quads ("groups"), which take k-blocks in turn, each with its
 // own A operand.
@@ -60,7 +64,7 @@ struct W8Params {
     int nt, tiles_t;     // tokens per tile, token tiles
     int split_log2;      // CTAs per tile
     int own4;            // 4-token pieces a CTA of a cluster finishes
-    int stages;          // at least kMaxGroups
+    int stages;          // at least as many as converter groups
     int recv_off, out_off, bar_off;  // byte offsets in shared memory
     int* status;
 };
@@ -349,10 +353,45 @@ int launch_w8(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w, const W8Para
 
 }  // namespace
 
+bool linear_w8_plan(int M, int N, int K, int sms, W8Plan* plan) {
+    W8Plan& pl = *plan;
+    const int kblocks = (K + kBK - 1) / kBK;
+    const long long tiles_f = (N + kBF - 1) / kBF;
+    pl.tiles_t = (M + kMaxTokens - 1) / kMaxTokens;
+    pl.nt = ((M + pl.tiles_t - 1) / pl.tiles_t + 15) / 16 * 16;
+    if (pl.tiles_t * tiles_f > sms) {  // several rounds: the smallest tiles that need no more of them
+        const long long rounds = (pl.tiles_t * tiles_f + sms - 1) / sms, most = rounds * sms / tiles_f;
+        pl.nt = (int)((M + most - 1) / most + 15) / 16 * 16;
+        pl.tiles_t = (M + pl.nt - 1) / pl.nt;
+    }
+    pl.tiles = pl.tiles_t * tiles_f;
+    // Long k-loops in several rounds keep the converters busy: four groups (8192 x 8192 x 4096 454 us, 507 with three).
+    // Everything else gains more from a third quad of epilogue warps (8192 x 768 x 768 16.7 against 24.6 us, with erf and
+    // residual 30 against 42; 400 x 3072 x 768 9.0 against 9.6), and a single token does not notice (16.0 both).
+    pl.groups = pl.tiles > sms && kblocks >= 48 ? 4 : 3;
+    // as many CTAs per tile as run at once (clusters of eight do not tile every GPC) with two k-blocks or more each
+    // (1 x 768 x 768: 4.0 us, with three or more 4.6 us)
+    pl.split = 1;
+    while (pl.split < 8 && pl.tiles * pl.split * 2 <= sms * 8 / 9 && kblocks >= pl.split * 2 * 2) pl.split *= 2;
+    const int stage_bytes = kBF * kBK + pl.nt * kBK * 2;  // at most 32 KB
+    for (;; pl.split /= 2) {
+        pl.own4 = pl.split > 1 ? (pl.nt / 4 + pl.split - 1) / pl.split : 0;
+        pl.recv_bytes = (pl.split - 1) * pl.own4 * kBF * 16;  // at most 84 KB (192 tokens, S = 8)
+        pl.stages = (kSmemMax - pl.recv_bytes - kOutBytes - kBarBytes - 1024) / stage_bytes;
+        if (pl.stages > kMaxStages) pl.stages = kMaxStages;
+        // The converters need a stage per group (their barrier parities, linear_w8_kernel).  192 tokens and S = 8 leave three
+        // stages for three groups; with S = 1 there are six and more.
+        if (pl.stages >= pl.groups || pl.split == 1) break;
+    }
+    return pl.tiles <= 2147483647LL && pl.stages >= pl.groups;
+}
+
 int linear_w8(const void* x, const void* w_int8, const float* scale, const void* b, const void* residual, void* y, int M,
               int N, int K, int act, cudaStream_t s) {
     const int sms = sm_count();
     if (sms <= 0) return FORGE_ERR_CUDA;
+    W8Plan pl;
+    if (!linear_w8_plan(M, N, K, sms, &pl)) return FORGE_ERR_UNSUPPORTED;
     W8Params p;
     p.bias = static_cast<const uint16_t*>(b);
     p.residual = static_cast<const uint16_t*>(residual);
@@ -360,30 +399,13 @@ int linear_w8(const void* x, const void* w_int8, const float* scale, const void*
     p.y = static_cast<uint16_t*>(y);
     p.M = M; p.N = N; p.K = K;
     p.act = act;
-    p.tiles_t = (M + kMaxTokens - 1) / kMaxTokens;
-    p.nt = ((M + p.tiles_t - 1) / p.tiles_t + 15) / 16 * 16;
-    const int kblocks = (K + kBK - 1) / kBK;
-    const long long tiles_f = (N + kBF - 1) / kBF;
-    if (p.tiles_t * tiles_f > sms) {  // several rounds: the smallest tiles that need no more of them
-        const long long rounds = (p.tiles_t * tiles_f + sms - 1) / sms, most = rounds * sms / tiles_f;
-        p.nt = (int)((M + most - 1) / most + 15) / 16 * 16;
-        p.tiles_t = (M + p.nt - 1) / p.nt;
-    }
-    const long long tiles = p.tiles_t * tiles_f;
-    if (tiles > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
-    // as many CTAs per tile as run at once (clusters of eight do not tile every GPC) with two k-blocks or more each
-    // (1 x 768 x 768: 4.0 us, with three or more 4.6 us)
-    int S = 1;
-    while (S < 8 && tiles * S * 2 <= sms * 8 / 9 && kblocks >= S * 2 * 2) S *= 2;
-    p.split_log2 = __builtin_ctz(S);
-    p.own4 = S > 1 ? (p.nt / 4 + S - 1) / S : 0;
-    const int stage_bytes = kBF * kBK + p.nt * kBK * 2;  // at most 32 KB
-    const int recv_bytes = (S - 1) * p.own4 * kBF * 16;  // at most 84 KB (192 tokens, S = 8): four stages remain
-    int stages = (kSmemMax - recv_bytes - kOutBytes - kBarBytes - 1024) / stage_bytes;
-    if (stages > kMaxStages) stages = kMaxStages;
-    p.stages = stages;
-    p.recv_off = stages * stage_bytes;
-    p.out_off = p.recv_off + recv_bytes;
+    p.nt = pl.nt;
+    p.tiles_t = pl.tiles_t;
+    p.split_log2 = __builtin_ctz(pl.split);
+    p.own4 = pl.own4;
+    p.stages = pl.stages;
+    p.recv_off = pl.stages * (kBF * kBK + pl.nt * kBK * 2);
+    p.out_off = p.recv_off + pl.recv_bytes;
     p.bar_off = p.out_off + kOutBytes;
     const int total = p.bar_off + kBarBytes + 1024;
     p.status = device_status_word();
@@ -401,12 +423,9 @@ int linear_w8(const void* x, const void* w_int8, const float* scale, const void*
         const uint32_t box[2] = {kBK, kBF};
         if (!encode_tmap_u8_sw64(&tmap_w, w_int8, 2, dims, strides, box)) return FORGE_ERR_CUDA;
     }
-    const long long grid = S > 1 ? tiles * S : (tiles < sms ? tiles : sms);
-    // Long k-loops in several rounds keep the converters busy: four groups (8192 x 8192 x 4096 454 us, 507 with three).
-    // Everything else gains more from a third quad of epilogue warps (8192 x 768 x 768 16.7 against 24.6 us, with erf and
-    // residual 30 against 42; 400 x 3072 x 768 9.0 against 9.6), and a single token does not notice (16.0 both).
-    return tiles > sms && kblocks >= 48 ? launch_w8<4>(tmap_x, tmap_w, p, (unsigned)grid, total, S, s)
-                                        : launch_w8<3>(tmap_x, tmap_w, p, (unsigned)grid, total, S, s);
+    const long long grid = pl.split > 1 ? pl.tiles * pl.split : (pl.tiles < sms ? pl.tiles : sms);
+    return pl.groups == 4 ? launch_w8<4>(tmap_x, tmap_w, p, (unsigned)grid, total, pl.split, s)
+                          : launch_w8<3>(tmap_x, tmap_w, p, (unsigned)grid, total, pl.split, s);
 }
 
 }  // namespace forge
