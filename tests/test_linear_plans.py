@@ -2,6 +2,8 @@
 import random
 
 import plans
+from test_parity_linear_split import SHAPES as SPLIT_SHAPES
+from test_parity_linear_w8_edges import SHAPES as W8_SHAPES
 
 
 def test_int8_linear_has_a_ring_stage_for_every_converter_group_and_fits_shared_memory():
@@ -27,3 +29,11 @@ def test_int8_linear_has_a_ring_stage_for_every_converter_group_and_fits_shared_
 
 def test_a_plan_exists_only_below_2_31_tiles():
     assert plans.w8((1 << 31) - 200, 64 * 8 * 400, 16) is None
+
+
+def test_the_shapes_of_the_parity_tests_take_the_paths_they_are_there_for():
+    for shape, want in W8_SHAPES.items():
+        p = plans.w8(*shape)
+        assert (p.nt, p.tiles, p.split, p.groups, p.stages) == want, shape
+    for shape, want in SPLIT_SHAPES.items():
+        assert plans.split(*shape) == want, shape

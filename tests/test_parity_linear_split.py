@@ -15,16 +15,19 @@ from util import Guarded, assert_close_bf16, to_device, to_f64
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [
-    (1, 8, 8), (1, 72, 136),            # one and three k-blocks, one column tile
-    (7, 200, 520), (8, 264, 576),       # 9 k-blocks: S = 4, shares of 2 and 3
-    (16, 768, 3080), (33, 768, 4096),   # S = 8; 49 k-blocks, the last of 8 columns; a second row warp
-    (64, 4104, 1024), (65, 776, 776),   # two CTAs per SM / one
-    (127, 2304, 768), (128, 768, 3072), # whole row tile, S = 2 and 8
-    (40, 17000, 192),                   # 128-column tiles, several rounds
-    (129, 2048, 1544), (184, 1032, 4096), (300, 264, 2056),  # several row tiles, clusters across them
-    (700, 3072, 136),                   # two CTAs per SM, several row tiles
-]
+# (M, N, K): (columns of a tile, CTAs per tile, two CTAs per SM) on 148 SMs (test_linear_plans.py checks that)
+SHAPES = {
+    (1, 8, 8): (64, 1, True), (1, 72, 136): (64, 1, True),             # one and three k-blocks, one column tile
+    (7, 200, 520): (64, 4, True), (8, 264, 576): (64, 4, True),        # 9 k-blocks: shares of 2 and 3
+    (16, 768, 3080): (64, 8, True), (33, 768, 4096): (64, 8, True),    # 49 k-blocks, the last of 8 columns; a second row warp
+    (64, 4104, 1024): (64, 4, True), (65, 776, 776): (64, 4, False),   # two CTAs per SM / one
+    (127, 2304, 768): (64, 2, False), (128, 768, 3072): (64, 8, False),  # whole row tile
+    (40, 17000, 192): (128, 1, True),                                  # 128-column tiles: 133 CTAs
+    (40, 38400, 192): (128, 1, True), (100, 38400, 136): (128, 1, True),  # 300 CTAs: more than run at once
+    (129, 2048, 1544): (64, 2, False), (184, 1032, 4096): (128, 4, False), (300, 264, 2056): (64, 8, False),  # several row tiles
+    (700, 3072, 136): (128, 1, False),                                 # several row tiles, one CTA per tile and per SM
+    (600, 3776, 136): (64, 1, True),                                   # two CTAs per SM, several row tiles: 295 CTAs
+}
 
 
 def _case(M, N, K, dtype="bf16"):
@@ -35,7 +38,7 @@ def _case(M, N, K, dtype="bf16"):
     return x, w, b, r
 
 
-@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("shape", list(SHAPES))
 @pytest.mark.parametrize("w_layout", [binding.W_KN, binding.W_NK])
 def test_edges_of_tiles_and_shares(shape, w_layout):
     M, N, K = shape

@@ -35,7 +35,7 @@ def test_shapes_and_activations(shape, act):
     assert_close_bf16(y, ref)
 
 
-@pytest.mark.parametrize("M", [128, 384])  # one row tile (one-CTA kernel) and several (CTA pairs)
+@pytest.mark.parametrize("M", [128, 384])  # one token tile and two
 def test_extreme_weights_are_widened_exactly(M):
     """-128, 127 and 0 only, identity-like activations: the result is an exact small integer combination."""
     N, K = 64, 64
