@@ -17,9 +17,13 @@
 // rest of the ring holds weights, and the copy unit does not fill rows that nobody needs (M = 1 took 23 us where M = 64
 // took 14 us with a 128-row box).  The MMA always reads 128 rows of A; those beyond xrows are whatever follows in
 // shared memory (inside the allocation) and only reach accumulator rows that nobody reads.
-// In configurations where two CTAs share an SM, the weights' first tiles are asked into L2 before the wait for the
-// previous kernel, whose tail they overlap (a prefetch into L2 is coherent: it may run ahead of a kernel that writes the
-// same lines).  With one CTA per SM there is no overlap to gain and the extra requests cost 0.3-0.6 us.
+// Where this grid finds room beside the previous kernel's (two CTAs per SM, or CTAs on at most half the SMs), the weights' first
+// tiles are asked into L2 before the wait for that kernel, whose tail they overlap (a prefetch into L2 is coherent: it may
+// run ahead of a kernel that writes the same lines).  With a CTA of its own on every SM there is no overlap to gain and
+// the extra requests cost 0.3-0.6 us.
+// A cluster's CTAs wait for one another, so two clusters must not each hold tensor memory that the other one's CTAs wait for.
+// Two of these CTAs fit an SM and take at most 256 of its 512 columns; beside a CTA of linear_pair.cu or linear_w8.cu (55000
+// registers and more) there is no room for their 23000-31000.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -426,11 +430,13 @@ SplitPlan linear_split_plan_row(bool gated, int M, int N, int K, int sms) {
     return pl;
 }
 
-// Several row tiles: the split kernel against CTA pairs, by estimated microseconds.  The constants are fits to
-// measurements of both kernels (each within 10 % on 20 shapes of 130-4342 rows, 256-14336 columns, K 384-14336):
-// fixed cost of launch, first copy, epilogue and exchange, plus the time of a k-block.  A 128 x 128 tile is bound by
-// shared memory (64 KB written and read per k-block, 0.28 us for 0.13 us of tensor core), a pair's 256 x 256 tile is not
-// (0.285 us for four times the work), but a quarter as many tiles leave SMs idle.
+// Several row tiles: the split kernel against CTA pairs, by estimated microseconds: fixed cost of launch, first copy, epilogue
+// and exchange, plus the time of a k-block.  A 128 x 128 tile is bound by shared memory (64 KB written and read per k-block,
+// up to 0.28 us for 0.13 us of tensor core), a pair's 256 x 256 tile is not (0.285 us for four times the work), but a quarter as many
+// tiles leave SMs idle.  The estimates rank the plans, they do not predict times (up to a third too long for one CTA
+// per tile and long K, a quarter too short for many rounds of pairs): of 22 shapes of 130-4342 rows, 256-14336 columns and K
+// 136-14336, measured with every plan, the plan taken was the fastest or within 3 % of it (256 x 4096 x 14336 35.5 us, pairs 72.5;
+// 596 x 3072 x 768 8.9 and 9.7; 458 x 8192 x 2048 pairs; profiles/linear_plan_rows.md has them all).
 bool linear_split_plan_rows(int M, int N, int K, int sms, SplitPlan* plan) {
     const int kblocks = (K + kBK - 1) / kBK;
     const long long t2 = (long long)((M + 255) / 256) * ((N + 255) / 256), pairs = sms / 2;
@@ -449,10 +455,6 @@ bool linear_split_plan_rows(int M, int N, int K, int sms, SplitPlan* plan) {
             if (tiles * S > (S == 1 ? sms : sms * 8 / 9)) break;
             const double t = 4.9 + (bn == 64 ? 0.18 : 0.28) * ((kblocks + S - 1) / S) + (S == 1 ? 0.0 : bn == 64 ? 0.8 : 1.3);
             if (t < best) { best = t; split = true; *plan = {bn, S, false}; }
-        }
-        if (bn == 64 && tiles > sms && tiles <= 2LL * sms) {  // two CTAs per SM
-            const double t = 5.0 + 0.31 * kblocks;
-            if (t < best) { best = t; split = true; *plan = {64, 1, true}; }
         }
     }
     return split;

@@ -26,7 +26,6 @@ SHAPES = {
     (40, 38400, 192): (128, 1, True), (100, 38400, 136): (128, 1, True),  # 300 CTAs: more than run at once
     (129, 2048, 1544): (64, 2, False), (184, 1032, 4096): (128, 4, False), (300, 264, 2056): (64, 8, False),  # several row tiles
     (700, 3072, 136): (128, 1, False),                                 # several row tiles, one CTA per tile and per SM
-    (600, 3776, 136): (64, 1, True),                                   # two CTAs per SM, several row tiles: 295 CTAs
 }
 
 
