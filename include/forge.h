@@ -134,7 +134,7 @@ int forge_attn_fused_f32(const void* q, const void* k, const void* v, void* out,
  * Split rule.  Every sequence is cut into pieces of c 16-row blocks, counted from its
  * start (the last piece may be shorter), with one c for the whole call, chosen on the
  * device from lens: the smallest c with
- *     c >= ceil(blocks of all sequences and kv heads / workers)   (workers = 8 per SM)
+ *     c >= ceil(blocks of all sequences and kv heads / workers)   (workers = 7 per SM)
  *     c >= ceil(blocks of the longest sequence / num_splits),
  * raised by up to a factor of about two if that leaves no more pieces than workers.
  * So num_splits is the largest number of pieces any sequence is cut into, and in a

@@ -14,7 +14,7 @@
 // worker: it owns whole pieces, keeps a private ring of 16-row blocks in shared memory filled by
 // TMA tile copies (16 rows x 64 columns each, 128-byte swizzle, completion counted on an mbarrier
 // per stage) that run ahead across piece boundaries (7 warps x 16 KB in flight per SM), and writes
-// its partial straight from registers.  No warp ever waits for another one.
+// its partial straight from registers.  While it streams, no warp waits for another one.
 //
 // Pieces.  All pieces of a call are C blocks of 16 rows long (the last piece of a sequence may be
 // shorter).  Every warp works C out for itself from lens: the smallest C that is at least the even
@@ -28,7 +28,9 @@
 // each worker writes its partial to the workspace and, with release-acquire ordering, adds one to
 // the arrival counter of its (batch, kv head); the worker that brings the counter to the number of
 // pieces merges all partials of the G heads, writes the output rows and puts the counter back to
-// zero.  Nobody waits: whoever arrives last does the merge.  The counters live at the start of the
+// zero.  Nobody waits: whoever arrives last does the merge.  That is the merge of up to 32 pieces; of more, it has a level
+// before it, either in the shared memory of the CTA whose warps hold neighbouring pieces (the one place where warps of a CTA
+// meet) or over groups of sixteen pieces with counters of their own (kGrouped, kTwoLevel below).  The counters live at the start of the
 // workspace and must be zero when a call starts; every call leaves them at zero.
 // The G = Hq / Hkv query heads that share a KV head are processed together, so every cached row
 // is read exactly once.  The dot products run on warp-level tensor-core MMAs (m16n8k16) with
@@ -66,7 +68,8 @@ constexpr int kPiecesPerLane = 1;          // no merge walks through more than 3
 //   kShort    up to 32 pieces, by one warp.
 //   kGrouped  33 to 140 pieces and never more pieces than workers: consecutive pieces of a kv head go to the warps of a CTA,
 //             which merge theirs in shared memory first; one level over at most 21 CTAs is left.  Against two levels:
-//             2 x 32/8 heads x 20000 33.6 -> 30.9 us, 3 x 32/8 x 6000, D = 64 17.1 -> 14.7, 1 x 32/8 x 32768 33.7 -> 32.8.
+//             2 x 32/8 heads x 20000 35.8 -> 33.2 us, 3 x 32/8 x 6000, D = 64 18.2 -> 15.7, 3 x 28/4 x 659..2639 24.1 -> 16.0;
+//             1 x 32/8 x 32768 33.7 -> 32.9 at best, level on some GPUs.
 //             (With 256 pieces of 7 heads each one warp merging 38 partials takes 34.0 us, two levels 31.1.)
 //   kTwoLevel the rest, and 7 or 8 heads of 128 per kv head with up to 32 pieces too: there the streaming loop that the compiler
 //             makes without the second level is the slower one (8 x 28/4 heads x 2396..9584: 29.2 us, 28.4 with it;

@@ -33,9 +33,10 @@ int sm_count();
 // Launches `kernel` with programmatic stream serialisation: its CTAs may become resident while the
 // previous kernel in the stream is still running (once that kernel has let its dependents go, or has
 // finished), so launch latency and the kernel's own set-up overlap the predecessor's tail.  Every kernel
-// of this library calls pdl_wait() before its first access to global memory, which blocks until the
+// of this library calls pdl_wait() before its first read or write of global memory, which blocks until the
 // predecessor has completed and its writes are visible; a predecessor that never lets go behaves as
-// with an ordinary launch.
+// with an ordinary launch.  Only requests that bring lines into L2 and nowhere else (linear_split.cu's first weights) may
+// go out before it: L2 is coherent, so they see nothing that a later read would not.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem_bytes, cudaStream_t s,
                               Args&&... args) {

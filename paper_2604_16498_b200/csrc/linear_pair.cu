@@ -1,6 +1,6 @@
-// Fused Linear + bias + activation (+ residual) on CTA pairs (Listing 6 / Eq. 11, the same operator as
-// linear_gelu.cu).  Why a second kernel: the one-CTA kernel is bound by the rate at which an SM can pull
-// operands out of L2 (a 128 x 192 tile reads 40 KB per 64-deep k-step for 384 tensor-core cycles, more
+// Fused Linear + bias + activation (+ residual) on CTA pairs (Listing 6 / Eq. 11), for outputs with enough tiles to fill the
+// GPU (linear_split.cu has the others; linear_gelu.cu chooses).  Why pairs: a CTA alone is bound by the rate at which an SM
+// can pull operands out of L2 (a 128 x 192 tile reads 40 KB per 64-deep k-step for 384 tensor-core cycles, more
 // than the SM's L2 port delivers).  Here two CTAs on neighbouring SMs (a cluster of two) share one
 // 256 x 256 output tile: each loads its own 128 rows of X and its own 128 columns of W, with its own TMA
 // copies (no multicast), and the tensor cores of both SMs read both halves of W (tcgen05.mma
