@@ -73,7 +73,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                    const __grid_constant__ CUtensorMap tmap_w2,
                    const __grid_constant__ CUtensorMap tmap_y, const uint16_t* __restrict__ bias,
-                   const uint16_t* __restrict__ residual, int M, int N, int K, int* __restrict__ status) {
+                   const uint16_t* __restrict__ residual, int M, int N, int K, int band_rows, int* __restrict__ status) {
     using L = PairSmem;
     extern __shared__ uint8_t smem_raw[];
     // the same offset in both CTAs (the dynamic shared memory of a kernel starts at the same address in each)
@@ -98,11 +98,18 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const bool split = !GATED && rem > 0 && 2 * rem <= num_pairs;
     const int n_whole = split ? num_tiles - rem : num_tiles;
     const int num_units = n_whole + (split ? 2 * rem : 0);
-    struct Unit { int tile, col0, width; };  // col0: first column of the unit inside its tile
+    // Tiles go down the columns of bands of band_rows row tiles (band_rows_of() has the rule).
+    struct Unit { int m0, n0, width; };  // first row and column, columns
     auto unit_of = [&](int u) {
         Unit x;
-        if (u < n_whole) { x.tile = u; x.col0 = 0; x.width = BNO; }
-        else { const int v = u - n_whole; x.tile = n_whole + (v >> 1); x.col0 = (v & 1) * (kBN / 2); x.width = kBN / 2; }
+        int tile = u, col0 = 0;
+        x.width = BNO;
+        if (u >= n_whole) { const int v = u - n_whole; tile = n_whole + (v >> 1); col0 = (v & 1) * (kBN / 2); x.width = kBN / 2; }
+        const int row0 = tile / (band_rows * tiles_n) * band_rows, in_band = tile - row0 * tiles_n;
+        const int rows = min(band_rows, tiles_m - row0);
+        const int col = in_band / rows;
+        x.m0 = (row0 + in_band - col * rows) * 2 * kBM;
+        x.n0 = col * BNO + col0;
         return x;
     };
 
@@ -135,10 +142,9 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             uint32_t phase = 0;
             for (int u = pair; u < num_units && !failed; u += num_pairs) {
                 const Unit un = unit_of(u);
-                const int tile = un.tile;
-                const int m0 = (tile / tiles_n) * 2 * kBM + (int)rank * kBM;
+                const int m0 = un.m0 + (int)rank * kBM;
                 // this CTA's columns of W: half of the unit's (gated: 64 gate columns and the same 64 up columns)
-                const int n0 = (tile % tiles_n) * BNO + un.col0 + (int)rank * (un.width / 2);
+                const int n0 = un.n0 + (int)rank * (un.width / 2);
                 const bool narrow = un.width < BNO;  // a half tile: 64 columns of W per CTA
                 for (int kb = 0; kb < kblocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1)) { failed = true; break; }
@@ -212,8 +218,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         int it = 0;
         for (int u = pair; u < num_units; u += num_pairs, ++it) {
             const Unit un = unit_of(u);
-            const int tile = un.tile;
-            const int m0 = (tile / tiles_n) * 2 * kBM + (int)rank * kBM, n0 = (tile % tiles_n) * BNO + un.col0;
+            const int m0 = un.m0 + (int)rank * kBM, n0 = un.n0;
             const int acc = it & 1;
             const uint32_t acc_phase = (it >> 1) & 1;
             if (!warp_wait(&tmem_full[acc], acc_phase)) { failed = true; break; }
@@ -315,6 +320,18 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     }
 }
 
+// Row tiles per band of the tile order.  The pairs that run at once should share operands: row by row, the 74 pairs of a round
+// read one row tile of X and 74 column tiles of W, and with N = 14336 (gated: 112 column tiles, 235 MB of W) every row tile reads all of
+// W from HBM again, 7.5 GB a call at 8192 rows.  Down the columns of a band of 24 row tiles a round reads 24 + 3 tiles, and the band's
+// rows of X stay in L2 while W passes once: 8192 x 14336 x 4096 gated 1485 -> 1323 us (8 / 16 rows: 1496 / 1398), 4096 x 14336 x 4096
+// 380 -> 349, 1024 x 14336 x 4096 gated 209 -> 187.  A band's rows of X are at most about 48 MB.  Up to 16 column tiles a round of
+// whole rows is nearly square already (8192 x 3072 x 768 37.3, 39.0 with bands of 16; 5027 x 4096 x 4096 130 and 136).
+inline int band_rows_of(int tiles_n, int K) {
+    if (tiles_n <= 16) return 1;
+    const long long fit = (48LL << 20) / (2LL * kBM * 2 * K);
+    return fit < 8 ? 8 : fit > 24 ? 24 : (int)fit;
+}
+
 template <int ACT, bool W_NK, bool F16, bool GATED = false>
 int launch_pair(const void* x, const void* w, const void* b, const void* residual, void* y, int M, int N, int K,
                 cudaStream_t s, const void* w_up = nullptr) {
@@ -361,7 +378,8 @@ int launch_pair(const void* x, const void* w, const void* b, const void* residua
     const int pairs = tiles < sms / 2 ? tiles : sms / 2;
     // the cluster shape is part of the kernel (__cluster_dims__); programmatic stream serialisation as everywhere
     FORGE_CUDA_TRY(launch_pdl(kernel, dim3(2 * pairs), dim3(kThreads), L::kAlloc, s, tmap_x, tmap_w, tmap_w2, tmap_y,
-                              static_cast<const uint16_t*>(b), static_cast<const uint16_t*>(residual), M, N, K, status));
+                              static_cast<const uint16_t*>(b), static_cast<const uint16_t*>(residual), M, N, K,
+                              band_rows_of((N + BNO - 1) / BNO, K), status));
     return finish_launch(1);
 }
 
