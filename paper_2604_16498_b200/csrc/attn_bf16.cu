@@ -38,6 +38,7 @@
 
 #include <type_traits>
 
+#include "attn_tiles.cuh"
 #include "attn_wide.cuh"
 #include "forge_common.cuh"
 #include "sm100_ptx.cuh"
@@ -173,10 +174,13 @@ struct AttnParams {
     int head_dim;  // elements per row in memory (<= the kernel's D; the TMA unit zero-fills the difference)
     int mask_kind;
     float scale_log2;  // > 0 (a zero scale is passed as the smallest normal number: every product flushes to 0)
+    int pack, head_rows;  // query heads in a tile and the rows of each (attn_tiles.cuh)
+    int tiles;            // query tiles of an item (1 or 2)
+    int steps, inner;     // items of a head group, head groups (two_streams: head pairs) per batch entry
     FastDiv div_heads;  // by the number of items per query step
-    FastDiv div_inner;  // by the head pairs (or heads) per batch entry
+    FastDiv div_inner;  // by `inner`
     FastDiv div_group;  // by the query heads per KV head
-    int sms;
+    int dynamic;        // more items than SMs
     int* status;
 };
 
@@ -185,7 +189,7 @@ struct ItemInfo {
     int b, kvlen;
     int kvh[kTilesPerCta];      // KV head of each tile (equal unless the tiles read separate K/V streams)
     int q0[kTilesPerCta];       // first query row of each of the two tiles
-    int h[kTilesPerCta];        // query head of each tile
+    int h[kTilesPerCta];        // (first) query head of each tile
     int nh[kTilesPerCta];       // 64-key half-steps visible to at least one row of each query tile (0: no work)
     int n_max;                  // the larger of the two
 };
@@ -193,7 +197,9 @@ struct ItemInfo {
 // element t of a two-element array without dynamic indexing (keeps the array in registers)
 __device__ __forceinline__ int pick(const int (&a)[kTilesPerCta], int t) { return t ? a[1] : a[0]; }
 
-template <int D, bool F16, bool BIAS>
+// PACK: several heads per tile.  (A parameter, because the instance with one head per tile is slower when it carries the divisions along:
+// 6 x 12 x 385 causal, D = 128, 12.6 -> 13.0 us.)
+template <int D, bool F16, bool BIAS, bool PACK>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                  const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_o,
@@ -226,20 +232,15 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(smem + L::kNextOff + 16 + 2 * 64);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // The two tiles of an item: with an even number of query heads per KV head, the same 128 query rows of
-    // two heads that share K and V (equal causal lengths, so neither tile waits for the other); otherwise
-    // two consecutive 128-row tiles of one head.
-    const int G = p.Hq / p.Hkv;
-    const bool pair_heads = (G % 2) == 0;
-    // With an odd group size and D = 64 (where shared memory has room for it) the two tiles are still two
-    // heads on the same query rows, each with its own K/V stream through half of the stage ring.
-    const bool two_streams = !pair_heads && kKVStages >= 8;
+    // A tile holds head_rows consecutive query rows of `pack` query heads that share K and V (attn_tiles.cuh).  An item is two
+    // consecutive tiles of a head group, or one (choose_tiles() has the rules).  Without packing at D = 64 (where shared memory
+    // has room for it) the two tiles are two heads on the same query rows instead, each with its own K/V stream through half
+    // of the stage ring.
+    const int head_rows = PACK ? p.head_rows : kBM, pack = PACK ? p.pack : 1;
+    const bool two_streams = !PACK && kKVStages >= 8 && p.tiles == 2;
     const int ring_len = two_streams ? kKVStages / 2 : kKVStages;
-    const int num_q_tiles = (p.Sq + kBM - 1) / kBM;
-    const int head_pairs = (p.Hq + 1) / 2;
-    const int rows_of_items = (pair_heads || two_streams) ? num_q_tiles : (num_q_tiles + 1) / 2;
-    const int heads = (pair_heads || two_streams) ? head_pairs * p.B : p.Hq * p.B;  // items per query step
-    const int num_items = rows_of_items * heads;
+    const int heads = p.inner * p.B;  // items per query step
+    const uint32_t q_bytes = (uint32_t)(pack * head_rows) * (D * 2);
     // ring slot and phase of the g-th KV tile of stream u
     auto kv_slot = [&](int u, int g) { return (two_streams ? u * ring_len : 0) + g % ring_len; };
     auto kv_phase = [&](int g) { return (uint32_t)((g / ring_len) & 1); };
@@ -251,22 +252,23 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     // launch queue, so whoever is done first gets it, whatever the items cost (padding, ragged tiles).  Against a fixed
     // order (item c of every round to CTA c, in alternating direction): 8 x 16/4 heads x 1000 x 1700 with lengths from 300
     // 74 -> 66 us, 2 x 28/4 x 2048 causal 65.6 -> 62.7, 8 x 12 x 1024 causal (an even load) 34.5 -> 34.1.
-    const bool dynamic = num_items > p.sms;  // else everything runs at once and nothing is left to take
+    const bool dynamic = p.dynamic != 0;  // else everything runs at once and nothing is left to take
     auto decode = [&](int i) {
         ItemInfo it;
         const int round_q = fast_div(i, p.div_heads);
-        const int qstep = rows_of_items - 1 - round_q;  // longest (causal) first
+        const int qstep = p.steps - 1 - round_q;  // longest (causal) first
         const int hb = i - round_q * heads;
         it.b = fast_div(hb, p.div_inner);
-        if (pair_heads || two_streams) {
-            const int hp = hb - it.b * head_pairs;
-            it.h[0] = 2 * hp;
-            it.h[1] = min(2 * hp + 1, p.Hq - 1);
-            it.q0[0] = it.q0[1] = qstep * kBM;
-            if (2 * hp + 1 >= p.Hq) it.q0[1] = num_q_tiles * kBM;  // odd head count: no second tile
+        const int in_b = hb - it.b * p.inner;
+        if (two_streams) {
+            it.h[0] = 2 * in_b;
+            it.h[1] = min(2 * in_b + 1, p.Hq - 1);
+            it.q0[0] = qstep * kBM;
+            it.q0[1] = 2 * in_b + 1 < p.Hq ? it.q0[0] : p.Sq;  // odd head count: no second tile
         } else {
-            it.h[0] = it.h[1] = hb - it.b * p.Hq;
-            it.q0[0] = 2 * qstep * kBM; it.q0[1] = (2 * qstep + 1) * kBM;
+            it.h[0] = it.h[1] = in_b * pack;
+            it.q0[0] = p.tiles * qstep * head_rows;
+            it.q0[1] = p.tiles == 2 ? it.q0[0] + head_rows : p.Sq;
         }
         it.kvh[0] = fast_div(it.h[0], p.div_group);
         it.kvh[1] = fast_div(it.h[1], p.div_group);
@@ -277,7 +279,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         for (int t = 0; t < kTilesPerCta; ++t) {
             const int q0 = it.q0[t];
             int kv_end = it.kvlen;
-            if (causal) kv_end = min(kv_end, min(q0 + kBM, p.Sq) + causal_off);
+            if (causal) kv_end = min(kv_end, min(q0 + head_rows, p.Sq) + causal_off);
             if (q0 >= p.Sq) kv_end = 0;
             kv_end = max(kv_end, 0);
             it.nh[t] = (kv_end + kHalf - 1) / kHalf;
@@ -292,13 +294,13 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         if (!(relaxed ? mbar_wait_relaxed(&next_full[n & 1], (n >> 1) & 1) : mbar_wait(&next_full[n & 1], (n >> 1) & 1))) return -1;
         return next_items[(n & 1) * 16];
     };
-    // Sends the rows from row r of query tile q0 on (a whole tile or a quarter of one) off, out of Q buffer `at`, where the output is
-    // staged; the map's box has that many rows.  Rows beyond Sq are clipped by the TMA unit.
-    auto store_rows = [&](const CUtensorMap* map, int at, int r, int q0, int head, int b) {
-        if (q0 + r >= p.Sq) return;
+    // Sends the tile's rows from `row` on off, out of Q buffer `at`, where the output is staged: as many as the map's box has (all
+    // rows in use, or a quarter of the tile).  Rows beyond Sq are clipped by the TMA unit.
+    auto store_rows = [&](const CUtensorMap* map, int at, int row, int q, int head, int b) {
+        if (q >= p.Sq) return;
 #pragma unroll
         for (int c = 0; c < D / 64; ++c)
-            tma_store_4d(map, sQ + at * L::kTileBytes + c * L::kChunkBytes + r * 128, c * 64, q0 + r, head, b);
+            tma_store_4d(map, sQ + at * L::kTileBytes + c * L::kChunkBytes + row * 128, c * 64, q, head, b);
         tma_store_commit();
     };
 
@@ -319,6 +321,13 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     if (warp == 9) {
         tmem_alloc(tmem_base_slot, kTmemCols);
         tmem_relinquish();
+    }
+    // Rows of a Q tile that are not in use are never written by the copies: zero scores, not whatever lies there.
+    if constexpr (PACK) {
+        for (int r = pack * head_rows + (int)threadIdx.x / 8; r < kBM; r += kThreads / 8)
+            for (int c = 0; c < 2 * kTilesPerCta * (D / 64); ++c)
+                *reinterpret_cast<uint4*>(sQ + c * L::kChunkBytes + r * 128 + (threadIdx.x % 8) * 16) = make_uint4(0, 0, 0, 0);
+        fence_proxy_async_smem();
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -344,7 +353,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                     const int u = q_loads[t] & 1, at = t * 2 + u;
                     if (!mbar_wait_relaxed(&q_empty[at], ((q_loads[t] >> 1) & 1) ^ 1)) return false;
                     ++q_loads[t];
-                    mbar_expect_tx(&q_full[at], L::kTileBytes);
+                    mbar_expect_tx(&q_full[at], q_bytes);
 #pragma unroll
                     for (int c = 0; c < D / 64; ++c)  // rows beyond Sq are zero-filled by the TMA unit
                         tma_load_4d(sQ + at * L::kTileBytes + c * L::kChunkBytes, &tmap_q, &q_full[at], c * 64, x.q0[t], x.h[t], x.b);
@@ -575,6 +584,12 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         const int t = warp >> 2;       // query tile of this warp group
         const int quarter = warp & 3;  // TMEM lane quarter this warp may access
         const int row = quarter * 32 + lane;
+        // this thread's query row and head within the tile; a row that is not in use goes along as the last head's row 0 with Q = 0
+        // (one word: row, head * 256, in use * 65536)
+        const int row_at = row < pack * head_rows ? row % head_rows + row / head_rows * 256 + 65536 : (pack - 1) * 256;
+        auto row_q = [&]() { return PACK ? row_at & 255 : row; };
+        auto row_h = [&]() { return PACK ? (row_at >> 8) & 255 : 0; };
+        auto live = [&]() { return PACK ? row_at >= 65536 : true; };
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint32_t col_s = kColS + t * kBN, col_o = kColO + t * D;
         const float sl2 = p.scale_log2;
@@ -596,7 +611,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
             b = it.b; kvlen = it.kvlen; n_max = it.n_max;
         }
         for (int r = 0, state = 1; !failed; ++r) {
-            const int qi = q0 + row;
+            const int qi = q0 + row_q();
             float m_run = -INFINITY;  // running maximum of the raw scores (reference of the exponentials)
             float l_run = 0.f;
             // last visible key of this row
@@ -631,10 +646,16 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 __syncwarp();
                 if (lane == 0) { mbar_arrive(&o_free[t]); mbar_arrive(&o_staged[t * 2 + ((q_uses - 1) & 1)]); }
             }
-            if (state != 1) {  // the CTA's last item (q0, head and b are still its own): no waiting for the other three warps
-                if (pending && lane == 0) {
-                    store_rows(&tmap_o32, t * 2 + ((q_uses - 1) & 1), quarter * 32, q0, head, b);
-                    tma_store_wait_all<0>();  // shared memory is not given up before it has been read
+            if (state != 1) {  // the CTA's last item (q0, head and b are still its own)
+                if (pending) {
+                    const int at = t * 2 + ((q_uses - 1) & 1), r0 = quarter * 32;
+                    if (pack * head_rows == kBM) {  // powers of two, so a warp's rows are a box: no waiting for the other three
+                        if (lane == 0) store_rows(&tmap_o32, at, r0, q0 + r0 % head_rows, head + r0 / head_rows, b);
+                    } else if (quarter == 0) {
+                        if (!warp_wait(&o_staged[at], ((q_uses - 1) >> 1) & 1)) { failed = true; break; }
+                        if (lane == 0) store_rows(&tmap_o, at, 0, q0, head, b);
+                    }
+                    if (lane == 0) tma_store_wait_all<0>();  // shared memory is not given up before it has been read
                 }
                 break;
             }
@@ -656,7 +677,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 [[maybe_unused]] float bias[BIAS ? kHalf + 4 : 1];
                 [[maybe_unused]] int lead = 0;  // elements of the first piece that lie before the row's first
                 if constexpr (BIAS) {
-                    const int hb = p.bias_heads == 1 ? 0 : head;
+                    const int hb = p.bias_heads == 1 ? 0 : head + row_h();
                     const float* brow = p.bias + (((size_t)b * p.bias_heads + hb) * p.Sq + min(qi, p.Sq - 1)) * (size_t)p.Skv + key0;
                     lead = (int)(reinterpret_cast<uintptr_t>(brow) >> 2) & 3;
                     const int nvalid = lead + min(kHalf, p.Skv - key0);  // columns beyond Skv are masked below
@@ -838,11 +859,11 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
             if (failed) break;
             if (nh > 0) {
                 pending = true;
-                out_inv = l_run > 0.f ? 1.f / l_run : 0.f;  // no visible key: zeros
+                out_inv = l_run > 0.f && live() ? 1.f / l_run : 0.f;  // no visible key, row not in use (its Q stays 0): zeros
                 ++q_uses;
                 steps += nh;
-            } else if (qi < p.Sq) {  // no visible key for any row of this tile
-                uint16_t* orow = p.out + b * p.o_sb + head * p.o_sh + qi * p.o_ss;
+            } else if (live() && qi < p.Sq) {  // no visible key for any row of this tile
+                uint16_t* orow = p.out + b * p.o_sb + (head + row_h()) * p.o_sh + qi * p.o_ss;
                 for (int c = 0; c < p.head_dim / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = make_uint4(0, 0, 0, 0);
             }
             kvbase += two_streams ? nh : n_max;
@@ -877,6 +898,31 @@ struct Strides {
 };
 inline Strides dense_strides(int H, int S, int D) { return {(long long)H * S * D, (long long)S * D, (long long)D}; }
 
+// How the query rows are cut into tiles and items.
+struct TilePlan {
+    int pack, head_rows;
+    bool two_streams;
+    int tiles, steps, inner;
+    long long items;
+};
+
+// One tile per item where that leaves no SM with two of them (a lone tile takes a little more than half the time of a pair: 1 x
+// 16 heads x 518 x 80 12.0 -> 10.5 us, 1 x 32/8 x 256 behind 1000 keys 25.0 -> 20.0), else two.
+template <int D>
+TilePlan choose_tiles(int B, int Hq, int Hkv, int Sq, int Skv, int mask_kind, int sms) {
+    TilePlan t;
+    const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, (mask_kind & FORGE_MASK_CAUSAL) != 0);
+    t.pack = hp.pack; t.head_rows = hp.rows;
+    const int q_tiles = (Sq + t.head_rows - 1) / t.head_rows;
+    const long long groups = (long long)(Hq / t.pack) * B;
+    t.tiles = groups * q_tiles <= sms ? 1 : 2;
+    t.two_streams = t.pack == 1 && t.tiles == 2 && AttnSmem<D>::kKVStages >= 8;  // the kernel asks the same
+    t.inner = t.two_streams ? (Hq + 1) / 2 : Hq / t.pack;
+    t.steps = t.two_streams ? q_tiles : (q_tiles + t.tiles - 1) / t.tiles;
+    t.items = (long long)t.inner * B * t.steps;
+    return t;
+}
+
 // D: the kernel's head dimension (64 or 128); head_dim <= D: the tensors' (a multiple of 8).  Columns beyond
 // head_dim are zero-filled on load and clipped on store by the TMA unit, so a padded head costs time, not memory.
 template <int D, bool F16, bool BIAS = false>
@@ -885,21 +931,25 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
                 int bias_heads = 1, const Strides* sq_ = nullptr, const Strides* sk_ = nullptr, const Strides* sv_ = nullptr,
                 const Strides* so_ = nullptr) {
     using L = AttnSmem<D>;
+    const int sms = sm_count();
+    if (sms <= 0) return FORGE_ERR_CUDA;
+    const TilePlan plan = choose_tiles<D>(B, Hq, Hkv, Sq, Skv, mask_kind, sms);
     const Strides sq = sq_ ? *sq_ : dense_strides(Hq, Sq, head_dim), so = so_ ? *so_ : dense_strides(Hq, Sq, head_dim);
     const Strides sk = sk_ ? *sk_ : dense_strides(Hkv, Skv, head_dim), sv = sv_ ? *sv_ : dense_strides(Hkv, Skv, head_dim);
     // every tensor as a 4-D map (D, rows, heads, batch): the strides carry the layout
-    auto encode = [&](CUtensorMap* m, const void* base, int H, int S, const Strides& st, uint32_t box_rows) {
-        const uint32_t box[4] = {64, box_rows, 1, 1};
+    auto encode = [&](CUtensorMap* m, const void* base, int H, int S, const Strides& st, int box_rows, int box_heads = 1) {
+        const uint32_t box[4] = {64, (uint32_t)box_rows, (uint32_t)box_heads, 1};
         const uint64_t dims[4] = {(uint64_t)head_dim, (uint64_t)S, (uint64_t)H, (uint64_t)B};
         const uint64_t strides[3] = {(uint64_t)st.s * 2, (uint64_t)st.h * 2, (uint64_t)st.b * 2};
         return encode_tmap_bf16_sw128(m, base, 4, dims, strides, box);
     };
     CUtensorMap tq, tk, tv, to, to32;
-    if (!encode(&tq, q, Hq, Sq, sq, 128)) return FORGE_ERR_CUDA;
+    if (!encode(&tq, q, Hq, Sq, sq, plan.head_rows, plan.pack)) return FORGE_ERR_CUDA;
     if (!encode(&tk, k, Hkv, Skv, sk, kHalf)) return FORGE_ERR_CUDA;
     if (!encode(&tv, v, Hkv, Skv, sv, kHalf)) return FORGE_ERR_CUDA;
-    if (!encode(&to, out, Hq, Sq, so, 128)) return FORGE_ERR_CUDA;
-    if (!encode(&to32, out, Hq, Sq, so, 32)) return FORGE_ERR_CUDA;  // a softmax warp's rows
+    if (!encode(&to, out, Hq, Sq, so, plan.head_rows, plan.pack)) return FORGE_ERR_CUDA;
+    const int warp_rows = plan.head_rows < 32 ? plan.head_rows : 32;  // a softmax warp's rows, where all 128 are in use
+    if (!encode(&to32, out, Hq, Sq, so, warp_rows, 32 / warp_rows)) return FORGE_ERR_CUDA;
     AttnParams p;
     p.out = static_cast<uint16_t*>(out);
     p.o_sb = so.b; p.o_sh = so.h; p.o_ss = so.s;
@@ -916,24 +966,18 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
     if (!(p.scale_log2 > 0.f)) p.scale_log2 = 1.17549435e-38f;
     p.status = device_status_word();
     if (!p.status) return FORGE_ERR_CUDA;
-    {
-        const int G = Hq / Hkv;
-        const bool by_pairs = (G % 2 == 0) || L::kKVStages >= 8;  // same rule as in the kernel
-        const int inner = by_pairs ? (Hq + 1) / 2 : Hq;
-        p.div_heads = make_fastdiv(inner * B);
-        p.div_inner = make_fastdiv(inner);
-        p.div_group = make_fastdiv(G);
-    }
-    auto kernel = attn_bf16_kernel<D, F16, BIAS>;
-    FORGE_SET_SMEM_ONCE(kernel, L::kAlloc);
-    const int sms = sm_count();
-    if (sms <= 0) return FORGE_ERR_CUDA;
-    const int q_tiles = (Sq + kBM - 1) / kBM;
-    const bool head_pairs = ((Hq / Hkv) % 2 == 0) || L::kKVStages >= 8;  // same rule as in the kernel
-    const long long items = head_pairs ? (long long)((Hq + 1) / 2) * B * q_tiles
-                                       : (long long)Hq * B * ((q_tiles + 1) / 2);
-    p.sms = sms;
-    FORGE_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)items), dim3(kThreads), L::kAlloc, s, tq, tk, tv, to, to32, p));
+    p.pack = plan.pack; p.head_rows = plan.head_rows;
+    p.tiles = plan.tiles;
+    p.steps = plan.steps; p.inner = plan.inner;
+    p.div_heads = make_fastdiv(plan.inner * B);
+    p.div_inner = make_fastdiv(plan.inner);
+    p.div_group = make_fastdiv(Hq / Hkv);
+    p.dynamic = plan.items > sms;
+    const auto packed = attn_bf16_kernel<D, F16, BIAS, true>, plain = attn_bf16_kernel<D, F16, BIAS, false>;
+    const auto kernel = plan.pack > 1 ? packed : plain;
+    if (plan.pack > 1) FORGE_SET_SMEM_ONCE(packed, L::kAlloc);
+    else FORGE_SET_SMEM_ONCE(plain, L::kAlloc);
+    FORGE_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)plan.items), dim3(kThreads), L::kAlloc, s, tq, tk, tv, to, to32, p));
     return finish_launch(1);
 }
 

@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "attn_tiles.cuh"
 #include "attn_wide.cuh"
 #include "forge_common.cuh"
 #include "sm100_ptx.cuh"
@@ -45,8 +46,8 @@ struct WideSmem {
     static constexpr int kKOff = kQOff + kQBytes;
     static constexpr int kVOff = kKOff + kStages * kKVBytes;
     static constexpr int kBarOff = kVOff + kStages * kKVBytes;
-    // q_full, q_empty, k_full[2], k_empty[2], v_full[2], v_empty[2], s_full[2], p_ready[2], pv_done[2], o_free
-    static constexpr int kNumBars = 2 + 4 * kStages + 7;
+    // q_full, q_empty, k_full[2], k_empty[2], v_full[2], v_empty[2], s_full[2], p_ready[2], pv_done[2], o_free, o_staged
+    static constexpr int kNumBars = 2 + 4 * kStages + 8;
     static constexpr int kTotal = kBarOff + kNumBars * 8 + 16;
     static constexpr int kAlloc = kTotal + 1024;
 };
@@ -72,6 +73,7 @@ struct WideParams {
     long long o_sb, o_sh, o_ss;  // element strides of out between batch entries, heads and rows
     const int32_t* lens;
     int B, Hq, Hkv, Sq, Skv, head_dim, mask_kind;
+    int pack, head_rows;  // query heads in a tile and the rows of each (attn_tiles.cuh)
     float scale_log2;  // > 0
     int* status;
 };
@@ -102,12 +104,13 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     uint64_t* p_ready = s_full + 2;          // [2]
     uint64_t* pv_done = p_ready + 2;         // [2] one completion per P V product of that parity
     uint64_t* o_free = pv_done + 2;          // the epilogue has read O
-    uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(o_free + 1);
+    uint64_t* o_staged = o_free + 1;         // all four warps' rows of the output lie in Q's place
+    uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(o_staged + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int G = p.Hq / p.Hkv;
-    const int num_q_tiles = (p.Sq + kBM - 1) / kBM;
-    const int heads = p.B * p.Hq;
+    const int num_q_tiles = (p.Sq + p.head_rows - 1) / p.head_rows;
+    const int groups = p.Hq / p.pack, heads = p.B * groups;
     const int num_items = num_q_tiles * heads;
     const int causal_off = p.Skv - p.Sq;
     const bool causal = (p.mask_kind & FORGE_MASK_CAUSAL) != 0;
@@ -123,14 +126,14 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         WideItem it;
         const int qstep = num_q_tiles - 1 - i / heads;
         const int bh = i % heads;
-        it.b = bh / p.Hq;
-        it.h = bh - it.b * p.Hq;
+        it.b = bh / groups;
+        it.h = (bh - it.b * groups) * p.pack;
         it.kvh = it.h / G;
-        it.q0 = qstep * kBM;
+        it.q0 = qstep * p.head_rows;
         it.kvlen = p.Skv;
         if (padding) it.kvlen = min(max(p.lens[it.b], 0), p.Skv);
         int kv_end = it.kvlen;
-        if (causal) kv_end = min(kv_end, min(it.q0 + kBM, p.Sq) + causal_off);
+        if (causal) kv_end = min(kv_end, min(it.q0 + p.head_rows, p.Sq) + causal_off);
         kv_end = max(kv_end, 0);
         it.nsteps = (kv_end + kStep - 1) / kStep;
         return it;
@@ -144,7 +147,7 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
             mbar_init(&v_full[i], 1); mbar_init(&v_empty[i], 1);
         }
         for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_ready[i], 4); mbar_init(&pv_done[i], 1); }
-        mbar_init(o_free, 4);
+        mbar_init(o_free, 4); mbar_init(o_staged, 4);
         fence_mbar_init();
         prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_o);
     }
@@ -152,6 +155,11 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         tmem_alloc(tmem_base_slot, kTmemCols);
         tmem_relinquish();
     }
+    // Rows of the Q tile that are not in use are never written by the copies: zero scores, not whatever lies there.
+    for (int r = p.pack * p.head_rows + (int)threadIdx.x / 8; r < kBM; r += kThreads / 8)
+        for (int c = 0; c < kD / 64; ++c)
+            *reinterpret_cast<uint4*>(sQ + c * L::kChunkBytes + r * 128 + (threadIdx.x % 8) * 16) = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -172,7 +180,7 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 if (it.nsteps == 0) continue;
                 if (!mbar_wait(q_empty, (q_loads & 1) ^ 1)) { failed = true; break; }
                 ++q_loads;
-                mbar_expect_tx(q_full, L::kQBytes);
+                mbar_expect_tx(q_full, (uint32_t)(p.pack * p.head_rows) * (kD * 2));
 #pragma unroll
                 for (int c = 0; c < kD / 64; ++c)  // rows beyond Sq and columns beyond head_dim are zero-filled
                     tma_load_4d(sQ + c * L::kChunkBytes, &tmap_q, q_full, c * 64, it.q0, it.h, it.b);
@@ -255,19 +263,23 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     } else {
         // ------------------------------------------------------------------ softmax / rescale / epilogue
         const int row = warp * 32 + lane;
+        // head and query row within the tile; a row that is not in use goes along as the last head's first with Q = 0
+        const bool live = row < p.pack * p.head_rows;
+        const int row_h = min(row / p.head_rows, p.pack - 1), row_q = live ? row - row_h * p.head_rows : 0;
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
         const float sl2 = p.scale_log2;
         int steps[2] = {0, 0};  // steps done so far per parity (phases of s_full, pv_done)
         int kvbase = 0;
+        int items = 0;  // items with work so far (phases of o_staged)
         for (int r = 0; !failed; ++r) {
             const int i = item_of_round(r);
             if (i >= num_items) break;
             const WideItem it = decode(i);
-            const int qi = it.q0 + row;
+            const int qi = it.q0 + row_q;
             const int n = it.nsteps;
             if (n == 0) {  // no visible key for any row of this tile: zeros, with plain stores
-                if (qi < p.Sq) {
-                    uint16_t* orow = p.out + it.b * p.o_sb + it.h * p.o_sh + qi * p.o_ss;
+                if (live && qi < p.Sq) {
+                    uint16_t* orow = p.out + it.b * p.o_sb + (it.h + row_h) * p.o_sh + qi * p.o_ss;
                     for (int c = 0; c < p.head_dim / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = make_uint4(0, 0, 0, 0);
                 }
                 continue;
@@ -372,19 +384,27 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
                         w[k] = pack16<F16>(__uint_as_float(cur[c * 8 + 2 * k]) * inv, __uint_as_float(cur[c * 8 + 2 * k + 1]) * inv);
-                    *reinterpret_cast<uint4*>(line + ((((c32 & 1) * 4 + c) ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                    if (live) *reinterpret_cast<uint4*>(line + ((((c32 & 1) * 4 + c) ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
                 }
             }
             tc_fence_before_sync();
             fence_proxy_async_smem();
+            // With all 128 rows in use (powers of two) a warp's rows are a box of their own; else the tile is one.
+            const bool own = p.pack * p.head_rows == kBM;
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(o_free);  // O may be overwritten by the next item's first product
-                const int row0 = it.q0 + warp * 32;
-                if (row0 < p.Sq) {
+                mbar_arrive(o_staged);
+            }
+            if (!own && warp == 0 && !warp_wait(o_staged, items & 1)) { failed = true; break; }
+            ++items;
+            if (lane == 0) {
+                const int r0 = own ? warp * 32 : 0;
+                const int q = it.q0 + r0 % p.head_rows, h = it.h + r0 / p.head_rows;
+                if (q < p.Sq && (own || warp == 0)) {
 #pragma unroll
                     for (int cb = 0; cb < kD / 64; ++cb)
-                        if (cb * 64 < p.head_dim) tma_store_4d(&tmap_o, sQ + cb * L::kChunkBytes + warp * 32 * 128, cb * 64, row0, it.h, it.b);
+                        if (cb * 64 < p.head_dim) tma_store_4d(&tmap_o, sQ + cb * L::kChunkBytes + r0 * 128, cb * 64, q, h, it.b);
                     tma_store_commit();
                     tma_store_wait_read<0>();  // the stores have read the staging rows: Q's place is free again
                 }
@@ -411,22 +431,27 @@ template <bool F16>
 int launch_wide(const void* q, const void* k, const void* v, void* out, int B, int Hq, int Hkv, int Sq, int Skv,
                 int head_dim, int mask_kind, const int32_t* lens, float scale, const long long (*st)[3], cudaStream_t s) {
     using L = WideSmem;
-    auto encode = [&](CUtensorMap* m, const void* base, int H, int S, const long long* str, uint32_t box_rows) {
-        const uint32_t box[4] = {64, box_rows, 1, 1};
+    auto encode = [&](CUtensorMap* m, const void* base, int H, int S, const long long* str, int box_rows, int box_heads = 1) {
+        const uint32_t box[4] = {64, (uint32_t)box_rows, (uint32_t)box_heads, 1};
         const uint64_t dims[4] = {(uint64_t)head_dim, (uint64_t)S, (uint64_t)H, (uint64_t)B};
         const uint64_t strides[3] = {(uint64_t)str[2] * 2, (uint64_t)str[1] * 2, (uint64_t)str[0] * 2};
         return encode_tmap_bf16_sw128(m, base, 4, dims, strides, box);
     };
     CUtensorMap tq, tk, tv, to;
-    if (!encode(&tq, q, Hq, Sq, st[0], kBM)) return FORGE_ERR_CUDA;
+    const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, (mask_kind & FORGE_MASK_CAUSAL) != 0);
+    if (!encode(&tq, q, Hq, Sq, st[0], hp.rows, hp.pack)) return FORGE_ERR_CUDA;
     if (!encode(&tk, k, Hkv, Skv, st[1], kStep)) return FORGE_ERR_CUDA;
     if (!encode(&tv, v, Hkv, Skv, st[2], kStep)) return FORGE_ERR_CUDA;
-    if (!encode(&to, out, Hq, Sq, st[3], 32)) return FORGE_ERR_CUDA;
+    // the output leaves in boxes of a warp's rows where all 128 are in use, else of the whole tile (the kernel asks the same)
+    const int warp_rows = hp.rows < 32 ? hp.rows : 32;
+    const bool own = hp.pack * hp.rows == kBM;
+    if (!encode(&to, out, Hq, Sq, st[3], own ? warp_rows : hp.rows, own ? 32 / warp_rows : hp.pack)) return FORGE_ERR_CUDA;
     WideParams p;
     p.out = static_cast<uint16_t*>(out);
     p.o_sb = st[3][0]; p.o_sh = st[3][1]; p.o_ss = st[3][2];
     p.lens = lens;
     p.B = B; p.Hq = Hq; p.Hkv = Hkv; p.Sq = Sq; p.Skv = Skv; p.head_dim = head_dim; p.mask_kind = mask_kind;
+    p.pack = hp.pack; p.head_rows = hp.rows;
     p.scale_log2 = scale * 1.4426950408889634f;
     // scale = 0 (uniform weights): any positive multiplier whose products with the scores flush to zero
     if (!(p.scale_log2 > 0.f)) p.scale_log2 = 1.17549435e-38f;
@@ -436,7 +461,7 @@ int launch_wide(const void* q, const void* k, const void* v, void* out, int B, i
     FORGE_SET_SMEM_ONCE(kernel, L::kAlloc);
     const int sms = sm_count();
     if (sms <= 0) return FORGE_ERR_CUDA;
-    const long long items = (long long)B * Hq * ((Sq + kBM - 1) / kBM);
+    const long long items = (long long)B * (Hq / hp.pack) * ((Sq + hp.rows - 1) / hp.rows);
     const int grid = items < sms ? (int)items : sms;
     FORGE_CUDA_TRY(launch_pdl(kernel, dim3(grid), dim3(kThreads), L::kAlloc, s, tq, tk, tv, to, p));
     return finish_launch(1);
