@@ -33,11 +33,10 @@
 // per CTA that is 0.4 us (6 x 12 heads x 385 causal, D = 128, 12.56 -> 12.15; 8 x 12 x 1024 x 64 32.26 -> 31.8).
 // Reading the output only after the next item's first half-step gained nothing more and cost short items their overlap
 // (64 x 16/4 x 64: 16.7 -> 21.3 us).  At D = 128 long runs are at the power limit: fewer cycles, lower clock.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include <type_traits>
 
+#include "attn_math.cuh"
+#include "attn_narrow.cuh"
 #include "attn_tiles.cuh"
 #include "attn_wide.cuh"
 #include "forge_common.cuh"
@@ -83,69 +82,6 @@ struct AttnSmem {
     static constexpr int kTotal = kNextOff + 16 + 2 * 64 + 16;
     static constexpr int kAlloc = kTotal + 1024;
 };
-
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// 3-input maximum and packed two-wide fp32 arithmetic (one instruction for two elements)
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
-    float2 d;
-    asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
-        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
-        "fma.rn.f32x2 rd, ra, rb, rc;\n\t"
-        "mov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
-    float2 d;
-    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
-        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-        "add.rn.f32x2 rd, ra, rb;\n\t"
-        "mov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
-}
-
-// 2^x for two values on the FMA and integer pipes instead of the special-function unit (which is the
-// narrowest pipe of the softmax): x = n + f with n = round(x), f in [-0.5, 0.5]; 2^f by a cubic with a
-// relative error of 7.6e-5 (far below the bf16 rounding of P); n is added to the exponent field.
-// Inputs below -125 give 2^-125 rather than 0, so this is used only where no score is masked.
-__device__ __forceinline__ float2 ex2_fma2(float2 x) {
-    const float kMagic = 12582912.f;  // 1.5 * 2^23: adding it leaves round(x) in the low mantissa bits
-    x.x = fmaxf(x.x, -125.f);
-    x.y = fmaxf(x.y, -125.f);
-    const float2 t = fadd2(x, make_float2(kMagic, kMagic));
-    const float2 n = fadd2(t, make_float2(-kMagic, -kMagic));
-    const float2 f = ffma2(n, make_float2(-1.f, -1.f), x);
-    float2 q = ffma2(f, make_float2(0.05520550534f, 0.05520550534f), make_float2(0.2426139712f, 0.2426139712f));
-    q = ffma2(q, f, make_float2(0.6932547688f, 0.6932547688f));
-    q = ffma2(q, f, make_float2(0.9999276996f, 0.9999276996f));
-    return make_float2(__int_as_float(__float_as_int(q.x) + (__float_as_int(t.x) << 23)),
-                       __int_as_float(__float_as_int(q.y) + (__float_as_int(t.y) << 23)));
-}
-
-// two fp32 values rounded to nearest even and packed as bf16 (F16 = false) or fp16 (F16 = true)
-template <bool F16>
-__device__ __forceinline__ uint32_t pack16(float lo, float hi) {
-    if constexpr (F16) {
-        __half2 v = __floats2half2_rn(lo, hi);
-        return *reinterpret_cast<uint32_t*>(&v);
-    } else {
-        __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-        return *reinterpret_cast<uint32_t*>(&v);
-    }
-}
 
 // Division by a divisor fixed at launch: floor(n / d) = high 64 bits of n * ceil(2^64 / d) for 0 <= n < 2^32.
 struct FastDiv {
@@ -927,15 +863,14 @@ TilePlan choose_tiles(int B, int Hq, int Hkv, int Sq, int Skv, int mask_kind, in
 // head_dim are zero-filled on load and clipped on store by the TMA unit, so a padded head costs time, not memory.
 template <int D, bool F16, bool BIAS = false>
 int launch_attn(const void* q, const void* k, const void* v, void* out, int B, int Hq, int Hkv, int Sq, int Skv,
-                int head_dim, int mask_kind, const int32_t* lens, float scale, cudaStream_t s, const float* bias = nullptr,
-                int bias_heads = 1, const Strides* sq_ = nullptr, const Strides* sk_ = nullptr, const Strides* sv_ = nullptr,
-                const Strides* so_ = nullptr) {
+                int head_dim, int mask_kind, const int32_t* lens, float scale, cudaStream_t s, const Strides* strides = nullptr,
+                const float* bias = nullptr, int bias_heads = 1) {
     using L = AttnSmem<D>;
     const int sms = sm_count();
     if (sms <= 0) return FORGE_ERR_CUDA;
     const TilePlan plan = choose_tiles<D>(B, Hq, Hkv, Sq, Skv, mask_kind, sms);
-    const Strides sq = sq_ ? *sq_ : dense_strides(Hq, Sq, head_dim), so = so_ ? *so_ : dense_strides(Hq, Sq, head_dim);
-    const Strides sk = sk_ ? *sk_ : dense_strides(Hkv, Skv, head_dim), sv = sv_ ? *sv_ : dense_strides(Hkv, Skv, head_dim);
+    const Strides a = dense_strides(Hq, Sq, head_dim), c = dense_strides(Hkv, Skv, head_dim);
+    const Strides sq = strides ? strides[0] : a, sk = strides ? strides[1] : c, sv = strides ? strides[2] : c, so = strides ? strides[3] : a;
     // every tensor as a 4-D map (D, rows, heads, batch): the strides carry the layout
     auto encode = [&](CUtensorMap* m, const void* base, int H, int S, const Strides& st, int box_rows, int box_heads = 1) {
         const uint32_t box[4] = {64, (uint32_t)box_rows, (uint32_t)box_heads, 1};
@@ -981,12 +916,19 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
     return finish_launch(1);
 }
 
-// Head sizes above 128 run on the one-tile-per-CTA kernel of attn_wide.cu.
-int wide_dense(bool f16, const void* q, const void* k, const void* v, void* out, int B, int Hq, int Hkv, int Sq, int Skv,
-               int D, int mask_kind, const int32_t* lens, float scale, cudaStream_t s) {
-    const Strides a = dense_strides(Hq, Sq, D), c = dense_strides(Hkv, Skv, D);
-    const long long st[4][3] = {{a.b, a.h, a.s}, {c.b, c.h, c.s}, {c.b, c.h, c.s}, {a.b, a.h, a.s}};
-    return attn_wide(f16, q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, st, s);
+// No bias: head sizes up to 64 run on the kernel of attn_narrow.cu, those above 128 on that of attn_wide.cu.  strides: of q, k, v, out,
+// or nullptr for dense tensors.
+template <bool F16>
+int attn_by_head_size(const void* q, const void* k, const void* v, void* out, int B, int Hq, int Hkv, int Sq, int Skv, int D,
+                      int mask_kind, const int32_t* lens, float scale, cudaStream_t s, const Strides* strides = nullptr) {
+    if (D > 64 && D <= 128)
+        return launch_attn<128, F16>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, strides);
+    const Strides a = dense_strides(Hq, Sq, D), c = dense_strides(Hkv, Skv, D), dense[4] = {a, c, c, a};
+    const Strides* t = strides ? strides : dense;
+    long long st[4][3];
+    for (int i = 0; i < 4; ++i) { st[i][0] = t[i].b; st[i][1] = t[i].h; st[i][2] = t[i].s; }
+    return D <= 64 ? attn_narrow(F16, q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, st, s)
+                   : attn_wide(F16, q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, st, s);
 }
 
 }  // namespace
@@ -1001,9 +943,7 @@ extern "C" int forge_attn_fused(const void* q, const void* k, const void* v, voi
     if ((long long)Hq * B * ((Sq + 127) / 128) > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
     if (!(scale >= 0.f)) return FORGE_ERR_UNSUPPORTED;  // the running maximum is taken on unscaled scores
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (D > 128) return wide_dense(false, q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s);
-    return D <= 64 ? launch_attn<64, false>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s)
-                   : launch_attn<128, false>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s);
+    return attn_by_head_size<false>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s);
 }
 
 extern "C" int forge_attn_fused_f16(const void* q, const void* k, const void* v, void* out,
@@ -1015,9 +955,7 @@ extern "C" int forge_attn_fused_f16(const void* q, const void* k, const void* v,
     if ((long long)Hq * B * ((Sq + 127) / 128) > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
     if (!(scale >= 0.f)) return FORGE_ERR_UNSUPPORTED;  // the running maximum is taken on unscaled scores
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (D > 128) return wide_dense(true, q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s);
-    return D <= 64 ? launch_attn<64, true>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s)
-                   : launch_attn<128, true>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s);
+    return attn_by_head_size<true>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s);
 }
 
 extern "C" int forge_attn_fused_bias(const void* q, const void* k, const void* v, void* out,
@@ -1032,8 +970,8 @@ extern "C" int forge_attn_fused_bias(const void* q, const void* k, const void* v
     if ((long long)Hq * B * ((Sq + 255) / 256) > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
     if (!(scale > 0.f)) return FORGE_ERR_UNSUPPORTED;  // the bias enters the kernel as bias / scale
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    return D <= 64 ? launch_attn<64, false, true>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, bias, bias_heads)
-                   : launch_attn<128, false, true>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, bias, bias_heads);
+    return D <= 64 ? launch_attn<64, false, true>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, nullptr, bias, bias_heads)
+                   : launch_attn<128, false, true>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, nullptr, bias, bias_heads);
 }
 
 extern "C" int forge_attn_fused_strided(const void* q, const void* k, const void* v, void* out,
@@ -1057,13 +995,5 @@ extern "C" int forge_attn_fused_strided(const void* q, const void* k, const void
         if (str[i].b >= (1LL << 38) || str[i].h >= (1LL << 38) || str[i].s >= (1LL << 38)) return FORGE_ERR_UNSUPPORTED;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (D > 128) {
-        long long w[4][3];
-        for (int i = 0; i < 4; ++i) { w[i][0] = str[i].b; w[i][1] = str[i].h; w[i][2] = str[i].s; }
-        return attn_wide(false, q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, w, s);
-    }
-    return D <= 64 ? launch_attn<64, false>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, nullptr, 1,
-                                            &str[0], &str[1], &str[2], &str[3])
-                   : launch_attn<128, false>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, nullptr, 1,
-                                             &str[0], &str[1], &str[2], &str[3]);
+    return attn_by_head_size<false>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, str);
 }

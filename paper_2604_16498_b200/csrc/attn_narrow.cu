@@ -1,0 +1,361 @@
+// Fused attention for head sizes up to 64 (Eq. 8 / Eq. 9, the same operator as attn_bf16.cu, without an additive bias).
+//
+// With 64 columns of output a 64-key step is 256 cycles of tensor core against 512 of the special-function unit's exponentials, and
+// the rest of a step (barriers, tensor-memory round trips, fences) is as long as both.  So the kernel is small and the SM
+// holds four of its CTAs: one query tile of 128 rows each, 160 threads, 48 KB of shared memory and 128 tensor-memory columns.
+// While one tile waits for its MMAs, its loads or its next item's start, the other three keep the special-function unit busy, and
+// the hardware scheduler hands out the tiles, longest first.  (Two tiles per SM in one persistent CTA, with two score buffers each:
+// about 950 cycles per tile and step.)
+//
+//   tensor memory   S at column 0 (64 fp32 columns), O at 64; P (16-bit, two per column) overwrites the first 32 columns of S and
+//                   is the A operand of P V
+//   shared memory   Q 16 KB (the output is staged in its place), two stages of 64 keys for K and two for V, 8 KB each
+//   warps 0-3       softmax, rescale and epilogue: thread = tile row = TMEM lane
+//   warp 4          one lane issues the copies and the MMAs; the warp owns the TMEM allocation
+// Per step g:  S(g) = Q K(g)^T complete -> softmax -> O += P(g) V(g), S(g + 1) = Q K(g + 1)^T.  MMAs of one thread execute in issue
+// order, so P(g) is read before S(g + 1) overwrites it, and S(g + 1)'s barrier also covers O.  S(g) complete means that K's
+// stage g % 2 and V's stage (g + 1) % 2 are free again: their next tiles are asked for then, most of a step before they are needed.
+// O is rescaled in tensor memory only when a row's maximum grows by more than 2^8 (the stale maximum is kept otherwise; the final
+// division by l uses the same reference).
+#include "attn_math.cuh"
+#include "attn_narrow.cuh"
+#include "attn_tiles.cuh"
+#include "forge_common.cuh"
+#include "sm100_ptx.cuh"
+#include "tmap.cuh"
+
+namespace forge {
+namespace {
+
+using namespace ptx;
+
+constexpr int kD = 64;            // the kernel's head dimension
+constexpr int kBM = 128;          // rows of a tile
+constexpr int kStep = 64;         // keys per step and per K/V stage
+constexpr int kThreads = 160;
+constexpr int kCtasPerSm = 4;
+constexpr int kTmemCols = 128;
+constexpr int kColO = 64;
+constexpr float kRescaleThreshold = 8.0f;  // log2 units
+
+struct NarrowSmem {
+    static constexpr int kQBytes = kBM * 128;
+    static constexpr int kKVBytes = kStep * 128;
+    static constexpr int kKOff = kQBytes;
+    static constexpr int kVOff = kKOff + 2 * kKVBytes;
+    static constexpr int kBarOff = kVOff + 2 * kKVBytes;
+    static constexpr int kNumBars = 8;  // q_full, k_full[2], v_full[2], s_full, p_ready, o_staged
+    static constexpr int kTotal = kBarOff + kNumBars * 8 + 16;
+    static constexpr int kAlloc = kTotal + 1024;
+};
+
+struct NarrowParams {
+    uint16_t* out;
+    long long o_sb, o_sh, o_ss;  // element strides of out between batch entries, heads and rows
+    const int32_t* lens;
+    int B, Hq, Hkv, Sq, Skv, head_dim, mask_kind;
+    int pack, head_rows;  // query heads in a tile and the rows of each (attn_tiles.cuh)
+    float scale_log2;     // > 0
+    int* status;
+};
+
+template <bool F16>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
+                   const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_o,
+                   const NarrowParams p) {
+    using L = NarrowSmem;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* sQ = smem;
+    uint8_t* sK = smem + L::kKOff;
+    uint8_t* sV = smem + L::kVOff;
+    uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
+    uint64_t* k_full = q_full + 1;   // [2] by step parity
+    uint64_t* v_full = k_full + 2;   // [2]
+    uint64_t* s_full = v_full + 2;   // S(g) is complete, and so is every MMA before it; once more after the last product
+    uint64_t* p_ready = s_full + 1;
+    uint64_t* o_staged = p_ready + 1;  // all four warps' rows of the output lie in Q's place
+    uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(o_staged + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int causal_off = p.Skv - p.Sq;
+    const bool causal = (p.mask_kind & FORGE_MASK_CAUSAL) != 0, padding = (p.mask_kind & FORGE_MASK_PADDING) != 0;
+    // tiles longest first (causal): the last rows of every head group, then the ones before, ...
+    const int groups = p.Hq / p.pack, heads = p.B * groups, q_tiles = (int)gridDim.x / heads;
+    const int round = (int)blockIdx.x / heads, bg = (int)blockIdx.x - round * heads;
+    const int b = bg / groups, head = (bg - b * groups) * p.pack, kvh = head / (p.Hq / p.Hkv);
+    const int q0 = (q_tiles - 1 - round) * p.head_rows;
+
+    if (threadIdx.x == 0) {
+        mbar_init(q_full, 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(&k_full[i], 1); mbar_init(&v_full[i], 1); }
+        mbar_init(s_full, 1); mbar_init(p_ready, 4); mbar_init(o_staged, 4);
+        fence_mbar_init();
+        prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_o);
+    }
+    if (warp == 4) {
+        tmem_alloc(tmem_base_slot, kTmemCols);
+        tmem_relinquish();
+    }
+    // Rows of the Q tile that are not in use are never written by the copy: zero scores, not whatever lies there.
+    const int rows = p.pack * p.head_rows;
+    if (rows < kBM) {
+        for (int i = rows * 8 + (int)threadIdx.x; i < kBM * 8; i += kThreads) reinterpret_cast<uint4*>(sQ)[i] = make_uint4(0, 0, 0, 0);
+        fence_proxy_async_smem();
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem_base = *tmem_base_slot;
+    bool failed = false;
+    pdl_launch_dependents();
+    pdl_wait();
+
+    int kvlen = p.Skv;
+    if (padding) kvlen = min(max(p.lens[b], 0), p.Skv);
+    const int kv_end = max(causal ? min(kvlen, min(q0 + p.head_rows, p.Sq) + causal_off) : kvlen, 0);
+    const int n = (kv_end + kStep - 1) / kStep;  // steps visible to at least one row of the tile
+
+    if (warp == 4) {
+        // ------------------------------------------------------------------ copies and MMAs
+        if (n > 0 && elect_one()) {
+            constexpr uint32_t idesc_s = F16 ? make_idesc_f16(kBM, kStep, false, false) : make_idesc_bf16(kBM, kStep, false, false);
+            constexpr uint32_t idesc_o = F16 ? make_idesc_f16(kBM, kD, false, true) : make_idesc_bf16(kBM, kD, false, true);
+            const uint64_t qd = make_smem_desc(smem_u32(sQ), 16, 1024);
+            auto load_k = [&](int g) {
+                mbar_expect_tx(&k_full[g & 1], L::kKVBytes);
+                tma_load_4d(sK + (g & 1) * L::kKVBytes, &tmap_k, &k_full[g & 1], 0, g * kStep, kvh, b);
+            };
+            auto load_v = [&](int g) {
+                mbar_expect_tx(&v_full[g & 1], L::kKVBytes);
+                tma_load_4d(sV + (g & 1) * L::kKVBytes, &tmap_v, &v_full[g & 1], 0, g * kStep, kvh, b);
+            };
+            auto issue_qk = [&](int g) {
+                tc_fence_after_sync();
+                const uint64_t kd = make_smem_desc(smem_u32(sK) + (g & 1) * L::kKVBytes, 16, 1024);
+#pragma unroll
+                for (int kk = 0; kk < kD / 16; ++kk) mma_ss(tmem_base, qd + kk * (32 >> 4), kd + kk * (32 >> 4), idesc_s, kk != 0);
+                mma_commit(s_full);
+            };
+            // rows beyond Sq and columns beyond head_dim are zero-filled by the TMA unit
+            mbar_expect_tx(q_full, (uint32_t)rows * 128);
+            tma_load_4d(sQ, &tmap_q, q_full, 0, q0, head, b);
+            load_k(0);
+            load_v(0);
+            if (n > 1) load_k(1);
+            if (!mbar_wait(q_full, 0) || !mbar_wait(&k_full[0], 0)) failed = true;
+            if (!failed) issue_qk(0);
+            for (int g = 0; g < n && !failed; ++g) {
+                if (!mbar_wait(s_full, g & 1)) { failed = true; break; }
+                if (g + 2 < n) load_k(g + 2);
+                if (g + 1 < n) load_v(g + 1);
+                // the operands of the next MMAs, before the probabilities: then those go out back to back
+                if (!mbar_wait(&v_full[g & 1], (g >> 1) & 1)) { failed = true; break; }
+                if (g + 1 < n && !mbar_wait(&k_full[(g + 1) & 1], ((g + 1) >> 1) & 1)) { failed = true; break; }
+                if (!mbar_wait(p_ready, g & 1)) { failed = true; break; }
+                tc_fence_after_sync();
+                // P: 16 keys = 8 columns of packed pairs.  V: MN-major, 16 keys = two 1024-byte groups (2048 bytes per MMA).
+                const uint64_t vd = make_smem_desc(smem_u32(sV) + (g & 1) * L::kKVBytes, L::kKVBytes, 1024);
+#pragma unroll
+                for (int kk = 0; kk < kStep / 16; ++kk)
+                    mma_ts(tmem_base + kColO, tmem_base + kk * 8, vd + kk * (2048 >> 4), idesc_o, (g | kk) != 0);
+                if (g + 1 < n) issue_qk(g + 1);
+                else mma_commit(s_full);
+            }
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------------------------ softmax / rescale / epilogue
+        const int row = warp * 32 + lane;
+        // head and query row within the tile; a row that is not in use goes along as the last head's first with Q = 0
+        const bool live = row < rows;
+        const int row_h = min(row / p.head_rows, p.pack - 1), qi = q0 + (live ? row - row_h * p.head_rows : 0);
+        const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
+        const float sl2 = p.scale_log2;
+        float m_run = -INFINITY, l_run = 0.f;  // running maximum of the raw scores (reference of the exponentials), sum
+        const int row_limit = min(kvlen - 1, causal ? qi + causal_off : 0x7fffffff);  // last visible key of this row
+#pragma unroll 1
+        for (int g = 0; g < n; ++g) {
+            const int key0 = g * kStep;
+            if (!warp_wait(s_full, g & 1)) { failed = true; break; }
+            tc_fence_after_sync();
+            float s[kStep];
+#pragma unroll
+            for (int c = 0; c < kStep / 32; ++c) {
+                uint32_t rr[32];
+                tmem_ld_x32(lane_base + c * 32, rr);
+#pragma unroll
+                for (int k = 0; k < 32; ++k) s[c * 32 + k] = __uint_as_float(rr[k]);
+            }
+            tmem_ld_wait();
+            const int lim = row_limit - key0;  // last visible column of this step
+            if (__any_sync(0xffffffffu, lim < kStep - 1)) {
+#pragma unroll
+                for (int k = 0; k < kStep; ++k) s[k] = (k <= lim) ? s[k] : -INFINITY;
+            }
+            float mx[4] = {s[0], s[1], s[2], s[3]};
+#pragma unroll
+            for (int k = 4; k + 7 < kStep; k += 8) {
+                mx[0] = max3(mx[0], s[k], s[k + 1]);
+                mx[1] = max3(mx[1], s[k + 2], s[k + 3]);
+                mx[2] = max3(mx[2], s[k + 4], s[k + 5]);
+                mx[3] = max3(mx[3], s[k + 6], s[k + 7]);
+            }
+            mx[0] = max3(mx[0], s[kStep - 4], s[kStep - 3]);
+            mx[1] = max3(mx[1], s[kStep - 2], s[kStep - 1]);
+            const float m_tile = max3(fmaxf(mx[0], mx[1]), mx[2], mx[3]);
+            // keep the old reference unless this step's maximum exceeds it by more than the threshold
+            bool grow = (m_tile - m_run) * sl2 > kRescaleThreshold || m_run == -INFINITY;
+            if (m_tile == -INFINITY) grow = false;
+            if (__any_sync(0xffffffffu, grow)) {
+                float alpha = 1.f;
+                if (grow) {
+                    // first visible keys of this row: nothing accumulated yet, nothing to rescale
+                    alpha = (m_run == -INFINITY) ? 1.f : ex2((m_run - m_tile) * sl2);
+                    m_run = m_tile;
+                }
+                l_run *= alpha;
+                if (g > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
+#pragma unroll 1
+                    for (int c = 0; c < kD / 16; ++c) {
+                        uint32_t rr[16];
+                        tmem_ld_x16(lane_base + kColO + c * 16, rr);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) rr[k] = __float_as_uint(__uint_as_float(rr[k]) * alpha);
+                        tmem_st_x16(lane_base + kColO + c * 16, rr);
+                    }
+                }
+            }
+            const float m_ref = (m_run == -INFINITY) ? 0.f : m_run;
+            const float2 sl2v = make_float2(sl2, sl2), neg_m = make_float2(-m_ref * sl2, -m_ref * sl2);
+            float2 lsum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            uint32_t packed[32];
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+                const float2 x = ffma2(make_float2(s[2 * k], s[2 * k + 1]), sl2v, neg_m);
+                const float2 pr = make_float2(ex2(x.x), ex2(x.y));  // masked: 0
+                lsum[k & 1] = fadd2(lsum[k & 1], pr);
+                packed[k] = pack16<F16>(pr.x, pr.y);
+            }
+            tmem_st_x32(lane_base, packed);
+            l_run += (lsum[0].x + lsum[0].y) + (lsum[1].x + lsum[1].y);
+            // V rows at and beyond lens[b] hold the caller's padding (possibly NaN, and 0 x NaN is NaN): zero them before the
+            // product may start.  Rows beyond Skv were zero-filled by the copy itself.
+            if (padding && key0 + kStep > kvlen && kvlen < p.Skv) {
+                if (!warp_wait(&v_full[g & 1], (g >> 1) & 1)) { failed = true; break; }
+                uint4* vt = reinterpret_cast<uint4*>(sV + (g & 1) * L::kKVBytes);
+                for (int i = max(kvlen - key0, 0) * 8 + row; i < kStep * 8; i += 128) vt[i] = make_uint4(0, 0, 0, 0);
+                fence_proxy_async_smem();
+            }
+            tmem_st_wait();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(p_ready);
+        }
+        if (n == 0) {  // no visible key for any row of this tile: zeros, with plain stores
+            if (live && qi < p.Sq) {
+                uint16_t* orow = p.out + b * p.o_sb + (head + row_h) * p.o_sh + qi * p.o_ss;
+                for (int c = 0; c < p.head_dim / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = make_uint4(0, 0, 0, 0);
+            }
+        } else if (!failed && warp_wait(s_full, n & 1)) {  // the last product
+            tc_fence_after_sync();
+            // O / l as 16-bit values into Q's place (all scores are done), in the copies' 128-byte swizzle
+            const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+            uint8_t* line = sQ + row * 128;
+#pragma unroll
+            for (int c32 = 0; c32 < 2; ++c32) {
+                uint32_t cur[32];
+                tmem_ld_x32(lane_base + kColO + c32 * 32, cur);
+                tmem_ld_wait();
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        w[k] = pack16<F16>(__uint_as_float(cur[c * 8 + 2 * k]) * inv, __uint_as_float(cur[c * 8 + 2 * k + 1]) * inv);
+                    *reinterpret_cast<uint4*>(line + (((c32 * 4 + c) ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (rows == kBM) {  // powers of two, so a warp's rows are a box: no waiting for the other three
+                const int r0 = warp * 32, q = q0 + r0 % p.head_rows;
+                if (lane == 0 && q < p.Sq) tma_store_4d(&tmap_o, sQ + r0 * 128, 0, q, head + r0 / p.head_rows, b);
+            } else {
+                if (lane == 0) mbar_arrive(o_staged);
+                if (warp == 0) {
+                    if (!warp_wait(o_staged, 0)) failed = true;
+                    else if (lane == 0) tma_store_4d(&tmap_o, sQ, 0, q0, head, b);
+                }
+            }
+            if (lane == 0) {
+                tma_store_commit();
+                tma_store_wait_all<0>();
+            }
+            __syncwarp();
+        } else {
+            failed = true;
+        }
+    }
+
+    if (failed) {
+        atomicExch(p.status, 1);
+        for (int i = 0; i < 2000; ++i) __nanosleep(1000);  // let copies and MMAs in flight land
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == 4) {
+        tc_fence_after_sync();
+        tmem_dealloc(tmem_base, kTmemCols);
+    }
+}
+
+template <bool F16>
+int launch_narrow(const void* q, const void* k, const void* v, void* out, int B, int Hq, int Hkv, int Sq, int Skv,
+                  int head_dim, int mask_kind, const int32_t* lens, float scale, const long long (*st)[3], cudaStream_t s) {
+    using L = NarrowSmem;
+    auto encode = [&](CUtensorMap* m, const void* base, int H, int S, const long long* str, int box_rows, int box_heads = 1) {
+        const uint32_t box[4] = {64, (uint32_t)box_rows, (uint32_t)box_heads, 1};
+        const uint64_t dims[4] = {(uint64_t)head_dim, (uint64_t)S, (uint64_t)H, (uint64_t)B};
+        const uint64_t strides[3] = {(uint64_t)str[2] * 2, (uint64_t)str[1] * 2, (uint64_t)str[0] * 2};
+        return encode_tmap_bf16_sw128(m, base, 4, dims, strides, box);
+    };
+    CUtensorMap tq, tk, tv, to;
+    const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, (mask_kind & FORGE_MASK_CAUSAL) != 0);
+    if (!encode(&tq, q, Hq, Sq, st[0], hp.rows, hp.pack)) return FORGE_ERR_CUDA;
+    if (!encode(&tk, k, Hkv, Skv, st[1], kStep)) return FORGE_ERR_CUDA;
+    if (!encode(&tv, v, Hkv, Skv, st[2], kStep)) return FORGE_ERR_CUDA;
+    // the output leaves in boxes of a warp's rows where all 128 are in use, else of the whole tile (the kernel asks the same)
+    const int warp_rows = hp.rows < 32 ? hp.rows : 32;
+    const bool own = hp.pack * hp.rows == kBM;
+    if (!encode(&to, out, Hq, Sq, st[3], own ? warp_rows : hp.rows, own ? 32 / warp_rows : hp.pack)) return FORGE_ERR_CUDA;
+    NarrowParams p;
+    p.out = static_cast<uint16_t*>(out);
+    p.o_sb = st[3][0]; p.o_sh = st[3][1]; p.o_ss = st[3][2];
+    p.lens = lens;
+    p.B = B; p.Hq = Hq; p.Hkv = Hkv; p.Sq = Sq; p.Skv = Skv; p.head_dim = head_dim; p.mask_kind = mask_kind;
+    p.pack = hp.pack; p.head_rows = hp.rows;
+    p.scale_log2 = scale * 1.4426950408889634f;
+    // scale = 0 (uniform weights): any positive multiplier whose products with the scores flush to zero
+    if (!(p.scale_log2 > 0.f)) p.scale_log2 = 1.17549435e-38f;
+    p.status = device_status_word();
+    if (!p.status) return FORGE_ERR_CUDA;
+    const auto kernel = attn_narrow_kernel<F16>;
+    FORGE_SET_SMEM_ONCE(kernel, L::kAlloc);
+    const long long tiles = (long long)B * (Hq / hp.pack) * ((Sq + hp.rows - 1) / hp.rows);
+    if (tiles > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
+    FORGE_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)tiles), dim3(kThreads), L::kAlloc, s, tq, tk, tv, to, p));
+    return finish_launch(1);
+}
+
+}  // namespace
+
+int attn_narrow(bool f16, const void* q, const void* k, const void* v, void* out, int B, int Hq, int Hkv, int Sq, int Skv,
+                int head_dim, int mask_kind, const int32_t* lens, float scale, const long long (*strides)[3], cudaStream_t s) {
+    return f16 ? launch_narrow<true>(q, k, v, out, B, Hq, Hkv, Sq, Skv, head_dim, mask_kind, lens, scale, strides, s)
+               : launch_narrow<false>(q, k, v, out, B, Hq, Hkv, Sq, Skv, head_dim, mask_kind, lens, scale, strides, s);
+}
+
+}  // namespace forge

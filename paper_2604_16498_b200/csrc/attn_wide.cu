@@ -13,9 +13,7 @@
 // only when a row's maximum grows by more than 2^8 (the stale maximum is kept otherwise; the final division by
 // l uses the same reference).  Head sizes that are not 256 (multiples of 8) cost time, not memory: the TMA unit
 // zero-fills the missing columns on load and clips them on store.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
+#include "attn_math.cuh"
 #include "attn_tiles.cuh"
 #include "attn_wide.cuh"
 #include "forge_common.cuh"
@@ -51,22 +49,6 @@ struct WideSmem {
     static constexpr int kTotal = kBarOff + kNumBars * 8 + 16;
     static constexpr int kAlloc = kTotal + 1024;
 };
-
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-template <bool F16>
-__device__ __forceinline__ uint32_t pack16(float lo, float hi) {
-    if constexpr (F16) {
-        __half2 v = __floats2half2_rn(lo, hi);
-        return *reinterpret_cast<uint32_t*>(&v);
-    } else {
-        __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-        return *reinterpret_cast<uint32_t*>(&v);
-    }
-}
 
 struct WideParams {
     uint16_t* out;
