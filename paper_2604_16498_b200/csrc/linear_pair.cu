@@ -92,10 +92,10 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const int num_tiles = tiles_m * tiles_n;
     const int kblocks = (K + kBK - 1) / kBK;
     // Work units.  The tiles of the last, incomplete round of the persistent schedule are cut into two halves of
-    // 128 columns when that lets them all run at once: the round then takes half as long, which matters when a
-    // pair only gets five or six tiles in all.  (Not for the gated form: a CTA's half would be 32 + 32 columns.)
+    // 128 columns (gated: 64 outputs) when that lets them all run at once: the round then takes half as long, which matters
+    // when a pair only gets five or six tiles in all.
     const int rem = num_tiles % num_pairs;
-    const bool split = !GATED && rem > 0 && 2 * rem <= num_pairs;
+    const bool split = rem > 0 && 2 * rem <= num_pairs;
     const int n_whole = split ? num_tiles - rem : num_tiles;
     const int num_units = n_whole + (split ? 2 * rem : 0);
     // Tiles go down the columns of bands of band_rows row tiles (band_rows_of() has the rule).
@@ -104,7 +104,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         Unit x;
         int tile = u, col0 = 0;
         x.width = BNO;
-        if (u >= n_whole) { const int v = u - n_whole; tile = n_whole + (v >> 1); col0 = (v & 1) * (kBN / 2); x.width = kBN / 2; }
+        if (u >= n_whole) { const int v = u - n_whole; tile = n_whole + (v >> 1); col0 = (v & 1) * (BNO / 2); x.width = BNO / 2; }
         const int row0 = tile / (band_rows * tiles_n) * band_rows, in_band = tile - row0 * tiles_n;
         const int rows = min(band_rows, tiles_m - row0);
         const int col = in_band / rows;
@@ -143,9 +143,11 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             for (int u = pair; u < num_units && !failed; u += num_pairs) {
                 const Unit un = unit_of(u);
                 const int m0 = un.m0 + (int)rank * kBM;
-                // this CTA's columns of W: half of the unit's (gated: 64 gate columns and the same 64 up columns)
-                const int n0 = un.n0 + (int)rank * (un.width / 2);
-                const bool narrow = un.width < BNO;  // a half tile: 64 columns of W per CTA
+                // This CTA's columns of W: half of the unit's (gated: 64 gate columns and the same 64 up columns).  A half tile has
+                // 64 columns of W per CTA; gated: the even CTA has the 64 gate columns, the odd one the 64 up columns, so the
+                // accumulator is [gate | up] once.
+                const bool narrow = un.width < BNO;
+                const int n0 = un.n0 + (GATED && narrow ? 0 : (int)rank * (un.width / 2));
                 for (int kb = 0; kb < kblocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1)) { failed = true; break; }
                     uint8_t* sa = smem + stage * L::kStageBytes;
@@ -156,16 +158,18 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                     tma_load_2d_pair(sa, &tmap_x, bar, kb * kBK, m0);
                     if constexpr (W_NK) {  // rows of W, 64 K-elements (one swizzle span) each
                         if constexpr (GATED) {
-                            tma_load_2d_pair(sb, &tmap_w, bar, kb * kBK, n0);               // 64 gate rows
-                            tma_load_2d_pair(sb + 64 * 128, &tmap_w2, bar, kb * kBK, n0);   // 64 up rows
+                            if (!narrow || rank == 0) tma_load_2d_pair(sb, &tmap_w, bar, kb * kBK, n0);  // 64 gate rows
+                            if (!narrow || rank != 0)                                                    // 64 up rows
+                                tma_load_2d_pair(sb + (narrow ? 0 : 64 * 128), &tmap_w2, bar, kb * kBK, n0);
                         } else {                                                             // one or two boxes of 64 rows
                             tma_load_2d_pair(sb, &tmap_w, bar, kb * kBK, n0);
                             if (!narrow) tma_load_2d_pair(sb + 64 * 128, &tmap_w, bar, kb * kBK, n0 + 64);
                         }
                     } else {               // boxes of 64 K-rows x 64 columns
-                        tma_load_2d_pair(sb, &tmap_w, bar, n0, kb * kBK);
-                        if constexpr (GATED) tma_load_2d_pair(sb + kBK * 128, &tmap_w2, bar, n0, kb * kBK);
-                        else if (!narrow) tma_load_2d_pair(sb + kBK * 128, &tmap_w, bar, n0 + 64, kb * kBK);
+                        if (!GATED || !narrow || rank == 0) tma_load_2d_pair(sb, &tmap_w, bar, n0, kb * kBK);
+                        if constexpr (GATED) {
+                            if (!narrow || rank != 0) tma_load_2d_pair(sb + (narrow ? 0 : kBK * 128), &tmap_w2, bar, n0, kb * kBK);
+                        } else if (!narrow) tma_load_2d_pair(sb + kBK * 128, &tmap_w, bar, n0 + 64, kb * kBK);
                     }
                     if (++stage == kStages) { stage = 0; phase ^= 1; }
                 }
@@ -182,7 +186,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             uint32_t phase = 0;
             int it = 0;
             for (int u = pair; u < num_units && !failed; u += num_pairs, ++it) {
-                const uint32_t idesc = (!GATED && unit_of(u).width < kBN) ? idesc_half : idesc_whole;
+                const uint32_t idesc = unit_of(u).width < BNO ? idesc_half : idesc_whole;
                 const int acc = it & 1;
                 const uint32_t acc_phase = (it >> 1) & 1;
                 if (!mbar_wait_cluster(&tmem_empty[acc], acc_phase ^ 1)) { failed = true; break; }
@@ -225,7 +229,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             tc_fence_after_sync();
             const int row = quarter * 32 + lane;  // row of this CTA's half of the tile = TMEM lane
             const uint32_t taddr = tmem_base + acc * kBN + (static_cast<uint32_t>(quarter * 32) << 16);
-            if (!GATED && blk * 64 >= un.width) {  // a half tile has no block for this warp: only the accumulator hand-back
+            if (blk * (BNO / 4) >= un.width) {  // a half tile has no block for this warp: only the accumulator hand-back
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(empty_on_leader + acc * 8);
