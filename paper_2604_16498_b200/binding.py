@@ -79,6 +79,12 @@ SIGNATURES.update({
 })
 
 _lib = None
+# host_calls.cpp: the frequent calls' marshalling in native code.  Its functions return -1 where a call is not plain (anything but
+# dense, contiguous CUDA tensors of matching shapes with the output given); then the Python below does it, with every check.
+_host_calls = None
+_HOST_CALLS_ENTRIES = ("forge_attn_fused", "forge_attn_fused_f16", "forge_attn_fused_f32", "forge_attn_decode_splitkv",
+                       "forge_attn_decode_splitkv_f16", "forge_linear_act", "forge_linear_act_f16", "forge_linear_act_w8a16",
+                       "forge_linear_swiglu")
 
 
 class ForgeError(RuntimeError):
@@ -103,7 +109,18 @@ def load() -> ctypes.CDLL:
             fn.restype = res
             fn.argtypes = args
         _lib = lib
+        _bind_host_calls(lib)
     return _lib
+
+
+def _bind_host_calls(lib) -> None:
+    global _host_calls
+    try:
+        from . import host_calls
+    except ImportError:  # built for another torch or Python: the general way
+        return
+    host_calls.bind(*(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _HOST_CALLS_ENTRIES))
+    _host_calls = host_calls
 
 
 def _find_raw_stream():
@@ -153,6 +170,11 @@ def _attn_dims(q, k, v):
 
 def attn_fused(q, k, v, mask_kind=MASK_NONE, lens=None, scale=None, out=None):
     """forge_attn_fused: bf16 tensors q [B,Hq,Sq,D], k/v [B,Hkv,Skv,D] on the GPU."""
+    if _host_calls is not None:
+        st = _host_calls.attn(0, q, k, v, mask_kind, lens, scale, out)
+        if st >= 0:
+            _check("forge_attn_fused", st)
+            return out
     B, Hq, Hkv, Sq, Skv, D = _attn_dims(q, k, v)
     out = torch.empty_like(q) if out is None else out
     scale = D ** -0.5 if scale is None else scale
@@ -185,6 +207,11 @@ def attn_fused_strided(q, k, v, out, mask_kind=MASK_NONE, lens=None, scale=None)
 
 def attn_fused_f16(q, k, v, mask_kind=MASK_NONE, lens=None, scale=None, out=None):
     """forge_attn_fused_f16: the same operator on fp16 tensors."""
+    if _host_calls is not None:
+        st = _host_calls.attn(1, q, k, v, mask_kind, lens, scale, out)
+        if st >= 0:
+            _check("forge_attn_fused_f16", st)
+            return out
     B, Hq, Hkv, Sq, Skv, D = _attn_dims(q, k, v)
     out = torch.empty_like(q) if out is None else out
     scale = D ** -0.5 if scale is None else scale
@@ -212,6 +239,11 @@ def attn_fused_bias(q, k, v, bias, mask_kind=MASK_NONE, lens=None, scale=None, o
 
 def attn_fused_f32(q, k, v, mask_kind=MASK_NONE, lens=None, scale=None, out=None):
     """forge_attn_fused_f32: the same operator on fp32 tensors."""
+    if _host_calls is not None:
+        st = _host_calls.attn(2, q, k, v, mask_kind, lens, scale, out)
+        if st >= 0:
+            _check("forge_attn_fused_f32", st)
+            return out
     B, Hq, Hkv, Sq, Skv, D = _attn_dims(q, k, v)
     out = torch.empty_like(q) if out is None else out
     scale = D ** -0.5 if scale is None else scale
@@ -236,6 +268,12 @@ def attn_decode_splitkv(q, k_cache, v_cache, lens, num_splits, scale=None, out=N
     """forge_attn_decode_splitkv (bf16 tensors) or forge_attn_decode_splitkv_f16 (fp16 tensors), chosen by
     q.dtype: q [B,Hq,D], caches [B,Hkv,Smax,D], lens int32 [B].  A workspace passed in must have been
     cleared once (attn_decode_workspace_init); without one, a fresh cleared workspace is allocated."""
+    if _host_calls is not None:
+        f16 = q.dtype == torch.float16
+        st = _host_calls.decode(1 if f16 else 0, q, k_cache, v_cache, lens, num_splits, scale, out, workspace)
+        if st >= 0:
+            _check("forge_attn_decode_splitkv_f16" if f16 else "forge_attn_decode_splitkv", st)
+            return out
     B, Hq, D = q.shape
     Bk, Hkv, Smax, Dk = k_cache.shape
     if (Bk, Dk) != (B, D) or tuple(v_cache.shape) != tuple(k_cache.shape):
@@ -296,6 +334,12 @@ W_KN, W_NK = 0, 1
 def linear_act(x, w, b=None, residual=None, act=ACT_GELU_TANH, w_layout=W_KN, out=None):
     """forge_linear_act (bf16 tensors) or forge_linear_act_f16 (fp16 tensors), chosen by x.dtype:
     act(x @ W + b) + residual with W given as [K,N] (W_KN) or [N,K] (W_NK)."""
+    if _host_calls is not None:
+        f16 = x.dtype == torch.float16
+        st = _host_calls.linear(1 if f16 else 0, x, w, b, residual, act, w_layout, out)
+        if st >= 0:
+            _check("forge_linear_act_f16" if f16 else "forge_linear_act", st)
+            return out
     M, K = x.shape
     N = w.shape[1] if w_layout == W_KN else w.shape[0]
     if tuple(w.shape) != ((K, N) if w_layout == W_KN else (N, K)):
@@ -316,6 +360,11 @@ def linear_act(x, w, b=None, residual=None, act=ACT_GELU_TANH, w_layout=W_KN, ou
 
 def linear_act_w8a16(x, w_int8, scale, b=None, residual=None, act=ACT_GELU_TANH, out=None):
     """forge_linear_act_w8a16: fp16 x [M,K], int8 weights [N,K], fp32 per-channel scale [N]."""
+    if _host_calls is not None:
+        st = _host_calls.linear_w8(x, w_int8, scale, b, residual, act, out)
+        if st >= 0:
+            _check("forge_linear_act_w8a16", st)
+            return out
     M, K = x.shape
     N = w_int8.shape[0]
     if tuple(w_int8.shape) != (N, K) or tuple(scale.shape) != (N,):
@@ -331,6 +380,11 @@ def linear_act_w8a16(x, w_int8, scale, b=None, residual=None, act=ACT_GELU_TANH,
 
 def linear_swiglu(x, w_gate, w_up, w_layout=W_KN, out=None):
     """forge_linear_swiglu: silu(x @ Wg) * (x @ Wu); both weights [K,N] (W_KN) or [N,K] (W_NK)."""
+    if _host_calls is not None:
+        st = _host_calls.swiglu(x, w_gate, w_up, w_layout, out)
+        if st >= 0:
+            _check("forge_linear_swiglu", st)
+            return out
     M, K = x.shape
     N = w_gate.shape[1] if w_layout == W_KN else w_gate.shape[0]
     want = (K, N) if w_layout == W_KN else (N, K)

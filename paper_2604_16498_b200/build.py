@@ -1,7 +1,8 @@
-"""Builds the CUDA library in-tree: ``paper_2604_16498_b200/libforge.so`` (sm_100a only).
+"""Builds the CUDA library in-tree: ``paper_2604_16498_b200/libforge.so`` (sm_100a only), and the native half of
+the Python binding, ``host_calls.so``.
 
 ``python -m paper_2604_16498_b200.build`` or ``build()`` from Python.  nvcc cross-compiles
-without a GPU.  The library is rebuilt when any source or header is newer than it.
+without a GPU.  Both are rebuilt when any source or header is newer than one of them.
 """
 from __future__ import annotations
 
@@ -9,12 +10,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libforge.so")
+HOST_CALLS = os.path.join(HERE, "host_calls.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 
 NVCC_FLAGS = [
@@ -29,11 +32,27 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(HOST_CALLS)):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(HOST_CALLS))
     deps = glob.glob(os.path.join(CSRC, "*")) + glob.glob(os.path.join(INCLUDE, "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _build_host_calls() -> None:
+    import torch
+    t = os.path.dirname(torch.__file__)
+    tmp = HOST_CALLS + f".tmp{os.getpid()}"
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) or "/usr/local/cuda"
+    inc = [os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
+    r = subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+                        f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", *(f"-I{i}" for i in inc),
+                        os.path.join(CSRC, "host_calls.cpp"), "-o", tmp, "-L" + os.path.join(t, "lib"),
+                        "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"], capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for host_calls.cpp:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, HOST_CALLS)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -53,8 +72,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if verbose:
             sys.stderr.write(r.stderr)
 
-    with ThreadPoolExecutor(max_workers=min(8, len(sources))) as pool:
+    with ThreadPoolExecutor(max_workers=min(8, len(sources)) + 1) as pool:
+        host = pool.submit(_build_host_calls)
         list(pool.map(compile_one, zip(sources, objs)))
+        host.result()
     tmp = LIB + f".tmp{os.getpid()}"
     r = subprocess.run([_nvcc(), "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"],
                        capture_output=True, text=True)
