@@ -58,6 +58,10 @@ constexpr int kBlockKeys = 16;             // cached rows per ring stage
 // saturated either way, and what is queued beyond that only adds to the latency of every block, which is what
 // the end of the call (the last blocks of the slowest warps) waits for.
 constexpr int kWarpRingBytes = 16 * 1024;
+#ifndef ASK
+#define ASK 2
+#endif
+constexpr int kAskBlocks = ASK;
 constexpr int kSingleLevelPieces = 32;     // up to this many pieces of a sequence are merged by one warp in one go
                                            // (one (m, l) pair per lane and head)
 constexpr int kMergeGroup = 16;            // beyond that: groups of sixteen, then the (at most sixteen) groups' results
@@ -142,7 +146,8 @@ struct Schedule {
     bool grouped;        // consecutive pieces of a (batch, kv head) go to the warps of a CTA
     int len0, P0, incl0; // of sequence `lane`: clamped length, pieces, pieces of sequences 0..lane
 };
-__device__ __forceinline__ int clamped_len(const int32_t* lens, int b, int Smax) { return min(max(lens[b], 0), Smax); }
+// (read past the L1: it is read before and after the previous kernel's end)
+__device__ __forceinline__ int clamped_len(const int32_t* lens, int b, int Smax) { return min(max(__ldcg(lens + b), 0), Smax); }
 __device__ __forceinline__ int blocks_of_len(int len) { return (len + kBlockKeys - 1) / kBlockKeys; }
 // pieces of a sequence of nb blocks: at least one, so that a sequence without rows still gets its zeros
 __device__ __forceinline__ int pieces_of(int nb, int C) { return max((nb + C - 1) / C, 1); }
@@ -513,14 +518,31 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
         ptx::prefetch_tmap(&tmap_v);
     }
     __syncwarp();
-    // Set-up done: the next kernel in the stream may move in as SMs free up.  Nothing global is touched
-    // before the previous kernel has completed and its writes are visible.
+    // Set-up done: the next kernel in the stream may move in as SMs free up.
     pdl_launch_dependents();
-    pdl_wait();
-
     const int workers = gridDim.x * kWarps;
     const int worker = warp * gridDim.x + blockIdx.x;
-    const Schedule sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
+    // Before the previous kernel has completed, its writes are not all visible: the schedule of the lengths as they are now serves
+    // to ask this worker's first blocks into L2, while SMs fall idle one by one at the end of that kernel (addresses only,
+    // within the cache whatever lens holds).  It is kept if the lengths turn out to be the same afterwards.
+    Schedule sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
+    {
+        const unsigned idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
+        if (idx < sched.num_items) {
+            const Item it = make_item<MODE>(idx, sched, lens, B, Hkv, Smax, lane);
+            const int row = it.s0 + lane * kBlockKeys;
+            if (lane < kAskBlocks && row < it.s1) {
+#pragma unroll
+                for (int cb = 0; cb < D / 64; ++cb) {
+                    ptx::tma_prefetch_l2_3d(&tmap_k, cb * 64, row, it.b * Hkv + it.kvh);
+                    ptx::tma_prefetch_l2_3d(&tmap_v, cb * 64, row, it.b * Hkv + it.kvh);
+                }
+            }
+        }
+    }
+    pdl_wait();
+    if (B > 32 || !__all_sync(0xffffffffu, sched.len0 == (lane < B ? clamped_len(lens, lane, Smax) : 0)))
+        sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
     const unsigned num_items = sched.num_items;
     const unsigned first_idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
     auto item_of_round = [&](int r) { return (unsigned)r * (unsigned)workers + first_idx; };
