@@ -2,8 +2,8 @@
 // tensors are checked and their addresses, the sizes and the current stream are passed to the C ABI.  The Python code
 // around ctypes takes 4 us a call, as long as the kernel of a small problem; this takes a few tenths.
 //
-// A call is made here only when everything about it is plain: torch.Tensor or Parameter itself, dense CUDA tensors without any
-// other dispatch key (no wrapper of a transform or mode), contiguous, of the expected type and shape, the output given, int and
+// A call is made here only when everything about it is plain: torch.Tensor or Parameter itself, dense CUDA tensors without the
+// dispatch key of a wrapper, transform or mode, contiguous, of the expected type and shape, the output given, int and
 // float options.  For anything else a function returns -1 without having done anything, and binding.py goes its general way, which
 // has the checks and raises the errors.  Otherwise the return value is the forge_status of the call.
 #include <torch/csrc/autograd/python_variable.h>
@@ -35,7 +35,7 @@ const at::Tensor* plain(PyObject* o, at::ScalarType type, int dims) {
     if (!THPVariable_CheckExact(o)) return nullptr;
     const at::Tensor& t = THPVariable_Unpack(o);
     static const uint64_t dense = c10::DispatchKeySet({c10::DispatchKey::CUDA, c10::DispatchKey::AutogradCUDA,
-                                                       c10::DispatchKey::ADInplaceOrView}).raw_repr();
+                                                       c10::DispatchKey::ADInplaceOrView, c10::DispatchKey::AutocastCUDA}).raw_repr();
     if (!t.defined() || (t.key_set().raw_repr() & ~dense) != 0 || !t.is_cuda() || t.scalar_type() != type || t.dim() != dims ||
         !t.is_contiguous())
         return nullptr;

@@ -62,7 +62,7 @@ struct W8Params {
     int M, N, K;
     int act;
     int nt, tiles_t;     // tokens per tile, token tiles
-    int split_log2;      // CTAs (pairs of CTAs) per tile
+    int split_log2;      // CTAs per tile
     int own4;            // 4-token pieces a CTA of a cluster finishes
     int stages;          // at least as many as converter groups
     int recv_off, out_off, bar_off;  // byte offsets in shared memory
@@ -74,7 +74,7 @@ __device__ __forceinline__ uint32_t widen2(uint32_t bits, __half2 off) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <int kGroups, bool PAIR>
+template <int kGroups>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_w8_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, const W8Params p) {
     constexpr int kEpiQuads = kWarpQuads - kGroups, kEpiWarps = 4 * kEpiQuads;
@@ -91,51 +91,36 @@ linear_w8_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int S = 1 << p.split_log2;
-    // PAIR: the CTA's place in its cluster is 2 * rank + half; half 0 issues the pair's MMAs
-    const int cluster_log2 = p.split_log2 + (PAIR ? 1 : 0), place = (int)blockIdx.x & ((1 << cluster_log2) - 1);
-    const int half = PAIR ? place & 1 : 0, rank = PAIR ? place >> 1 : place;
-    const int first_tile = (int)blockIdx.x >> cluster_log2, tile_step = (int)gridDim.x >> cluster_log2;
-    constexpr int kTileF = PAIR ? 2 * kBF : kBF;
-    const int num_tiles = p.tiles_t * ((p.N + kTileF - 1) / kTileF);
+    const int rank = (int)blockIdx.x & (S - 1);
+    const int first_tile = (int)blockIdx.x >> p.split_log2, tile_step = (int)gridDim.x >> p.split_log2;
+    const int num_tiles = p.tiles_t * ((p.N + kBF - 1) / kBF);
     const int kblocks = (p.K + kBK - 1) / kBK;
     const int kb0 = (int)((long long)kblocks * rank >> p.split_log2);
     const int nkb = (int)((long long)kblocks * (rank + 1) >> p.split_log2) - kb0;
     constexpr int kRawBytes = kBF * kBK;
-    const int xrows = PAIR ? p.nt / 2 : p.nt;                // tokens whose X this CTA copies
-    const int stage_bytes = kRawBytes + xrows * (kBK * 2);  // int8 rows, then X
+    const int stage_bytes = kRawBytes + p.nt * (kBK * 2);  // int8 rows, then X
     // tiles of the same features follow one another: their weights are still in L2
-    auto feature0 = [&](int tile) { return tile / p.tiles_t * kTileF + half * kBF; };
+    auto feature0 = [&](int tile) { return tile / p.tiles_t * kBF; };
     auto token0 = [&](int tile) { return tile % p.tiles_t * p.nt; };
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < p.stages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-        for (int i = 0; i < kGroups; ++i) { mbar_init(&conv_full[i], PAIR ? 8 : 4); mbar_init(&conv_empty[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&tmem_full[i], 1); mbar_init(&tmem_empty[i], PAIR ? 2 * kEpiWarps : kEpiWarps); }
+        for (int i = 0; i < kGroups; ++i) { mbar_init(&conv_full[i], 4); mbar_init(&conv_empty[i], 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&tmem_full[i], 1); mbar_init(&tmem_empty[i], kEpiWarps); }
         fence_mbar_init();
         prefetch_tmap(&tmap_w);
         prefetch_tmap(&tmap_x);
     }
     if (warp == 1) {
-        if constexpr (PAIR) {
-            tmem_alloc_pair(tmem_base_slot, kTmemCols);
-            tmem_relinquish_pair();
-        } else {
-            tmem_alloc(tmem_base_slot, kTmemCols);
-            tmem_relinquish();
-        }
+        tmem_alloc(tmem_base_slot, kTmemCols);
+        tmem_relinquish();
     }
     tc_fence_before_sync();
     __syncthreads();
-    if constexpr (PAIR) cluster_sync();  // both CTAs' barriers exist before anyone signals across
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_base_slot;
     bool failed = false;
-    if (!PAIR && S > 1) cluster_arrive();  // this CTA runs: its shared memory may be written (awaited before the exchange)
-    // An arrival on a barrier of the CTA that issues the MMAs (this one, or the even one of the pair).
-    auto arrive_issuer = [&](uint64_t* bar) {
-        if constexpr (PAIR) mbar_arrive_cluster(map_to_cta(bar, place & ~1));
-        else mbar_arrive(bar);
-    };
+    if (S > 1) cluster_arrive();  // this CTA runs: its shared memory may be written (awaited before the exchange)
     pdl_launch_dependents();
     pdl_wait();
 
@@ -151,7 +136,7 @@ linear_w8_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
                     uint8_t* raw = smem + stage * stage_bytes;
                     mbar_expect_tx(&full[stage], stage_bytes);
                     tma_load_2d(raw, &tmap_w, &full[stage], kb * kBK, f0);
-                    tma_load_2d(raw + kRawBytes, &tmap_x, &full[stage], kb * kBK, t0 + half * xrows);
+                    tma_load_2d(raw + kRawBytes, &tmap_x, &full[stage], kb * kBK, t0);
                     if (++stage == p.stages) { stage = 0; phase ^= 1; }
                 }
             }
@@ -159,39 +144,31 @@ linear_w8_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (half == 0 && elect_one()) {
-            const uint32_t idesc = make_idesc_f16(kTileF, p.nt, /*a_mn_major=*/false, /*b_mn_major=*/false);
-            const uint16_t both = (uint16_t)(3u << place);  // PAIR: this CTA and its neighbour
-            auto wait = [&](uint64_t* bar, uint32_t parity) { return PAIR ? mbar_wait_cluster(bar, parity) : mbar_wait(bar, parity); };
-            auto commit = [&](uint64_t* bar) {
-                if constexpr (PAIR) mma_commit_pair(bar, both);
-                else mma_commit(bar);
-            };
+        if (elect_one()) {
+            const uint32_t idesc = make_idesc_f16(kBF, p.nt, /*a_mn_major=*/false, /*b_mn_major=*/false);
             int stage = 0, grp = 0, it = 0;
             uint32_t gphase = 0;
             for (int tile = first_tile; tile < num_tiles && !failed; tile += tile_step, ++it) {
                 const int acc = it & 1;
-                if (!wait(&tmem_empty[acc], ((it >> 1) & 1) ^ 1)) { failed = true; break; }
+                if (!mbar_wait(&tmem_empty[acc], ((it >> 1) & 1) ^ 1)) { failed = true; break; }
                 tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + acc * kMaxTokens;
                 for (int kb = 0; kb < nkb; ++kb) {
-                    // the converters (of both CTAs) have seen their stage's barrier complete: X has landed too
-                    if (!wait(&conv_full[grp], gphase)) { failed = true; break; }
+                    // the converters have seen the stage's barrier complete: X has landed too
+                    if (!mbar_wait(&conv_full[grp], gphase)) { failed = true; break; }
                     tc_fence_after_sync();
                     const uint32_t a_tmem = tmem_base + kColA + grp * (kBK / 2);
                     const uint64_t b_desc = make_smem_desc(smem_u32(smem + stage * stage_bytes + kRawBytes), 16, 1024);
 #pragma unroll
-                    for (int k = 0; k < kBK / 16; ++k) {
-                        if constexpr (PAIR) mma_ts_pair(d_tmem, a_tmem + k * 8, b_desc + k * (32 >> 4), idesc, (kb | k) != 0);
-                        else mma_ts(d_tmem, a_tmem + k * 8, b_desc + k * (32 >> 4), idesc, (kb | k) != 0);
-                    }
-                    commit(&conv_empty[grp]);
-                    commit(&empty[stage]);
+                    for (int k = 0; k < kBK / 16; ++k)
+                        mma_ts(d_tmem, a_tmem + k * 8, b_desc + k * (32 >> 4), idesc, (kb | k) != 0);
+                    mma_commit(&conv_empty[grp]);
+                    mma_commit(&empty[stage]);
                     if (++grp == kGroups) { grp = 0; gphase ^= 1; }
                     if (++stage == p.stages) stage = 0;
                 }
                 if (failed) break;
-                commit(&tmem_full[acc]);
+                mma_commit(&tmem_full[acc]);
             }
         }
         __syncwarp();
@@ -230,7 +207,7 @@ linear_w8_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
             tmem_st_wait();
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) arrive_issuer(&conv_full[group]);
+            if (lane == 0) mbar_arrive(&conv_full[group]);
             if ((stage += kGroups) >= p.stages) { stage -= p.stages; phase ^= 1; }
         }
         __syncwarp();
@@ -299,14 +276,14 @@ linear_w8_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
                 }
                 tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) arrive_issuer(&tmem_empty[acc]);
+                if (lane == 0) mbar_arrive(&tmem_empty[acc]);
             } else {
                 // one tile per cluster.  recv of an owner: [source slot][4-token piece][feature] of 16 bytes
                 uint8_t* recv = smem + p.recv_off;
                 const uint32_t recv0 = smem_u32(recv);
                 const int pieces = (ntok + 3) >> 2;
                 const int own_begin = rank * p.own4, own_end = min(own_begin + p.own4, pieces);
-                if (!PAIR) cluster_wait();  // every CTA of the cluster runs
+                cluster_wait();  // every CTA of the cluster runs
 #pragma unroll 1
                 for (int c = share * 4; c < pieces; c += kEpiQuads * 4) {
                     uint32_t r[16];
@@ -318,7 +295,7 @@ linear_w8_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
                         if (owner == rank || piece >= pieces) continue;
                         const int slot = rank - (rank > owner ? 1 : 0);
                         const uint32_t at = (uint32_t)((slot * p.own4 + piece - owner * p.own4) * kBF + frow) * 16;
-                        st_cluster_v4(map_addr_to_cta(recv0 + at, PAIR ? 2 * owner + half : owner), r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+                        st_cluster_v4(map_addr_to_cta(recv0 + at, owner), r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
                     }
                 }
                 cluster_arrive();
@@ -344,16 +321,12 @@ linear_w8_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
                 }
             }
         }
-        if (S > 1 && failed) {  // the one tile's barriers were not reached
-            if (!PAIR) cluster_wait();
-            cluster_arrive();
-            cluster_wait();
-        }
+        if (S > 1 && failed) { cluster_wait(); cluster_arrive(); cluster_wait(); }  // the one tile's barriers were not reached
         __syncwarp();
     }
     // every thread of the cluster takes part in both phases of the cluster barrier
     if (S > 1 && !(warp >= 2 && warp < 2 + kEpiWarps)) {
-        if (!PAIR) cluster_wait();
+        cluster_wait();
         cluster_arrive();
         cluster_wait();
     }
@@ -364,20 +337,17 @@ linear_w8_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     }
     tc_fence_before_sync();
     __syncthreads();
-    if constexpr (PAIR) cluster_sync();  // neither CTA leaves while the other may signal its barriers
     if (warp == 1) {
         tc_fence_after_sync();
-        if constexpr (PAIR) tmem_dealloc_pair(tmem_base, kTmemCols);
-        else tmem_dealloc(tmem_base, kTmemCols);
+        tmem_dealloc(tmem_base, kTmemCols);
     }
 }
 
-template <int kGroups, bool PAIR>
-int launch_w8(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w, const W8Params& p, unsigned grid, int smem_bytes, int cluster,
+template <int kGroups>
+int launch_w8(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w, const W8Params& p, unsigned grid, int smem_bytes, int S,
               cudaStream_t s) {
-    const auto kernel = linear_w8_kernel<kGroups, PAIR>;
-    FORGE_SET_SMEM_ONCE(kernel, kSmemMax);
-    FORGE_CUDA_TRY(launch_pdl_cluster(kernel, dim3(grid), dim3(kThreads), smem_bytes, cluster, s, tmap_x, tmap_w, p));
+    FORGE_SET_SMEM_ONCE(linear_w8_kernel<kGroups>, kSmemMax);
+    FORGE_CUDA_TRY(launch_pdl_cluster(linear_w8_kernel<kGroups>, dim3(grid), dim3(kThreads), smem_bytes, S, s, tmap_x, tmap_w, p));
     return finish_launch(1);
 }
 
@@ -416,37 +386,12 @@ bool linear_w8_plan(int M, int N, int K, int sms, W8Plan* plan) {
     return pl.tiles <= 2147483647LL && pl.stages >= pl.groups;
 }
 
-bool linear_w8_pair_plan(int M, int N, int K, int sms, W8Plan* plan) {
-    W8Plan& pl = *plan;
-    const int kblocks = (K + kBK - 1) / kBK, pairs = sms / 2;
-    const long long tiles_f = (N + 2 * kBF - 1) / (2 * kBF);
-    pl.tiles_t = (M + kMaxTokens - 1) / kMaxTokens;
-    pl.nt = ((M + pl.tiles_t - 1) / pl.tiles_t + 31) / 32 * 32;
-    if (pl.tiles_t * tiles_f > pairs) {  // several rounds: the smallest tiles that need no more of them
-        const long long rounds = (pl.tiles_t * tiles_f + pairs - 1) / pairs, most = rounds * pairs / tiles_f;
-        pl.nt = (int)((M + most - 1) / most + 31) / 32 * 32;
-        pl.tiles_t = (M + pl.nt - 1) / pl.nt;
-    }
-    pl.tiles = pl.tiles_t * tiles_f;
-    pl.groups = pl.tiles > pairs && kblocks >= 48 ? 4 : 3;
-    pl.split = 1;
-    while (pl.split < 4 && pl.tiles * pl.split * 2 <= pairs * 8 / 9 && kblocks >= pl.split * 2 * 2) pl.split *= 2;
-    const int stage_bytes = kBF * kBK + pl.nt / 2 * kBK * 2;  // at most 20 KB
-    pl.own4 = pl.split > 1 ? (pl.nt / 4 + pl.split - 1) / pl.split : 0;
-    pl.recv_bytes = (pl.split - 1) * pl.own4 * kBF * 16;  // at most 72 KB (192 tokens, S = 4)
-    pl.stages = (kSmemMax - pl.recv_bytes - kOutBytes - kBarBytes - 1024) / stage_bytes;  // at least six
-    if (pl.stages > kMaxStages) pl.stages = kMaxStages;
-    return pl.tiles <= 1073741823LL;
-}
-
 int linear_w8(const void* x, const void* w_int8, const float* scale, const void* b, const void* residual, void* y, int M,
               int N, int K, int act, cudaStream_t s) {
     const int sms = sm_count();
     if (sms <= 0) return FORGE_ERR_CUDA;
     W8Plan pl;
-    const bool pair = M > 64;
-    if (!(pair ? linear_w8_pair_plan(M, N, K, sms, &pl) : linear_w8_plan(M, N, K, sms, &pl))) return FORGE_ERR_UNSUPPORTED;
-    const int xrows = pair ? pl.nt / 2 : pl.nt;
+    if (!linear_w8_plan(M, N, K, sms, &pl)) return FORGE_ERR_UNSUPPORTED;
     W8Params p;
     p.bias = static_cast<const uint16_t*>(b);
     p.residual = static_cast<const uint16_t*>(residual);
@@ -459,7 +404,7 @@ int linear_w8(const void* x, const void* w_int8, const float* scale, const void*
     p.split_log2 = __builtin_ctz(pl.split);
     p.own4 = pl.own4;
     p.stages = pl.stages;
-    p.recv_off = pl.stages * (kBF * kBK + xrows * kBK * 2);
+    p.recv_off = pl.stages * (kBF * kBK + pl.nt * kBK * 2);
     p.out_off = p.recv_off + pl.recv_bytes;
     p.bar_off = p.out_off + kOutBytes;
     const int total = p.bar_off + kBarBytes + 1024;
@@ -469,7 +414,7 @@ int linear_w8(const void* x, const void* w_int8, const float* scale, const void*
     {
         const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M};
         const uint64_t strides[1] = {(uint64_t)K * 2};
-        const uint32_t box[2] = {kBK, (uint32_t)xrows};
+        const uint32_t box[2] = {kBK, (uint32_t)p.nt};
         if (!encode_tmap_bf16_sw128(&tmap_x, x, 2, dims, strides, box)) return FORGE_ERR_CUDA;
     }
     {
@@ -478,11 +423,9 @@ int linear_w8(const void* x, const void* w_int8, const float* scale, const void*
         const uint32_t box[2] = {kBK, kBF};
         if (!encode_tmap_u8_sw64(&tmap_w, w_int8, 2, dims, strides, box)) return FORGE_ERR_CUDA;
     }
-    const int width = pair ? 2 : 1, most = sms / width;  // CTAs per tile and share of K; tiles at once
-    const unsigned grid = (unsigned)(width * (pl.split > 1 ? pl.tiles * pl.split : (pl.tiles < most ? pl.tiles : most)));
-    const auto launch = pair ? (pl.groups == 4 ? launch_w8<4, true> : launch_w8<3, true>)
-                             : (pl.groups == 4 ? launch_w8<4, false> : launch_w8<3, false>);
-    return launch(tmap_x, tmap_w, p, grid, total, width * pl.split, s);
+    const long long grid = pl.split > 1 ? pl.tiles * pl.split : (pl.tiles < sms ? pl.tiles : sms);
+    return pl.groups == 4 ? launch_w8<4>(tmap_x, tmap_w, p, (unsigned)grid, total, pl.split, s)
+                          : launch_w8<3>(tmap_x, tmap_w, p, (unsigned)grid, total, pl.split, s);
 }
 
 }  // namespace forge

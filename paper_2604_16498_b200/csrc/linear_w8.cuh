@@ -17,8 +17,6 @@ struct W8Plan {
 
 // The plan for an M x N output on a GPU with `sms` SMs; false for a size that has none (2^31 tiles or more).
 bool linear_w8_plan(int M, int N, int K, int sms, W8Plan* plan);
-// The same for pairs of CTAs (256 features per tile; tokens a multiple of 32; split: pairs per tile, 1, 2 or 4).
-bool linear_w8_pair_plan(int M, int N, int K, int sms, W8Plan* plan);
 
 // act((X Wq^T) * scale + b) + residual; arguments as forge_linear_act_w8a16.
 int linear_w8(const void* x, const void* w_int8, const float* scale, const void* b, const void* residual, void* y, int M,
