@@ -643,8 +643,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 }
                 tmem_ld_wait();
 
-                const bool need_mask = (key0 + kHalf > kvlen) || (causal && (key0 + kHalf - 1 > q0 + causal_off)) ||
-                                       BIAS;  // a bias may hold -inf: the path that tolerates it
+                const bool need_mask = (key0 + kHalf > kvlen) || (causal && (key0 + kHalf - 1 > q0 + causal_off));
                 if constexpr (BIAS) {
                     // Eq. 8's mask node as a tensor: scale * s + bias = scale * (s + bias / scale)
                     if ((p.Skv & 3) != 0) {
@@ -701,7 +700,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                             stored = true;
                         }
                     };
-                    if (need_mask) fast_path(std::false_type{});
+                    if (BIAS || need_mask) fast_path(std::false_type{});  // (a bias may hold -inf too)
                     else fast_path(std::true_type{});
                 }
                 if (!stored) {

@@ -58,10 +58,6 @@ constexpr int kBlockKeys = 16;             // cached rows per ring stage
 // saturated either way, and what is queued beyond that only adds to the latency of every block, which is what
 // the end of the call (the last blocks of the slowest warps) waits for.
 constexpr int kWarpRingBytes = 16 * 1024;
-#ifndef ASK
-#define ASK 2
-#endif
-constexpr int kAskBlocks = ASK;
 constexpr int kSingleLevelPieces = 32;     // up to this many pieces of a sequence are merged by one warp in one go
                                            // (one (m, l) pair per lane and head)
 constexpr int kMergeGroup = 16;            // beyond that: groups of sixteen, then the (at most sixteen) groups' results
@@ -522,31 +518,16 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
     pdl_launch_dependents();
     const int workers = gridDim.x * kWarps;
     const int worker = warp * gridDim.x + blockIdx.x;
-    // Before the previous kernel has completed, its writes are not all visible: the schedule of the lengths as they are now serves
-    // to ask this worker's first blocks into L2, while SMs fall idle one by one at the end of that kernel (addresses only,
-    // within the cache whatever lens holds).  It is kept if the lengths turn out to be the same afterwards.
+    // Before the previous kernel has completed, its writes are not all visible; nothing but lens is read.  The schedule of the lengths
+    // as they are now serves to ask this worker's first blocks into L2, while SMs fall idle one by one at the end of that
+    // kernel (addresses only, within the cache whatever lens holds), and to start the first copies right after it.  By the
+    // time these land it is known whether the lengths are still the same; if not, the copies are dropped and the schedule is
+    // made again.  (More than 32 sequences: the schedule reads lens several times and is made once, afterwards.)
+    const bool early = B <= 32;
+    if (!early) pdl_wait();
     Schedule sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
-    {
-        const unsigned idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
-        if (idx < sched.num_items) {
-            const Item it = make_item<MODE>(idx, sched, lens, B, Hkv, Smax, lane);
-            const int row = it.s0 + lane * kBlockKeys;
-            if (lane < kAskBlocks && row < it.s1) {
-#pragma unroll
-                for (int cb = 0; cb < D / 64; ++cb) {
-                    ptx::tma_prefetch_l2_3d(&tmap_k, cb * 64, row, it.b * Hkv + it.kvh);
-                    ptx::tma_prefetch_l2_3d(&tmap_v, cb * 64, row, it.b * Hkv + it.kvh);
-                }
-            }
-        }
-    }
-    pdl_wait();
-    if (B > 32 || !__all_sync(0xffffffffu, sched.len0 == (lane < B ? clamped_len(lens, lane, Smax) : 0)))
-        sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
-    const unsigned num_items = sched.num_items;
-    const unsigned first_idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
+    unsigned first_idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
     auto item_of_round = [&](int r) { return (unsigned)r * (unsigned)workers + first_idx; };
-    if (MODE == kGrouped && sched.grouped && lane == 0) merge_info[warp][0] = -1;
 
     // ---- prefetch cursor: runs kStages blocks ahead of the compute, across item boundaries (a stage is
     // refilled as soon as its fragments are in registers, before the MMAs on them)
@@ -555,7 +536,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
     int p_bk = 0;  // batch * Hkv + kv head of the cursor's item
     int p_n = 0;  // blocks issued
     auto p_open = [&]() {  // position the cursor on the first block of the next non-empty item
-        while (p_idx < num_items) {
+        while (p_idx < sched.num_items) {
             const Item it = make_item<MODE>(p_idx, sched, lens, B, Hkv, Smax, lane);
             if (it.s1 > it.s0) {
                 p_j0 = it.s0;
@@ -570,7 +551,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
     // partials, the queries and whatever the caller keeps in L2 out of it (2 us of 31 at B 16, lengths 1024..4096).
     const uint64_t stream_policy = ptx::l2_policy_evict_first();
     auto issue = [&]() {  // one lane starts the block's tile copies (rows past the cache's end are zero-filled)
-        if (p_idx < num_items) {
+        if (p_idx < sched.num_items) {
             if (lane == 0) {
                 const int st = p_n % kStages;
                 const uint32_t dst = ring + st * kStageBytes;
@@ -587,8 +568,33 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
         }
     };
     p_open();
+    if (early) {
+        const int row = p_j0 + lane * kBlockKeys;
+        if (p_idx < sched.num_items && lane < kStages && row < p_s1) {
+#pragma unroll
+            for (int cb = 0; cb < D / 64; ++cb) {
+                ptx::tma_prefetch_l2_3d(&tmap_k, cb * 64, row, p_bk);
+                ptx::tma_prefetch_l2_3d(&tmap_v, cb * 64, row, p_bk);
+            }
+        }
+        pdl_wait();
+    }
+    const int len_now = lane < B ? clamped_len(lens, lane, Smax) : 0;
 #pragma unroll
     for (int i = 0; i < kStages; ++i) issue();
+    bool failed = false;
+    int n = 0;  // blocks consumed
+    if (early && !__all_sync(0xffffffffu, sched.len0 == len_now)) {
+        for (; n < p_n && !failed; ++n) failed = !ptx::warp_wait(&full[n % kStages], (n / kStages) & 1);
+        sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
+        first_idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
+        p_round = 0;
+        p_idx = item_of_round(0);
+        p_open();
+        for (int i = 0; i < kStages && !failed; ++i) issue();
+    }
+    const unsigned num_items = sched.num_items;
+    if (MODE == kGrouped && sched.grouped && lane == 0) merge_info[warp][0] = -1;
 
     // Q fragment of an item: head g (zero rows for g >= G), 8 dims at c*8 of every 32-dim block
     auto load_q = [&](const Item& it, uint32_t (&qr)[NKB][4]) {
@@ -607,9 +613,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
         nxt = make_item<MODE>(item_of_round(0), sched, lens, B, Hkv, Smax, lane);
         load_q(nxt, qn);
     }
-    int n = 0;  // blocks consumed
-    bool failed = false;
-    for (int round = 0; item_of_round(round) < num_items; ++round) {
+    for (int round = 0; !failed && item_of_round(round) < num_items; ++round) {
         const Item it = nxt;
         uint32_t qr[NKB][4];
 #pragma unroll

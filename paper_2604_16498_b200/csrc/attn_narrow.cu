@@ -2,19 +2,19 @@
 //
 // With 64 columns of output a 64-key step is 256 cycles of tensor core against 512 of the special-function unit's exponentials, and
 // the rest of a step (barriers, tensor-memory round trips, fences) is as long as both.  So the kernel is small and the SM
-// holds four of its CTAs: one query tile of 128 rows each, 160 threads, 48 KB of shared memory and 128 tensor-memory columns.
-// While one tile waits for its MMAs, its loads or its next item's start, the other three keep the special-function unit busy, and
-// the hardware scheduler hands out the tiles, longest first.  (Two tiles per SM in one persistent CTA, with two score buffers each:
-// about 950 cycles per tile and step.)
+// holds three of its CTAs: one query tile of 128 rows each, 160 threads, 65 KB of shared memory and 160 tensor-memory columns.
+// While one tile waits, the others keep the special-function unit busy, and the hardware scheduler hands out the tiles, longest
+// first.
 //
-//   tensor memory   S at column 0 (64 fp32 columns), O at 64; P (16-bit, two per column) overwrites the first 32 columns of S and
-//                   is the A operand of P V
-//   shared memory   Q 16 KB (the output is staged in its place), two stages of 64 keys for K and two for V, 8 KB each
+//   tensor memory   S at column 0 (64 fp32 columns), O at 64; P (16-bit, two per column) in 32 columns of an allocation of its own,
+//                   from where it is the A operand of P V
+//   shared memory   Q 16 KB (the output is staged in its place), three stages of 64 keys for K and three for V, 8 KB each
 //   warps 0-3       softmax, rescale and epilogue: thread = tile row = TMEM lane
-//   warp 4          one lane issues the copies and the MMAs; the warp owns the TMEM allocation
-// Per step g:  S(g) = Q K(g)^T complete -> softmax -> O += P(g) V(g), S(g + 1) = Q K(g + 1)^T.  MMAs of one thread execute in issue
-// order, so P(g) is read before S(g + 1) overwrites it, and S(g + 1)'s barrier also covers O.  S(g) complete means that K's
-// stage g % 2 and V's stage (g + 1) % 2 are free again: their next tiles are asked for then, most of a step before they are needed.
+//   warp 4          one lane issues the copies and the MMAs; the warp owns the TMEM allocations
+// Per step g: S(g) complete -> the softmax warps read it into registers -> S(g + 1) = Q K(g + 1)^T is issued into the same columns and
+// runs beside the exponentials of step g -> P(g) stored -> O += P(g) V(g).  P(g) may be stored once the product of step g - 1 has
+// read P(g - 1); with P over S instead, the next scores waited for this step's product, and four CTAs per SM took 870 cycles per
+// tile and step.
 // O is rescaled in tensor memory only when a row's maximum grows by more than 2^8 (the stale maximum is kept otherwise; the final
 // division by l uses the same reference).
 #include "attn_math.cuh"
@@ -23,6 +23,8 @@
 #include "forge_common.cuh"
 #include "sm100_ptx.cuh"
 #include "tmap.cuh"
+
+#include <type_traits>
 
 namespace forge {
 namespace {
@@ -33,18 +35,24 @@ constexpr int kD = 64;            // the kernel's head dimension
 constexpr int kBM = 128;          // rows of a tile
 constexpr int kStep = 64;         // keys per step and per K/V stage
 constexpr int kThreads = 160;
-constexpr int kCtasPerSm = 4;
-constexpr int kTmemCols = 128;
+constexpr int kCtasPerSm = 3;
+constexpr int kStages = 3;        // of K and of V
+constexpr int kTmemCols = 128;    // S and O
+constexpr int kTmemColsP = 32;
 constexpr int kColO = 64;
+#ifndef NFMA
+#define NFMA 8
+#endif
+constexpr int kFmaExpPairs = NFMA;
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
 
 struct NarrowSmem {
     static constexpr int kQBytes = kBM * 128;
     static constexpr int kKVBytes = kStep * 128;
     static constexpr int kKOff = kQBytes;
-    static constexpr int kVOff = kKOff + 2 * kKVBytes;
-    static constexpr int kBarOff = kVOff + 2 * kKVBytes;
-    static constexpr int kNumBars = 8;  // q_full, k_full[2], v_full[2], s_full, p_ready, o_staged
+    static constexpr int kVOff = kKOff + kStages * kKVBytes;
+    static constexpr int kBarOff = kVOff + kStages * kKVBytes;
+    static constexpr int kNumBars = 6 + 2 * kStages;  // q_full, k_full[3], v_full[3], s_full, s_read, p_ready, pv_done, o_staged
     static constexpr int kTotal = kBarOff + kNumBars * 8 + 16;
     static constexpr int kAlloc = kTotal + 1024;
 };
@@ -71,11 +79,13 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
     uint8_t* sK = smem + L::kKOff;
     uint8_t* sV = smem + L::kVOff;
     uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
-    uint64_t* k_full = q_full + 1;   // [2] by step parity
-    uint64_t* v_full = k_full + 2;   // [2]
-    uint64_t* s_full = v_full + 2;   // S(g) is complete, and so is every MMA before it; once more after the last product
-    uint64_t* p_ready = s_full + 1;
-    uint64_t* o_staged = p_ready + 1;  // all four warps' rows of the output lie in Q's place
+    uint64_t* k_full = q_full + 1;         // [3] step g uses stage g % 3
+    uint64_t* v_full = k_full + kStages;   // [3]
+    uint64_t* s_full = v_full + kStages;   // S(g) is complete
+    uint64_t* s_read = s_full + 1;         // S(g) is in the softmax threads' registers
+    uint64_t* p_ready = s_read + 1;
+    uint64_t* pv_done = p_ready + 1;       // O holds the product of step g
+    uint64_t* o_staged = pv_done + 1;      // all four warps' rows of the output lie in Q's place
     uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(o_staged + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -89,13 +99,14 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
 
     if (threadIdx.x == 0) {
         mbar_init(q_full, 1);
-        for (int i = 0; i < 2; ++i) { mbar_init(&k_full[i], 1); mbar_init(&v_full[i], 1); }
-        mbar_init(s_full, 1); mbar_init(p_ready, 4); mbar_init(o_staged, 4);
+        for (int i = 0; i < kStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&v_full[i], 1); }
+        mbar_init(s_full, 1); mbar_init(s_read, 4); mbar_init(p_ready, 4); mbar_init(pv_done, 1); mbar_init(o_staged, 4);
         fence_mbar_init();
         prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_o);
     }
     if (warp == 4) {
         tmem_alloc(tmem_base_slot, kTmemCols);
+        tmem_alloc(tmem_base_slot + 1, kTmemColsP);
         tmem_relinquish();
     }
     // Rows of the Q tile that are not in use are never written by the copy: zero scores, not whatever lies there.
@@ -107,7 +118,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_base_slot;
+    const uint32_t tmem_base = tmem_base_slot[0], tmem_p = tmem_base_slot[1];
     bool failed = false;
     pdl_launch_dependents();
     pdl_wait();
@@ -123,17 +134,16 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
             constexpr uint32_t idesc_s = F16 ? make_idesc_f16(kBM, kStep, false, false) : make_idesc_bf16(kBM, kStep, false, false);
             constexpr uint32_t idesc_o = F16 ? make_idesc_f16(kBM, kD, false, true) : make_idesc_bf16(kBM, kD, false, true);
             const uint64_t qd = make_smem_desc(smem_u32(sQ), 16, 1024);
-            auto load_k = [&](int g) {
-                mbar_expect_tx(&k_full[g & 1], L::kKVBytes);
-                tma_load_4d(sK + (g & 1) * L::kKVBytes, &tmap_k, &k_full[g & 1], 0, g * kStep, kvh, b);
+            auto load = [&](const CUtensorMap* map, uint8_t* ring, uint64_t* full, int g) {
+                if (g >= n) return;
+                const int st = g % kStages;
+                mbar_expect_tx(&full[st], L::kKVBytes);
+                tma_load_4d(ring + st * L::kKVBytes, map, &full[st], 0, g * kStep, kvh, b);
             };
-            auto load_v = [&](int g) {
-                mbar_expect_tx(&v_full[g & 1], L::kKVBytes);
-                tma_load_4d(sV + (g & 1) * L::kKVBytes, &tmap_v, &v_full[g & 1], 0, g * kStep, kvh, b);
-            };
+            auto landed = [&](uint64_t* full, int g) { return mbar_wait(&full[g % kStages], (g / kStages) & 1); };
             auto issue_qk = [&](int g) {
                 tc_fence_after_sync();
-                const uint64_t kd = make_smem_desc(smem_u32(sK) + (g & 1) * L::kKVBytes, 16, 1024);
+                const uint64_t kd = make_smem_desc(smem_u32(sK) + (g % kStages) * L::kKVBytes, 16, 1024);
 #pragma unroll
                 for (int kk = 0; kk < kD / 16; ++kk) mma_ss(tmem_base, qd + kk * (32 >> 4), kd + kk * (32 >> 4), idesc_s, kk != 0);
                 mma_commit(s_full);
@@ -141,27 +151,27 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
             // rows beyond Sq and columns beyond head_dim are zero-filled by the TMA unit
             mbar_expect_tx(q_full, (uint32_t)rows * 128);
             tma_load_4d(sQ, &tmap_q, q_full, 0, q0, head, b);
-            load_k(0);
-            load_v(0);
-            if (n > 1) load_k(1);
-            if (!mbar_wait(q_full, 0) || !mbar_wait(&k_full[0], 0)) failed = true;
+            for (int g = 0; g < kStages; ++g) {
+                load(&tmap_k, sK, k_full, g);
+                load(&tmap_v, sV, v_full, g);
+            }
+            if (!mbar_wait(q_full, 0) || !landed(k_full, 0)) failed = true;
             if (!failed) issue_qk(0);
             for (int g = 0; g < n && !failed; ++g) {
-                if (!mbar_wait(s_full, g & 1)) { failed = true; break; }
-                if (g + 2 < n) load_k(g + 2);
-                if (g + 1 < n) load_v(g + 1);
-                // the operands of the next MMAs, before the probabilities: then those go out back to back
-                if (!mbar_wait(&v_full[g & 1], (g >> 1) & 1)) { failed = true; break; }
-                if (g + 1 < n && !mbar_wait(&k_full[(g + 1) & 1], ((g + 1) >> 1) & 1)) { failed = true; break; }
-                if (!mbar_wait(p_ready, g & 1)) { failed = true; break; }
+                // operands before the softmax warps' arrivals: then the MMAs go out at once
+                if (g + 1 < n && !landed(k_full, g + 1)) { failed = true; break; }
+                if (!mbar_wait(s_read, g & 1)) { failed = true; break; }
+                if (g + 1 < n) issue_qk(g + 1);
+                load(&tmap_k, sK, k_full, g + kStages);  // S(g) was complete: its K tile has been read
+                if (!landed(v_full, g) || !mbar_wait(p_ready, g & 1)) { failed = true; break; }
                 tc_fence_after_sync();
                 // P: 16 keys = 8 columns of packed pairs.  V: MN-major, 16 keys = two 1024-byte groups (2048 bytes per MMA).
-                const uint64_t vd = make_smem_desc(smem_u32(sV) + (g & 1) * L::kKVBytes, L::kKVBytes, 1024);
+                const uint64_t vd = make_smem_desc(smem_u32(sV) + (g % kStages) * L::kKVBytes, L::kKVBytes, 1024);
 #pragma unroll
                 for (int kk = 0; kk < kStep / 16; ++kk)
-                    mma_ts(tmem_base + kColO, tmem_base + kk * 8, vd + kk * (2048 >> 4), idesc_o, (g | kk) != 0);
-                if (g + 1 < n) issue_qk(g + 1);
-                else mma_commit(s_full);
+                    mma_ts(tmem_base + kColO, tmem_p + kk * 8, vd + kk * (2048 >> 4), idesc_o, (g | kk) != 0);
+                mma_commit(pv_done);
+                if (g > 0) load(&tmap_v, sV, v_full, g - 1 + kStages);  // P(g) was stored after product g - 1: its V tile has been read
             }
         }
         __syncwarp();
@@ -171,7 +181,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
         // head and query row within the tile; a row that is not in use goes along as the last head's first with Q = 0
         const bool live = row < rows;
         const int row_h = min(row / p.head_rows, p.pack - 1), qi = q0 + (live ? row - row_h * p.head_rows : 0);
-        const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
+        const uint32_t lanes = static_cast<uint32_t>(warp * 32) << 16, lane_base = tmem_base + lanes;
         const float sl2 = p.scale_log2;
         float m_run = -INFINITY, l_run = 0.f;  // running maximum of the raw scores (reference of the exponentials), sum
         const int row_limit = min(kvlen - 1, causal ? qi + causal_off : 0x7fffffff);  // last visible key of this row
@@ -189,8 +199,12 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
                 for (int k = 0; k < 32; ++k) s[c * 32 + k] = __uint_as_float(rr[k]);
             }
             tmem_ld_wait();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(s_read);  // the next scores may take S's columns
             const int lim = row_limit - key0;  // last visible column of this step
-            if (__any_sync(0xffffffffu, lim < kStep - 1)) {
+            const bool masked = __any_sync(0xffffffffu, lim < kStep - 1);
+            if (masked) {
 #pragma unroll
                 for (int k = 0; k < kStep; ++k) s[k] = (k <= lim) ? s[k] : -INFINITY;
             }
@@ -217,6 +231,8 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
                 }
                 l_run *= alpha;
                 if (g > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
+                    if (!warp_wait(pv_done, (g - 1) & 1)) { failed = true; break; }  // O holds every product, none is in flight
+                    tc_fence_after_sync();
 #pragma unroll 1
                     for (int c = 0; c < kD / 16; ++c) {
                         uint32_t rr[16];
@@ -232,20 +248,30 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
             const float2 sl2v = make_float2(sl2, sl2), neg_m = make_float2(-m_ref * sl2, -m_ref * sl2);
             float2 lsum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
             uint32_t packed[32];
+            auto exponentials = [&](auto fma_tag) {
+                constexpr int kOnFma = decltype(fma_tag)::value;  // of the 32 pairs, evenly spaced
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                const float2 x = ffma2(make_float2(s[2 * k], s[2 * k + 1]), sl2v, neg_m);
-                const float2 pr = make_float2(ex2(x.x), ex2(x.y));  // masked: 0
-                lsum[k & 1] = fadd2(lsum[k & 1], pr);
-                packed[k] = pack16<F16>(pr.x, pr.y);
+                for (int k = 0; k < 32; ++k) {
+                    const float2 x = ffma2(make_float2(s[2 * k], s[2 * k + 1]), sl2v, neg_m);
+                    const bool on_fma = ((k + 1) * kOnFma / 32) != (k * kOnFma / 32);
+                    const float2 pr = on_fma ? ex2_fma2_fine(x) : make_float2(ex2(x.x), ex2(x.y));  // masked: 0
+                    lsum[k & 1] = fadd2(lsum[k & 1], pr);
+                    packed[k] = pack16<F16>(pr.x, pr.y);
+                }
+            };
+            if (masked) exponentials(std::integral_constant<int, 0>{});
+            else exponentials(std::integral_constant<int, kFmaExpPairs>{});
+            if (g > 0) {  // the product of the step before has read its P
+                if (!warp_wait(pv_done, (g - 1) & 1)) { failed = true; break; }
+                tc_fence_after_sync();
             }
-            tmem_st_x32(lane_base, packed);
+            tmem_st_x32(tmem_p + lanes, packed);
             l_run += (lsum[0].x + lsum[0].y) + (lsum[1].x + lsum[1].y);
             // V rows at and beyond lens[b] hold the caller's padding (possibly NaN, and 0 x NaN is NaN): zero them before the
             // product may start.  Rows beyond Skv were zero-filled by the copy itself.
             if (padding && key0 + kStep > kvlen && kvlen < p.Skv) {
-                if (!warp_wait(&v_full[g & 1], (g >> 1) & 1)) { failed = true; break; }
-                uint4* vt = reinterpret_cast<uint4*>(sV + (g & 1) * L::kKVBytes);
+                if (!warp_wait(&v_full[g % kStages], (g / kStages) & 1)) { failed = true; break; }
+                uint4* vt = reinterpret_cast<uint4*>(sV + (g % kStages) * L::kKVBytes);
                 for (int i = max(kvlen - key0, 0) * 8 + row; i < kStep * 8; i += 128) vt[i] = make_uint4(0, 0, 0, 0);
                 fence_proxy_async_smem();
             }
@@ -259,7 +285,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
                 uint16_t* orow = p.out + b * p.o_sb + (head + row_h) * p.o_sh + qi * p.o_ss;
                 for (int c = 0; c < p.head_dim / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = make_uint4(0, 0, 0, 0);
             }
-        } else if (!failed && warp_wait(s_full, n & 1)) {  // the last product
+        } else if (!failed && warp_wait(pv_done, (n - 1) & 1)) {  // the last product
             tc_fence_after_sync();
             // O / l as 16-bit values into Q's place (all scores are done), in the copies' 128-byte swizzle
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
@@ -309,6 +335,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
     if (warp == 4) {
         tc_fence_after_sync();
         tmem_dealloc(tmem_base, kTmemCols);
+        tmem_dealloc(tmem_p, kTmemColsP);
     }
 }
 
