@@ -142,8 +142,9 @@ struct Schedule {
     bool grouped;        // consecutive pieces of a (batch, kv head) go to the warps of a CTA
     int len0, P0, incl0; // of sequence `lane`: clamped length, pieces, pieces of sequences 0..lane
 };
-// (read past the L1: it is read before and after the previous kernel's end)
-__device__ __forceinline__ int clamped_len(const int32_t* lens, int b, int Smax) { return min(max(__ldcg(lens + b), 0), Smax); }
+__device__ __forceinline__ int clamped_len(const int32_t* lens, int b, int Smax) { return min(max(lens[b], 0), Smax); }
+// of the first 32 sequences: past the L1, since it may be read before and after the previous kernel's end
+__device__ __forceinline__ int first_len(const int32_t* lens, int b, int Smax) { return min(max(__ldcg(lens + b), 0), Smax); }
 __device__ __forceinline__ int blocks_of_len(int len) { return (len + kBlockKeys - 1) / kBlockKeys; }
 // pieces of a sequence of nb blocks: at least one, so that a sequence without rows still gets its zeros
 __device__ __forceinline__ int pieces_of(int nb, int C) { return max((nb + C - 1) / C, 1); }
@@ -160,7 +161,7 @@ template <int MODE>
 __device__ __forceinline__ Schedule make_schedule(const int32_t* lens, int B, int Hkv, int Smax, int num_splits,
                                                   int workers, int lane) {
     Schedule s;
-    s.len0 = (lane < B) ? clamped_len(lens, lane, Smax) : 0;
+    s.len0 = (lane < B) ? first_len(lens, lane, Smax) : 0;
     const int nb0 = blocks_of_len(s.len0);
     unsigned total = nb0;
     int max_nb = nb0;
@@ -579,7 +580,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
         }
         pdl_wait();
     }
-    const int len_now = lane < B ? clamped_len(lens, lane, Smax) : 0;
+    const int len_now = early && lane < B ? first_len(lens, lane, Smax) : 0;
 #pragma unroll
     for (int i = 0; i < kStages; ++i) issue();
     bool failed = false;

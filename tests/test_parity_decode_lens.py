@@ -17,11 +17,11 @@ pytestmark = pytest.mark.gpu
                                                     (40, 8, 2, 300, 64, 16), (2, 8, 2, 6000, 64, 86), (3, 4, 1, 9000, 128, 256)])
 def test_lengths_written_by_the_previous_kernel(B, Hq, Hkv, Smax, D, splits):
     w = wl.decode_workload("t", 95, B, Hq, Hkv, Smax, D, splits, D ** -0.5, (128, Smax))
-    q, k, v = to_device(w.q), to_device(w.k), to_device(w.v)
+    q, k, v = to_device(w.q), to_device(w.k_cache), to_device(w.v_cache)
     rng = np.random.RandomState(B)
     # lengths as the bits of pairs (low, high) of bf16 numbers: 128 and more are normal numbers, which the product with 1 keeps
     choices = [np.full(B, Smax, np.int32), rng.randint(128, Smax + 1, B).astype(np.int32), np.full(B, 128, np.int32)]
-    want = [oracle.attn_decode(w.q.values, w.k.values, w.v.values, c, w.scale) for c in choices]
+    want = [oracle.attn_decode(w.q.values, w.k_cache.values, w.v_cache.values, c, w.scale) for c in choices]
     x = [torch.zeros((1, 128), dtype=torch.int16, device="cuda") for _ in choices]
     for t, c in zip(x, choices):
         t[0, :2 * B:2] = torch.from_numpy(c.astype(np.int16)).cuda()
