@@ -274,8 +274,12 @@ int launch_f32(const float* q, const float* k, const float* v, float* out, int B
                int mask_kind, const int32_t* lens, float scale_log2, cudaStream_t s) {
     using T = Tile<D, KSPLIT>;
     const dim3 grid((Sq + T::BM - 1) / T::BM, Hq, B);
-    FORGE_SET_SMEM_ONCE((attn_f32_kernel<D, KSPLIT>), T::kBytes);
-    FORGE_CUDA_TRY(launch_pdl(attn_f32_kernel<D, KSPLIT>, grid, dim3(kThreads), T::kBytes, s, q, k, v, out, Hq, Hkv, Sq, Skv,
+    // A grid of no more CTAs than SMs takes shared memory for one per SM: launched early, beside the previous kernel's CTAs, two of them would
+    // share an SM that is free already while others fall idle a moment later (1 x 12 x 128 back to back: 8.3 us a call).
+    constexpr int kAlone = 116 * 1024;
+    const int smem = T::kBytes < kAlone && (long long)grid.x * Hq * B <= sm_count() ? kAlone : T::kBytes;
+    FORGE_SET_SMEM_ONCE((attn_f32_kernel<D, KSPLIT>), T::kBytes < kAlone ? kAlone : T::kBytes);
+    FORGE_CUDA_TRY(launch_pdl(attn_f32_kernel<D, KSPLIT>, grid, dim3(kThreads), smem, s, q, k, v, out, Hq, Hkv, Sq, Skv,
                               mask_kind, lens, scale_log2));
     return finish_launch(1);
 }
