@@ -97,20 +97,50 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
     const int b = bg / groups, head = (bg - b * groups) * p.pack, kvh = head / (p.Hq / p.Hkv);
     const int q0 = (q_tiles - 1 - round) * p.head_rows;
 
-    if (threadIdx.x == 0) {
-        mbar_init(q_full, 1);
-        for (int i = 0; i < kStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&v_full[i], 1); }
-        mbar_init(s_full, 1); mbar_init(s_read, 4); mbar_init(p_ready, 4); mbar_init(pv_done, 1); mbar_init(o_staged, 4);
-        fence_mbar_init();
-        prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_o);
-    }
+    int kvlen = p.Skv, n = 0;  // n: steps visible to at least one row of the tile
+    auto measure = [&]() {
+        if (padding) kvlen = min(max(p.lens[b], 0), p.Skv);
+        const int kv_end = max(causal ? min(kvlen, min(q0 + p.head_rows, p.Sq) + causal_off) : kvlen, 0);
+        n = (kv_end + kStep - 1) / kStep;
+    };
+    const int rows = p.pack * p.head_rows;
+    auto load = [&](const CUtensorMap* map, uint8_t* ring, uint64_t* full, int g) {
+        if (g >= n) return;
+        const int st = g % kStages;
+        mbar_expect_tx(&full[st], L::kKVBytes);
+        tma_load_4d(ring + st * L::kKVBytes, map, &full[st], 0, g * kStep, kvh, b);
+    };
+    // The first copies leave before the CTA's other threads are ready: their latency covers the rest of the set-up.  (The next kernel
+    // may move in once every CTA has its tensor memory.)
+    bool control = false;
     if (warp == 4) {
         tmem_alloc(tmem_base_slot, kTmemCols);
         tmem_alloc(tmem_base_slot + 1, kTmemColsP);
         tmem_relinquish();
+        if (elect_one()) {
+            control = true;
+            prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_o);
+            mbar_init(q_full, 1);
+            for (int i = 0; i < kStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&v_full[i], 1); }
+            mbar_init(s_full, 1); mbar_init(s_read, 4); mbar_init(p_ready, 4); mbar_init(pv_done, 1); mbar_init(o_staged, 4);
+            fence_mbar_init();
+            fence_proxy_async_smem();
+            pdl_launch_dependents();
+            pdl_wait();
+            measure();
+            if (n > 0) {
+                // rows beyond Sq and columns beyond head_dim are zero-filled by the TMA unit
+                mbar_expect_tx(q_full, (uint32_t)rows * 128);
+                tma_load_4d(sQ, &tmap_q, q_full, 0, q0, head, b);
+                for (int g = 0; g < kStages; ++g) {
+                    load(&tmap_k, sK, k_full, g);
+                    load(&tmap_v, sV, v_full, g);
+                }
+            }
+        }
+        __syncwarp();
     }
     // Rows of the Q tile that are not in use are never written by the copy: zero scores, not whatever lies there.
-    const int rows = p.pack * p.head_rows;
     if (rows < kBM) {
         for (int i = rows * 8 + (int)threadIdx.x; i < kBM * 8; i += kThreads) reinterpret_cast<uint4*>(sQ)[i] = make_uint4(0, 0, 0, 0);
         fence_proxy_async_smem();
@@ -120,26 +150,15 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot[0], tmem_p = tmem_base_slot[1];
     bool failed = false;
-    pdl_launch_dependents();
     pdl_wait();
-
-    int kvlen = p.Skv;
-    if (padding) kvlen = min(max(p.lens[b], 0), p.Skv);
-    const int kv_end = max(causal ? min(kvlen, min(q0 + p.head_rows, p.Sq) + causal_off) : kvlen, 0);
-    const int n = (kv_end + kStep - 1) / kStep;  // steps visible to at least one row of the tile
+    if (!control) measure();
 
     if (warp == 4) {
         // ------------------------------------------------------------------ copies and MMAs
-        if (n > 0 && elect_one()) {
+        if (elect_one() && n > 0) {
             constexpr uint32_t idesc_s = F16 ? make_idesc_f16(kBM, kStep, false, false) : make_idesc_bf16(kBM, kStep, false, false);
             constexpr uint32_t idesc_o = F16 ? make_idesc_f16(kBM, kD, false, true) : make_idesc_bf16(kBM, kD, false, true);
             const uint64_t qd = make_smem_desc(smem_u32(sQ), 16, 1024);
-            auto load = [&](const CUtensorMap* map, uint8_t* ring, uint64_t* full, int g) {
-                if (g >= n) return;
-                const int st = g % kStages;
-                mbar_expect_tx(&full[st], L::kKVBytes);
-                tma_load_4d(ring + st * L::kKVBytes, map, &full[st], 0, g * kStep, kvh, b);
-            };
             auto landed = [&](uint64_t* full, int g) { return mbar_wait(&full[g % kStages], (g / kStages) & 1); };
             auto issue_qk = [&](int g) {
                 tc_fence_after_sync();
@@ -148,13 +167,6 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
                 for (int kk = 0; kk < kD / 16; ++kk) mma_ss(tmem_base, qd + kk * (32 >> 4), kd + kk * (32 >> 4), idesc_s, kk != 0);
                 mma_commit(s_full);
             };
-            // rows beyond Sq and columns beyond head_dim are zero-filled by the TMA unit
-            mbar_expect_tx(q_full, (uint32_t)rows * 128);
-            tma_load_4d(sQ, &tmap_q, q_full, 0, q0, head, b);
-            for (int g = 0; g < kStages; ++g) {
-                load(&tmap_k, sK, k_full, g);
-                load(&tmap_v, sV, v_full, g);
-            }
             if (!mbar_wait(q_full, 0) || !landed(k_full, 0)) failed = true;
             if (!failed) issue_qk(0);
             for (int g = 0; g < n && !failed; ++g) {
@@ -318,7 +330,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
             }
             if (lane == 0) {
                 tma_store_commit();
-                tma_store_wait_all<0>();
+                tma_store_wait_read<0>();  // shared memory is not given up before it has been read
             }
             __syncwarp();
         } else {
