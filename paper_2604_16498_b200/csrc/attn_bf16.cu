@@ -846,7 +846,7 @@ struct TilePlan {
 template <int D>
 TilePlan choose_tiles(int B, int Hq, int Hkv, int Sq, int Skv, int mask_kind, int sms) {
     TilePlan t;
-    const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, (mask_kind & FORGE_MASK_CAUSAL) != 0);
+    const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, (mask_kind & FORGE_MASK_CAUSAL) != 0, true);
     t.pack = hp.pack; t.head_rows = hp.rows;
     const int q_tiles = (Sq + t.head_rows - 1) / t.head_rows;
     const long long groups = (long long)(Hq / t.pack) * B;

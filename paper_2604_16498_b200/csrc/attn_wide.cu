@@ -64,7 +64,8 @@ struct WideItem {
     int b, h, kvh, q0, kvlen, nsteps;  // nsteps: 64-key steps visible to at least one row of the tile (0: no work)
 };
 
-template <bool F16>
+// PACK: several heads per tile (attn_tiles.cuh).
+template <bool F16, bool PACK>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                  const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_o,
@@ -91,8 +92,9 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int G = p.Hq / p.Hkv;
-    const int num_q_tiles = (p.Sq + p.head_rows - 1) / p.head_rows;
-    const int groups = p.Hq / p.pack, heads = p.B * groups;
+    const int head_rows = PACK ? p.head_rows : kBM, pack = PACK ? p.pack : 1;
+    const int num_q_tiles = (p.Sq + head_rows - 1) / head_rows;
+    const int groups = p.Hq / pack, heads = p.B * groups;
     const int num_items = num_q_tiles * heads;
     const int causal_off = p.Skv - p.Sq;
     const bool causal = (p.mask_kind & FORGE_MASK_CAUSAL) != 0;
@@ -109,13 +111,13 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         const int qstep = num_q_tiles - 1 - i / heads;
         const int bh = i % heads;
         it.b = bh / groups;
-        it.h = (bh - it.b * groups) * p.pack;
+        it.h = (bh - it.b * groups) * pack;
         it.kvh = it.h / G;
-        it.q0 = qstep * p.head_rows;
+        it.q0 = qstep * head_rows;
         it.kvlen = p.Skv;
         if (padding) it.kvlen = min(max(p.lens[it.b], 0), p.Skv);
         int kv_end = it.kvlen;
-        if (causal) kv_end = min(kv_end, min(it.q0 + p.head_rows, p.Sq) + causal_off);
+        if (causal) kv_end = min(kv_end, min(it.q0 + head_rows, p.Sq) + causal_off);
         kv_end = max(kv_end, 0);
         it.nsteps = (kv_end + kStep - 1) / kStep;
         return it;
@@ -138,10 +140,12 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         tmem_relinquish();
     }
     // Rows of the Q tile that are not in use are never written by the copies: zero scores, not whatever lies there.
-    for (int r = p.pack * p.head_rows + (int)threadIdx.x / 8; r < kBM; r += kThreads / 8)
-        for (int c = 0; c < kD / 64; ++c)
-            *reinterpret_cast<uint4*>(sQ + c * L::kChunkBytes + r * 128 + (threadIdx.x % 8) * 16) = make_uint4(0, 0, 0, 0);
-    fence_proxy_async_smem();
+    if constexpr (PACK) {
+        for (int r = pack * head_rows + (int)threadIdx.x / 8; r < kBM; r += kThreads / 8)
+            for (int c = 0; c < kD / 64; ++c)
+                *reinterpret_cast<uint4*>(sQ + c * L::kChunkBytes + r * 128 + (threadIdx.x % 8) * 16) = make_uint4(0, 0, 0, 0);
+        fence_proxy_async_smem();
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -162,7 +166,7 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 if (it.nsteps == 0) continue;
                 if (!mbar_wait(q_empty, (q_loads & 1) ^ 1)) { failed = true; break; }
                 ++q_loads;
-                mbar_expect_tx(q_full, (uint32_t)(p.pack * p.head_rows) * (kD * 2));
+                mbar_expect_tx(q_full, (uint32_t)(pack * head_rows) * (kD * 2));
 #pragma unroll
                 for (int c = 0; c < kD / 64; ++c)  // rows beyond Sq and columns beyond head_dim are zero-filled
                     tma_load_4d(sQ + c * L::kChunkBytes, &tmap_q, q_full, c * 64, it.q0, it.h, it.b);
@@ -246,8 +250,8 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         // ------------------------------------------------------------------ softmax / rescale / epilogue
         const int row = warp * 32 + lane;
         // head and query row within the tile; a row that is not in use goes along as the last head's first with Q = 0
-        const bool live = row < p.pack * p.head_rows;
-        const int row_h = min(row / p.head_rows, p.pack - 1), row_q = live ? row - row_h * p.head_rows : 0;
+        const bool live = row < pack * head_rows;
+        const int row_h = min(row / head_rows, pack - 1), row_q = live ? row - row_h * head_rows : 0;
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
         const float sl2 = p.scale_log2;
         int steps[2] = {0, 0};  // steps done so far per parity (phases of s_full, pv_done)
@@ -372,17 +376,17 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
             tc_fence_before_sync();
             fence_proxy_async_smem();
             // With all 128 rows in use (powers of two) a warp's rows are a box of their own; else the tile is one.
-            const bool own = p.pack * p.head_rows == kBM;
+            const bool own = pack * head_rows == kBM;
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(o_free);  // O may be overwritten by the next item's first product
-                mbar_arrive(o_staged);
+                if (!own) mbar_arrive(o_staged);
             }
             if (!own && warp == 0 && !warp_wait(o_staged, items & 1)) { failed = true; break; }
             ++items;
             if (lane == 0) {
                 const int r0 = own ? warp * 32 : 0;
-                const int q = it.q0 + r0 % p.head_rows, h = it.h + r0 / p.head_rows;
+                const int q = it.q0 + r0 % head_rows, h = it.h + r0 / head_rows;
                 if (q < p.Sq && (own || warp == 0)) {
 #pragma unroll
                     for (int cb = 0; cb < kD / 64; ++cb)
@@ -420,7 +424,7 @@ int launch_wide(const void* q, const void* k, const void* v, void* out, int B, i
         return encode_tmap_bf16_sw128(m, base, 4, dims, strides, box);
     };
     CUtensorMap tq, tk, tv, to;
-    const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, (mask_kind & FORGE_MASK_CAUSAL) != 0);
+    const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, (mask_kind & FORGE_MASK_CAUSAL) != 0, false);
     if (!encode(&tq, q, Hq, Sq, st[0], hp.rows, hp.pack)) return FORGE_ERR_CUDA;
     if (!encode(&tk, k, Hkv, Skv, st[1], kStep)) return FORGE_ERR_CUDA;
     if (!encode(&tv, v, Hkv, Skv, st[2], kStep)) return FORGE_ERR_CUDA;
@@ -439,8 +443,10 @@ int launch_wide(const void* q, const void* k, const void* v, void* out, int B, i
     if (!(p.scale_log2 > 0.f)) p.scale_log2 = 1.17549435e-38f;
     p.status = device_status_word();
     if (!p.status) return FORGE_ERR_CUDA;
-    auto kernel = attn_wide_kernel<F16>;
-    FORGE_SET_SMEM_ONCE(kernel, L::kAlloc);
+    const auto packed = attn_wide_kernel<F16, true>, plain = attn_wide_kernel<F16, false>;
+    const auto kernel = hp.pack > 1 ? packed : plain;
+    if (hp.pack > 1) FORGE_SET_SMEM_ONCE(packed, L::kAlloc);
+    else FORGE_SET_SMEM_ONCE(plain, L::kAlloc);
     const int sms = sm_count();
     if (sms <= 0) return FORGE_ERR_CUDA;
     const long long items = (long long)B * (Hq / hp.pack) * ((Sq + hp.rows - 1) / hp.rows);

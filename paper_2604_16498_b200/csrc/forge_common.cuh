@@ -36,7 +36,8 @@ int sm_count();
 // of this library calls pdl_wait() before its first read or write of global memory, which blocks until the
 // predecessor has completed and its writes are visible; a predecessor that never lets go behaves as
 // with an ordinary launch.  Only requests that bring lines into L2 and nowhere else (linear_split.cu's first weights) may
-// go out before it: L2 is coherent, so they see nothing that a later read would not.
+// go out before it: L2 is coherent, so they see nothing that a later read would not.  (attn_decode.cuh also reads the lengths before it,
+// to know what to ask for; what it computes follows from the lengths read afterwards.)
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem_bytes, cudaStream_t s,
                               Args&&... args) {
