@@ -13,9 +13,6 @@
 //               frees the tensor memory.
 //   warps 2-17: epilogue of this CTA's 128 x 256 half of the tile; each warp on its own (no barriers)
 // Two accumulators of 256 columns: the epilogue of tile i overlaps the main loop of tile i + 1.
-// Long k-loops take two column tiles at a time (WIDE): one k-loop fills both accumulators, so a row tile of X is read for 512 columns, 48 KB
-// per 1024 tensor-core cycles instead of 64.  What bounds these products is what L2 delivers to all SMs together, about 12 TB/s (8192 x
-// 6144 x 4096: 3.2 GB in 270 us).  The epilogue overlaps the k-loop no more, which a long one makes up for.
 // Gated form (SwiGLU, silu(X Wg) * (X Wu)): the pair's tile is 256 rows x 128 output columns; each CTA loads 64
 // gate columns and the 64 up columns of the same outputs, so the accumulator holds [gate | up] of CTA 0's columns,
 // then [gate | up] of CTA 1's, and the epilogue multiplies the two halves as it reads them back.
@@ -36,20 +33,15 @@ using namespace ptx;
 constexpr int kBM = 128;          // rows per CTA
 constexpr int kBN = 256;          // columns of the pair's tile (128 loaded per CTA)
 constexpr int kBK = 64;
+constexpr int kStages = 5;
 constexpr int kEpiWarps = 16;     // four per TMEM lane quarter, one 64-column block of the tile each
 constexpr int kThreads = 64 + kEpiWarps * 32;
 constexpr int kTmemCols = 512;    // two accumulators of 256 columns
-#ifndef WIDEK
-#define WIDEK 2048
-#endif
-constexpr int kWideK = WIDEK;
 
-template <bool WIDE>
 struct PairSmem {
-    static constexpr int kStages = WIDE ? 3 : 5;
     static constexpr int kABytes = kBM * kBK * 2;          // 16 KB: 128 rows of X
     static constexpr int kBBytes = kBK * (kBN / 2) * 2;    // 16 KB: 128 columns of W
-    static constexpr int kStageBytes = kABytes + (WIDE ? 2 : 1) * kBBytes;
+    static constexpr int kStageBytes = kABytes + kBBytes;
     static constexpr int kOutBytes = kEpiWarps * 4096;     // output staging: 32 rows x 64 elements per epilogue warp
     static constexpr int kOutOffset = kStages * kStageBytes;
     static constexpr int kBarOffset = kOutOffset + kOutBytes;
@@ -75,16 +67,14 @@ __device__ __forceinline__ float widen16(uint16_t bits) {
     else return __uint_as_float(static_cast<uint32_t>(bits) << 16);
 }
 
-// WIDE: units of two column tiles, see the head of the file.
 // GATED: tmap_w = gate weights, tmap_w2 = up weights, tmap_y stores boxes of 32 columns; no bias, residual or ACT.
-template <int ACT, bool W_NK, bool F16, bool GATED, bool WIDE>
+template <int ACT, bool W_NK, bool F16, bool GATED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                    const __grid_constant__ CUtensorMap tmap_w2,
                    const __grid_constant__ CUtensorMap tmap_y, const uint16_t* __restrict__ bias,
                    const uint16_t* __restrict__ residual, int M, int N, int K, int band_rows, int* __restrict__ status) {
-    using L = PairSmem<WIDE>;
-    constexpr int kStages = L::kStages;
+    using L = PairSmem;
     extern __shared__ uint8_t smem_raw[];
     // the same offset in both CTAs (the dynamic shared memory of a kernel starts at the same address in each)
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -99,38 +89,27 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
     constexpr int BNO = GATED ? kBN / 2 : kBN;  // output columns of the pair's tile
     const int tiles_m = (M + 2 * kBM - 1) / (2 * kBM), tiles_n = (N + BNO - 1) / BNO;
+    const int num_tiles = tiles_m * tiles_n;
     const int kblocks = (K + kBK - 1) / kBK;
-    // Work units.  WIDE: whole rounds of units of two column tiles first; what is left goes tile by tile.  The tiles of the
-    // last, incomplete round of the persistent schedule are cut into two halves of 128 columns (gated: 64 outputs) when that
-    // lets them all run at once: the round then takes half as long, which matters when a pair only gets five or six tiles in
-    // all.
-    const int tiles_n2 = tiles_n / 2, doubles = WIDE ? tiles_m * tiles_n2 : 0, n_wide = doubles - doubles % num_pairs;
-    const int num_tiles = tiles_m * tiles_n - 2 * n_wide;  // one by one
+    // Work units.  The tiles of the last, incomplete round of the persistent schedule are cut into two halves of
+    // 128 columns (gated: 64 outputs) when that lets them all run at once: the round then takes half as long, which matters
+    // when a pair only gets five or six tiles in all.
     const int rem = num_tiles % num_pairs;
     const bool split = rem > 0 && 2 * rem <= num_pairs;
-    const int n_whole = n_wide + (split ? num_tiles - rem : num_tiles);
+    const int n_whole = split ? num_tiles - rem : num_tiles;
     const int num_units = n_whole + (split ? 2 * rem : 0);
-    // Tiles (double tiles) go down the columns of bands of band_rows row tiles (band_rows_of() has the rule).
+    // Tiles go down the columns of bands of band_rows row tiles (band_rows_of() has the rule).
     struct Unit { int m0, n0, width; };  // first row and column, columns
     auto unit_of = [&](int u) {
         Unit x;
-        int tile, half = 0, cols = tiles_n, at = 0;  // `at`: which column tile of a double one
+        int tile = u, col0 = 0;
         x.width = BNO;
-        if (u < n_wide) { tile = u; cols = tiles_n2; x.width = 2 * BNO; }
-        else {
-            tile = u - n_wide;
-            if (u >= n_whole) { const int v = u - n_whole; tile = n_whole - n_wide + (v >> 1); half = v & 1; x.width = BNO / 2; }
-            if (WIDE) {
-                const int left = 2 * (doubles - n_wide);  // tiles of double tiles that no round of units is full of
-                if (tile < left) { at = tile & 1; tile = n_wide + (tile >> 1); cols = tiles_n2; }
-                else { x.m0 = (tile - left) * 2 * kBM; x.n0 = (tiles_n - 1) * BNO + half * (BNO / 2); return x; }  // an odd last column
-            }
-        }
-        const int row0 = tile / (band_rows * cols) * band_rows, in_band = tile - row0 * cols;
+        if (u >= n_whole) { const int v = u - n_whole; tile = n_whole + (v >> 1); col0 = (v & 1) * (BNO / 2); x.width = BNO / 2; }
+        const int row0 = tile / (band_rows * tiles_n) * band_rows, in_band = tile - row0 * tiles_n;
         const int rows = min(band_rows, tiles_m - row0);
         const int col = in_band / rows;
         x.m0 = (row0 + in_band - col * rows) * 2 * kBM;
-        x.n0 = (WIDE ? 2 * col + at : col) * BNO + half * (BNO / 2);
+        x.n0 = col * BNO + col0;
         return x;
     };
 
@@ -164,36 +143,33 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             for (int u = pair; u < num_units && !failed; u += num_pairs) {
                 const Unit un = unit_of(u);
                 const int m0 = un.m0 + (int)rank * kBM;
-                // This CTA's columns of W: half of the tile's (gated: 64 gate columns and the same 64 up columns).  A half tile has
+                // This CTA's columns of W: half of the unit's (gated: 64 gate columns and the same 64 up columns).  A half tile has
                 // 64 columns of W per CTA; gated: the even CTA has the 64 gate columns, the odd one the 64 up columns, so the
                 // accumulator is [gate | up] once.
                 const bool narrow = un.width < BNO;
-                const int subs = un.width > BNO ? 2 : 1;
+                const int n0 = un.n0 + (GATED && narrow ? 0 : (int)rank * (un.width / 2));
                 for (int kb = 0; kb < kblocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1)) { failed = true; break; }
                     uint8_t* sa = smem + stage * L::kStageBytes;
+                    uint8_t* sb = sa + L::kABytes;
                     // one arrival and the bytes of BOTH CTAs' tiles, announced by the even CTA on its barrier
-                    if (rank == 0) mbar_expect_tx(&full[stage], 2 * (L::kABytes + (narrow ? L::kBBytes / 2 : subs * L::kBBytes)));
+                    if (rank == 0) mbar_expect_tx(&full[stage], 2 * (L::kABytes + (narrow ? L::kBBytes / 2 : L::kBBytes)));
                     const uint32_t bar = map_to_cta(&full[stage], 0);
                     tma_load_2d_pair(sa, &tmap_x, bar, kb * kBK, m0);
-                    for (int sub = 0; sub < subs; ++sub) {
-                        uint8_t* sb = sa + L::kABytes + sub * L::kBBytes;
-                        const int n0 = un.n0 + sub * BNO + (GATED && narrow ? 0 : (int)rank * ((narrow ? BNO / 2 : BNO) / 2));
-                        if constexpr (W_NK) {  // rows of W, 64 K-elements (one swizzle span) each
-                            if constexpr (GATED) {
-                                if (!narrow || rank == 0) tma_load_2d_pair(sb, &tmap_w, bar, kb * kBK, n0);  // 64 gate rows
-                                if (!narrow || rank != 0)                                                    // 64 up rows
-                                    tma_load_2d_pair(sb + (narrow ? 0 : 64 * 128), &tmap_w2, bar, kb * kBK, n0);
-                            } else {                                                             // one or two boxes of 64 rows
-                                tma_load_2d_pair(sb, &tmap_w, bar, kb * kBK, n0);
-                                if (!narrow) tma_load_2d_pair(sb + 64 * 128, &tmap_w, bar, kb * kBK, n0 + 64);
-                            }
-                        } else {               // boxes of 64 K-rows x 64 columns
-                            if (!GATED || !narrow || rank == 0) tma_load_2d_pair(sb, &tmap_w, bar, n0, kb * kBK);
-                            if constexpr (GATED) {
-                                if (!narrow || rank != 0) tma_load_2d_pair(sb + (narrow ? 0 : kBK * 128), &tmap_w2, bar, n0, kb * kBK);
-                            } else if (!narrow) tma_load_2d_pair(sb + kBK * 128, &tmap_w, bar, n0 + 64, kb * kBK);
+                    if constexpr (W_NK) {  // rows of W, 64 K-elements (one swizzle span) each
+                        if constexpr (GATED) {
+                            if (!narrow || rank == 0) tma_load_2d_pair(sb, &tmap_w, bar, kb * kBK, n0);  // 64 gate rows
+                            if (!narrow || rank != 0)                                                    // 64 up rows
+                                tma_load_2d_pair(sb + (narrow ? 0 : 64 * 128), &tmap_w2, bar, kb * kBK, n0);
+                        } else {                                                             // one or two boxes of 64 rows
+                            tma_load_2d_pair(sb, &tmap_w, bar, kb * kBK, n0);
+                            if (!narrow) tma_load_2d_pair(sb + 64 * 128, &tmap_w, bar, kb * kBK, n0 + 64);
                         }
+                    } else {               // boxes of 64 K-rows x 64 columns
+                        if (!GATED || !narrow || rank == 0) tma_load_2d_pair(sb, &tmap_w, bar, n0, kb * kBK);
+                        if constexpr (GATED) {
+                            if (!narrow || rank != 0) tma_load_2d_pair(sb + (narrow ? 0 : kBK * 128), &tmap_w2, bar, n0, kb * kBK);
+                        } else if (!narrow) tma_load_2d_pair(sb + kBK * 128, &tmap_w, bar, n0 + 64, kb * kBK);
                     }
                     if (++stage == kStages) { stage = 0; phase ^= 1; }
                 }
@@ -209,36 +185,30 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             int stage = 0;
             uint32_t phase = 0;
             int it = 0;
-            for (int u = pair; u < num_units && !failed; u += num_pairs) {
-                const int width = unit_of(u).width, subs = width > BNO ? 2 : 1;
-                const uint32_t idesc = width < BNO ? idesc_half : idesc_whole;
-                if (!mbar_wait_cluster(&tmem_empty[it & 1], ((it >> 1) & 1) ^ 1)) { failed = true; break; }
+            for (int u = pair; u < num_units && !failed; u += num_pairs, ++it) {
+                const uint32_t idesc = unit_of(u).width < BNO ? idesc_half : idesc_whole;
+                const int acc = it & 1;
+                const uint32_t acc_phase = (it >> 1) & 1;
+                if (!mbar_wait_cluster(&tmem_empty[acc], acc_phase ^ 1)) { failed = true; break; }
                 tc_fence_after_sync();
+                const uint32_t d_tmem = tmem_base + acc * kBN;
                 for (int kb = 0; kb < kblocks; ++kb) {
                     if (!mbar_wait_cluster(&full[stage], phase)) { failed = true; break; }
                     tc_fence_after_sync();
                     const uint32_t sa = smem_u32(smem + stage * L::kStageBytes);
-                    for (int sub = 0; sub < subs; ++sub) {
-                        if (kb == 0 && sub == 1) {  // the second accumulator may still be read when the first one is free
-                            if (!mbar_wait_cluster(&tmem_empty[(it + 1) & 1], (((it + 1) >> 1) & 1) ^ 1)) { failed = true; break; }
-                            tc_fence_after_sync();
-                        }
-                        const uint32_t sb = sa + L::kABytes + sub * L::kBBytes;
-                        const uint32_t d_tmem = tmem_base + ((it + sub) & 1) * kBN;
+                    const uint32_t sb = sa + L::kABytes;
 #pragma unroll
-                        for (int k = 0; k < kBK / 16; ++k) {
-                            const uint64_t a_desc = make_smem_desc(sa + k * 32, 16, 1024);
-                            const uint64_t b_desc = W_NK ? make_smem_desc(sb + k * 32, 16, 1024)
-                                                         : make_smem_desc(sb + k * 2048, kBK * 128, 1024);
-                            mma_ss_pair(d_tmem, a_desc, b_desc, idesc, (kb | k) != 0);
-                        }
+                    for (int k = 0; k < kBK / 16; ++k) {
+                        const uint64_t a_desc = make_smem_desc(sa + k * 32, 16, 1024);
+                        const uint64_t b_desc = W_NK ? make_smem_desc(sb + k * 32, 16, 1024)
+                                                     : make_smem_desc(sb + k * 2048, kBK * 128, 1024);
+                        mma_ss_pair(d_tmem, a_desc, b_desc, idesc, (kb | k) != 0);
                     }
-                    if (failed) break;
                     mma_commit_pair(&empty[stage], 0x3);  // both CTAs' stages are free once these MMAs have read them
                     if (++stage == kStages) { stage = 0; phase ^= 1; }
                 }
                 if (failed) break;
-                for (int sub = 0; sub < subs; ++sub, ++it) mma_commit_pair(&tmem_full[it & 1], 0x3);  // both epilogues may read it
+                mma_commit_pair(&tmem_full[acc], 0x3);    // both epilogues may read the accumulator
             }
         }
     } else if (warp >= 2) {
@@ -250,11 +220,9 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         uint8_t* stage_out = smem + L::kOutOffset + (warp - 2) * 4096;
         const uint32_t empty_on_leader = map_to_cta(&tmem_empty[0], 0);  // [acc] at + 8 * acc
         int it = 0;
-        for (int u = pair, sub = 0; u < num_units; ++it) {
+        for (int u = pair; u < num_units; u += num_pairs, ++it) {
             const Unit un = unit_of(u);
-            const int m0 = un.m0 + (int)rank * kBM, n0 = un.n0 + sub * BNO;
-            if (un.width > BNO && sub == 0) sub = 1;  // the unit's second tile comes next
-            else { sub = 0; u += num_pairs; }
+            const int m0 = un.m0 + (int)rank * kBM, n0 = un.n0;
             const int acc = it & 1;
             const uint32_t acc_phase = (it >> 1) & 1;
             if (!warp_wait(&tmem_full[acc], acc_phase)) { failed = true; break; }
@@ -368,10 +336,10 @@ inline int band_rows_of(int tiles_n, int K) {
     return fit < 8 ? 8 : fit > 24 ? 24 : (int)fit;
 }
 
-template <int ACT, bool W_NK, bool F16, bool GATED, bool WIDE>
-int launch_pair_as(const void* x, const void* w, const void* b, const void* residual, void* y, int M, int N, int K,
-                cudaStream_t s, const void* w_up) {
-    using L = PairSmem<WIDE>;
+template <int ACT, bool W_NK, bool F16, bool GATED = false>
+int launch_pair(const void* x, const void* w, const void* b, const void* residual, void* y, int M, int N, int K,
+                cudaStream_t s, const void* w_up = nullptr) {
+    using L = PairSmem;
     constexpr int BNO = GATED ? kBN / 2 : kBN;
     CUtensorMap tmap_x, tmap_w, tmap_w2, tmap_y;
     {
@@ -408,25 +376,15 @@ int launch_pair_as(const void* x, const void* w, const void* b, const void* resi
     if (!status) return FORGE_ERR_CUDA;
     const int sms = sm_count();
     if (sms <= 1) return FORGE_ERR_CUDA;
-    auto kernel = linear_pair_kernel<ACT, W_NK, F16, GATED, WIDE>;
+    auto kernel = linear_pair_kernel<ACT, W_NK, F16, GATED>;
     FORGE_SET_SMEM_ONCE(kernel, L::kAlloc);
     const int tiles = ((M + 2 * kBM - 1) / (2 * kBM)) * ((N + BNO - 1) / BNO);
     const int pairs = tiles < sms / 2 ? tiles : sms / 2;
     // the cluster shape is part of the kernel (__cluster_dims__); programmatic stream serialisation as everywhere
     FORGE_CUDA_TRY(launch_pdl(kernel, dim3(2 * pairs), dim3(kThreads), L::kAlloc, s, tmap_x, tmap_w, tmap_w2, tmap_y,
                               static_cast<const uint16_t*>(b), static_cast<const uint16_t*>(residual), M, N, K,
-                              band_rows_of((N + BNO - 1) / BNO / (WIDE ? 2 : 1), K), status));
+                              band_rows_of((N + BNO - 1) / BNO, K), status));
     return finish_launch(1);
-}
-
-template <int ACT, bool W_NK, bool F16, bool GATED = false>
-int launch_pair(const void* x, const void* w, const void* b, const void* residual, void* y, int M, int N, int K,
-                cudaStream_t s, const void* w_up = nullptr) {
-    constexpr int BNO = GATED ? kBN / 2 : kBN;
-    const long long doubles = (long long)((M + 2 * kBM - 1) / (2 * kBM)) * ((N + BNO - 1) / BNO / 2);
-    return K >= kWideK && doubles >= sm_count() / 2
-               ? launch_pair_as<ACT, W_NK, F16, GATED, true>(x, w, b, residual, y, M, N, K, s, w_up)
-               : launch_pair_as<ACT, W_NK, F16, GATED, false>(x, w, b, residual, y, M, N, K, s, w_up);
 }
 
 template <bool W_NK, bool F16>
