@@ -384,10 +384,14 @@ int launch_narrow(const void* q, const void* k, const void* v, void* out, int B,
     p.status = device_status_word();
     if (!p.status) return FORGE_ERR_CUDA;
     const auto kernel = attn_narrow_kernel<F16>;
-    FORGE_SET_SMEM_ONCE(kernel, L::kAlloc);
+    constexpr int kAlone = 116 * 1024, kTwo = 78 * 1024;
+    FORGE_SET_SMEM_ONCE(kernel, kAlone);
     const long long tiles = (long long)B * (Hq / hp.pack) * ((Sq + hp.rows - 1) / hp.rows);
     if (tiles > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
-    FORGE_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)tiles), dim3(kThreads), L::kAlloc, s, tq, tk, tv, to, p));
+    // No more CTAs per SM than it takes to run all tiles at once: launched early, beside the previous kernel's, three of them would share an
+    // SM that is free already while others fall idle a moment later.
+    const int sms = sm_count(), smem = tiles <= sms ? kAlone : tiles <= 2LL * sms ? kTwo : L::kAlloc;
+    FORGE_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)tiles), dim3(kThreads), smem, s, tq, tk, tv, to, p));
     return finish_launch(1);
 }
 

@@ -326,14 +326,15 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
 
 // Row tiles per band of the tile order.  The pairs that run at once should share operands: row by row, the 74 pairs of a round
 // read one row tile of X and 74 column tiles of W, and with N = 14336 (gated: 112 column tiles, 235 MB of W) every row tile reads all of
-// W from HBM again, 7.5 GB a call at 8192 rows.  Down the columns of a band of 24 row tiles a round reads 24 + 3 tiles, and the band's
-// rows of X stay in L2 while W passes once: 8192 x 14336 x 4096 gated 1485 -> 1323 us (8 / 16 rows: 1496 / 1398), 4096 x 14336 x 4096
-// 380 -> 349, 1024 x 14336 x 4096 gated 209 -> 187.  A band's rows of X are at most about 48 MB.  Up to 16 column tiles a round of
-// whole rows is nearly square already (8192 x 3072 x 768 37.3, 39.0 with bands of 16; 5027 x 4096 x 4096 130 and 136).
+// W from HBM again, 7.5 GB a call at 8192 rows.  Down the columns of a band of 16 row tiles a round reads 16 + 5 tiles, and the band's
+// rows of X stay in L2 while W passes once.  Sustained, us, row by row and with bands of 8 / 16 / 24 / 32: 8192 x 14336 x 4096 gated
+// 1665, 1391 / 1352 / 1398 / 1399; 2314 rows 514, 437 / 424 / 427 / 432; 4096 x 14336 x 4096 412, 361 / 357 / 356 / 356; 8192 x 6144 x
+// 4096 323, 317 / 312 / 317 / 337.  A band's rows of X are at most about 48 MB.  Up to 16 column tiles a round of whole rows is nearly
+// square already (8192 x 3072 x 768 37.3, 39.0 with bands of 16; 5027 x 4096 x 4096 130 and 136).
 inline int band_rows_of(int tiles_n, int K) {
     if (tiles_n <= 16) return 1;
     const long long fit = (48LL << 20) / (2LL * kBM * 2 * K);
-    return fit < 8 ? 8 : fit > 24 ? 24 : (int)fit;
+    return fit < 8 ? 8 : fit > 16 ? 16 : (int)fit;
 }
 
 template <int ACT, bool W_NK, bool F16, bool GATED = false>
