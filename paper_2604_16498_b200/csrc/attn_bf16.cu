@@ -1,6 +1,7 @@
 // Fused attention, 16-bit in / fp32 accumulate / 16-bit out (Eq. 8 / Eq. 9): scores, mask, online
 // softmax and the product with V in one kernel; S and P never reach global memory.  The element type
 // is bf16 or fp16 (a template parameter: the MMA operand format and the two conversions differ).
+// Head sizes 72 .. 128, and up to 64 with an additive bias (attn_narrow.cu has the rest up to 64).
 //
 // One work item = two 128-row query tiles (see the item decoding below).  Every 128-key tile of S is
 // computed, normalised and multiplied with V in two 64-key halves with their own barriers, so each
@@ -28,9 +29,9 @@
 // Between items: each tile has two Q buffers, so the issuer sends the first two scores of the next item right behind
 // the last products of this one; the output is staged in the Q buffer of its own item (whose last reader was that item's
 // last S) and stored from there by warp 11, which then hands the buffer back.  A boundary costs the softmax warps
-// about 3100 cycles instead of 4700 (8 x 12 x 1024 x 64 causal 34.1 -> 32.3 us, 18 x 32/8 x 895 x 96 padded 153 -> 149).
+// about 3100 cycles instead of 4700 (18 x 32/8 x 895 x 96 padded 153 -> 149 us).
 // The CTA's last output is stored by the softmax warps, each its own rows, without the way through warp 11: with one item
-// per CTA that is 0.4 us (6 x 12 heads x 385 causal, D = 128, 12.56 -> 12.15; 8 x 12 x 1024 x 64 32.26 -> 31.8).
+// per CTA that is 0.4 us (6 x 12 heads x 385 causal, D = 128, 12.56 -> 12.15).
 // Reading the output only after the next item's first half-step gained nothing more and cost short items their overlap
 // (64 x 16/4 x 64: 16.7 -> 21.3 us).  At D = 128 long runs are at the power limit: fewer cycles, lower clock.
 #include <type_traits>
@@ -596,12 +597,8 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 break;
             }
             pending = false;
-            // One half-step.  At D = 64 the first one of an item has code of its own, without the votes and branches that its
-            // state decides (34.0 -> 32.3 us at 8 x 12 x 1024); at D = 128 and with a bias the second copy of the code
-            // costs as much as it saves.
-            constexpr bool kOwnFirst = D == 64 && !BIAS;
-            auto do_step = [&](auto first_tag, int g) -> bool {
-                constexpr bool kFirst = decltype(first_tag)::value;
+            // One half-step.
+            auto do_step = [&](int g) -> bool {
                 const int step = steps + g, hh = step & 1;
                 const uint32_t col_h = col_s + hh * kHalf;
                 const int key0 = g * kHalf;
@@ -675,7 +672,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 // current reference in the same pass that finds the maximum.  Valid as long as no row's
                 // maximum exceeds its reference by more than the threshold, which is what the lazy rescale
                 // tolerates anyway; otherwise the half is redone below with a new reference.
-                if (!kFirst && !stored && __all_sync(0xffffffffu, m_run != -INFINITY)) {
+                if (!stored && __all_sync(0xffffffffu, m_run != -INFINITY)) {
                     auto fast_path = [&](auto fma_tag) {
                         constexpr bool kUseFma = decltype(fma_tag)::value;
                         const float2 neg_m = make_float2(-m_run * sl2, -m_run * sl2);
@@ -727,7 +724,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                         alpha = (m_run == -INFINITY) ? 1.f : ex2((m_run - m_tile) * sl2);
                         m_run = m_tile;
                     }
-                    if (!kFirst && (kOwnFirst || g > 0) && __any_sync(0xffffffffu, alpha != 1.f)) {
+                    if (g > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
                         // O_t must hold every product issued so far and none may be in flight: the product of
                         // half-step g - 1 (the other half's latest) is the only one the barrier above does not cover.
                         if (!warp_wait(&pv_done[t * 2 + (hh ^ 1)], ((step - 1) >> 1) & 1)) return false;
@@ -783,14 +780,9 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 if (lane == 0) mbar_arrive(&p_ready[t * 2 + hh]);  // one arrival per warp
                 return true;
             };
-            int g = 0;
-            if constexpr (kOwnFirst) {
-                if (nh > 0 && !do_step(std::true_type{}, 0)) { failed = true; break; }
-                g = 1;
-            }
 #pragma unroll 1
-            for (; g < nh; ++g)
-                if (!do_step(std::false_type{}, g)) { failed = true; break; }
+            for (int g = 0; g < nh; ++g)
+                if (!do_step(g)) { failed = true; break; }
             if (failed) break;
             if (nh > 0) {
                 pending = true;

@@ -40,10 +40,9 @@ constexpr int kStages = 3;        // of K and of V
 constexpr int kTmemCols = 128;    // S and O
 constexpr int kTmemColsP = 32;
 constexpr int kColO = 64;
-#ifndef NFMA
-#define NFMA 8
-#endif
-constexpr int kFmaExpPairs = NFMA;
+// of the 32 score pairs of an unmasked step, how many take their exponentials on the FMA pipe (0 / 4 / 8 / 12: 4 x 16 heads x 2048 not
+// causal 97.9 / 97.0 / 95.1 / 97.6 us)
+constexpr int kFmaExpPairs = 8;
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
 
 struct NarrowSmem {
