@@ -45,7 +45,6 @@ constexpr int kThreads = 64 + kEpiWarps * 32;
 constexpr int kMaxStages = 10;          // deeper rings only lengthen the queue in front of the last tile (13.8 against 14.7 us at 4 x 8192 x 2048 gated)
 constexpr int kAhead = 4;                // 8-element pieces of the residual that a thread has in flight
 constexpr int kABytes = kBM * kBK * 2;   // what an MMA reads of A
-constexpr int kAlone = 116 * 1024;       // shared memory that leaves no room for a second CTA on the SM
 
 struct SplitParams {
     const uint16_t* bias;
@@ -382,9 +381,6 @@ int launch_split(const SplitPlan& plan, const void* x, const void* w, const void
     const long long ctas = (long long)((M + kBM - 1) / kBM) * ((N + bno - 1) / bno) * S;
     if (ctas > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
     p.prefetch = plan.two_per_sm || ctas * 2 <= sm_count();
-    // A grid of no more CTAs than SMs takes an SM for each: launched early, beside the previous kernel's CTAs, two of them would share an SM
-    // that is free already while others fall idle a moment later (back to back: 49 x 792 x 480 5.1 -> 4.7 us, 1 x 328 x 3232 5.7 -> 5.3).
-    if (ctas <= sm_count() && total < kAlone) total = kAlone;
     p.status = device_status_word();
     if (!p.status) return FORGE_ERR_CUDA;
 
