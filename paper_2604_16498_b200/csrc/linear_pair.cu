@@ -133,20 +133,6 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const uint32_t tmem_base = *tmem_base_slot;
     bool failed = false;
     pdl_launch_dependents();
-    // While the previous kernel's last CTAs still run, the first k-blocks are asked into L2 (8192 x 3072 x 768 33.5 -> 33.0 us,
-    // 2048 x 3072 x 768 14.7 -> 14.3; the weights alone give a third of that).
-    if (warp == 0 && pair < num_units && elect_one()) {
-        const Unit un = unit_of(pair);
-        const bool narrow = un.width < BNO;
-        const int n0 = un.n0 + (GATED && narrow ? 0 : (int)rank * (un.width / 2));
-        auto ask = [&](const CUtensorMap* map, int kb, int col) { tma_prefetch_l2_2d(map, W_NK ? kb * kBK : col, W_NK ? col : kb * kBK); };
-        for (int kb = 0; kb < min(kblocks, kStages); ++kb) {
-            tma_prefetch_l2_2d(&tmap_x, kb * kBK, un.m0 + (int)rank * kBM);
-            if (!GATED || !narrow || rank == 0) ask(&tmap_w, kb, n0);
-            if (GATED ? !narrow || rank != 0 : !narrow) ask(GATED ? &tmap_w2 : &tmap_w, kb, GATED ? n0 : n0 + 64);
-        }
-    }
-    __syncwarp();
     pdl_wait();
 
     if (warp == 0) {
