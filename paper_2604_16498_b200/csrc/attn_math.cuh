@@ -20,6 +20,12 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
+// the same, NaN if one of them is
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+    float d;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
     float2 d;
     asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
@@ -44,7 +50,7 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
 // 2^x for two values on the FMA and integer pipes instead of the special-function unit (which is the
 // narrowest pipe of the softmax): x = n + f with n = round(x), f in [-0.5, 0.5]; 2^f by a cubic with a
 // relative error of 7.6e-5 (far below the bf16 rounding of P); n is added to the exponent field.
-// Inputs below -125 give 2^-125 rather than 0, so this is used only where no score is masked.
+// Inputs below -125, -infinity and NaN give 2^-125, so this is used only where no score is masked or NaN and the row's reference is finite.
 __device__ __forceinline__ float2 ex2_fma2(float2 x) {
     const float kMagic = 12582912.f;  // 1.5 * 2^23: adding it leaves round(x) in the low mantissa bits
     x.x = fmaxf(x.x, -125.f);

@@ -224,24 +224,26 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
             float mx[4] = {s[0], s[1], s[2], s[3]};
 #pragma unroll
             for (int k = 4; k + 7 < kStep; k += 8) {
-                mx[0] = max3(mx[0], s[k], s[k + 1]);
-                mx[1] = max3(mx[1], s[k + 2], s[k + 3]);
-                mx[2] = max3(mx[2], s[k + 4], s[k + 5]);
-                mx[3] = max3(mx[3], s[k + 6], s[k + 7]);
+                mx[0] = max3_nan(mx[0], s[k], s[k + 1]);
+                mx[1] = max3_nan(mx[1], s[k + 2], s[k + 3]);
+                mx[2] = max3_nan(mx[2], s[k + 4], s[k + 5]);
+                mx[3] = max3_nan(mx[3], s[k + 6], s[k + 7]);
             }
-            mx[0] = max3(mx[0], s[kStep - 4], s[kStep - 3]);
-            mx[1] = max3(mx[1], s[kStep - 2], s[kStep - 1]);
-            const float m_tile = max3(fmaxf(mx[0], mx[1]), mx[2], mx[3]);
-            // keep the old reference unless this step's maximum exceeds it by more than the threshold
-            bool grow = (m_tile - m_run) * sl2 > kRescaleThreshold || m_run == -INFINITY;
-            if (m_tile == -INFINITY) grow = false;
-            if (__any_sync(0xffffffffu, grow)) {
+            mx[0] = max3_nan(mx[0], s[kStep - 4], s[kStep - 3]);
+            mx[1] = max3_nan(mx[1], s[kStep - 2], s[kStep - 1]);
+            const float m_tile = max3_nan(max3_nan(mx[0], mx[1], mx[1]), mx[2], mx[3]);  // NaN if a score is
+            // Keep the old reference unless this step's maximum exceeds it by more than the threshold.  The comparison also fails for a
+            // row without a reference yet, a NaN and a second +inf.
+            bool exact = masked;  // no exponentials on the FMA pipe: there a score of -inf or NaN would count as a small one
+            if (__any_sync(0xffffffffu, !((m_tile - m_run) * sl2 <= kRescaleThreshold))) {
+                const bool grow = m_tile > -INFINITY && !((m_tile - m_run) * sl2 <= kRescaleThreshold);  // never by a NaN
                 float alpha = 1.f;
                 if (grow) {
                     // first visible keys of this row: nothing accumulated yet, nothing to rescale
                     alpha = (m_run == -INFINITY) ? 1.f : ex2((m_run - m_tile) * sl2);
                     m_run = m_tile;
                 }
+                exact = exact || __any_sync(0xffffffffu, m_tile != m_tile || fabsf(m_run) == INFINITY);
                 l_run *= alpha;
                 if (g > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
                     if (!warp_wait(pv_done, (g - 1) & 1)) { failed = true; break; }  // O holds every product, none is in flight
@@ -272,7 +274,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
                     packed[k] = pack16<F16>(pr.x, pr.y);
                 }
             };
-            if (masked) exponentials(std::integral_constant<int, 0>{});
+            if (exact) exponentials(std::integral_constant<int, 0>{});
             else exponentials(std::integral_constant<int, kFmaExpPairs>{});
             if (g > 0) {  // the product of the step before has read its P
                 if (!warp_wait(pv_done, (g - 1) & 1)) { failed = true; break; }
