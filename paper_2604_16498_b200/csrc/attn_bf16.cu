@@ -671,7 +671,8 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 // Fast path (once every row of the warp has a finite reference): exponentials against the
                 // current reference in the same pass that finds the maximum.  Valid as long as no row's
                 // maximum exceeds its reference by more than the threshold, which is what the lazy rescale
-                // tolerates anyway; otherwise the half is redone below with a new reference.
+                // tolerates anyway, and no score is NaN (nor +inf against a reference of +inf), which the exponentials on the FMA
+                // pipe would drop; otherwise the half is redone below, with a new reference where one is due.
                 if (!stored && __all_sync(0xffffffffu, m_run != -INFINITY)) {
                     auto fast_path = [&](auto fma_tag) {
                         constexpr bool kUseFma = decltype(fma_tag)::value;
@@ -682,7 +683,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
 #pragma unroll
                         for (int k = 0; k < 32; ++k) {
                             const float s0 = s[2 * k], s1 = s[2 * k + 1];
-                            mx[k & 3] = max3(mx[k & 3], s0, s1);
+                            mx[k & 3] = max3_nan(mx[k & 3], s0, s1);
                             const float2 x = ffma2(make_float2(s0, s1), sl2v, neg_m);
                             // evenly spaced pairs go to the FMA pipe, the rest to the special-function unit
                             const bool on_fma = kUseFma && ((k + 1) * kFmaExpPairs / 32) != (k * kFmaExpPairs / 32);
@@ -690,8 +691,8 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                             lsum[k & 1] = fadd2(lsum[k & 1], pr);
                             packed[k] = pack16<F16>(pr.x, pr.y);
                         }
-                        const float m_tile = max3(fmaxf(mx[0], mx[1]), mx[2], mx[3]);
-                        if (!__any_sync(0xffffffffu, (m_tile - m_run) * sl2 > kRescaleThreshold)) {
+                        const float m_tile = max3_nan(max3_nan(mx[0], mx[1], mx[1]), mx[2], mx[3]);  // NaN if a score is
+                        if (!__any_sync(0xffffffffu, !((m_tile - m_run) * sl2 <= kRescaleThreshold))) {
                             tmem_st_x32(lane_base + col_h, packed);
                             l_run += (lsum[0].x + lsum[0].y) + (lsum[1].x + lsum[1].y);
                             stored = true;

@@ -8,7 +8,8 @@ from paper_2604_16498_b200 import binding
 
 pytestmark = pytest.mark.gpu
 
-SIZES = [(40, torch.bfloat16), (64, torch.bfloat16), (64, torch.float16)]
+SIZES = [(40, torch.bfloat16), (64, torch.bfloat16), (64, torch.float16), (80, torch.bfloat16), (128, torch.bfloat16), (128, torch.float16),
+         (192, torch.bfloat16)]
 
 
 def _run(q, k, v, mask=0):
