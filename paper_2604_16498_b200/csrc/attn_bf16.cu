@@ -1,7 +1,7 @@
 // Fused attention, 16-bit in / fp32 accumulate / 16-bit out (Eq. 8 / Eq. 9): scores, mask, online
 // softmax and the product with V in one kernel; S and P never reach global memory.  The element type
 // is bf16 or fp16 (a template parameter: the MMA operand format and the two conversions differ).
-// Head sizes 72 .. 128, and up to 64 with an additive bias (attn_narrow.cu has the rest up to 64).
+// Head sizes 72 .. 128, and up to 64 with an additive bias or in many short tiles (many_short_tiles(); attn_narrow.cu has the rest up to 64).
 //
 // One work item = two 128-row query tiles (see the item decoding below).  Every 128-key tile of S is
 // computed, normalised and multiplied with V in two 64-key halves with their own barriers, so each
@@ -174,7 +174,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     // has room for it) the two tiles are two heads on the same query rows instead, each with its own K/V stream through half
     // of the stage ring.
     const int head_rows = PACK ? p.head_rows : kBM, pack = PACK ? p.pack : 1;
-    const bool two_streams = !PACK && kKVStages >= 8 && p.tiles == 2;
+    const bool two_streams = !PACK && kKVStages >= 8 && (!BIAS || p.tiles == 2);  // (without a bias always two tiles: choose_tiles())
     const int ring_len = two_streams ? kKVStages / 2 : kKVStages;
     const int heads = p.inner * p.B;  // items per query step
     const uint32_t q_bytes = (uint32_t)(pack * head_rows) * (D * 2);
@@ -597,8 +597,12 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 break;
             }
             pending = false;
-            // One half-step.
-            auto do_step = [&](int g) -> bool {
+            // One half-step.  At D = 64 the first one of an item has code of its own, without the votes and branches that its
+            // state decides (64 x 16 heads x 128 causal, with a fixed choice of two_streams, 18.3 -> 18.0 us; 64 x 12 x 192 25.6 -> 24.6); at
+            // D = 128 and with a bias the second copy of the code costs as much as it saves.
+            constexpr bool kOwnFirst = D == 64 && !BIAS;
+            auto do_step = [&](auto first_tag, int g) -> bool {
+                constexpr bool kFirst = decltype(first_tag)::value;
                 const int step = steps + g, hh = step & 1;
                 const uint32_t col_h = col_s + hh * kHalf;
                 const int key0 = g * kHalf;
@@ -673,7 +677,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 // maximum exceeds its reference by more than the threshold, which is what the lazy rescale
                 // tolerates anyway, and no score is NaN (nor +inf against a reference of +inf), which the exponentials on the FMA
                 // pipe would drop; otherwise the half is redone below, with a new reference where one is due.
-                if (!stored && __all_sync(0xffffffffu, m_run != -INFINITY)) {
+                if (!kFirst && !stored && __all_sync(0xffffffffu, m_run != -INFINITY)) {
                     auto fast_path = [&](auto fma_tag) {
                         constexpr bool kUseFma = decltype(fma_tag)::value;
                         const float2 neg_m = make_float2(-m_run * sl2, -m_run * sl2);
@@ -687,7 +691,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                             const float2 x = ffma2(make_float2(s0, s1), sl2v, neg_m);
                             // evenly spaced pairs go to the FMA pipe, the rest to the special-function unit
                             const bool on_fma = kUseFma && ((k + 1) * kFmaExpPairs / 32) != (k * kFmaExpPairs / 32);
-                            const float2 pr = on_fma ? ex2_fma2(x) : make_float2(ex2(x.x), ex2(x.y));
+                            const float2 pr = !on_fma ? make_float2(ex2(x.x), ex2(x.y)) : D == 64 ? ex2_fma2_fine(x) : ex2_fma2(x);
                             lsum[k & 1] = fadd2(lsum[k & 1], pr);
                             packed[k] = pack16<F16>(pr.x, pr.y);
                         }
@@ -725,7 +729,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                         alpha = (m_run == -INFINITY) ? 1.f : ex2((m_run - m_tile) * sl2);
                         m_run = m_tile;
                     }
-                    if (g > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
+                    if (!kFirst && (kOwnFirst || g > 0) && __any_sync(0xffffffffu, alpha != 1.f)) {
                         // O_t must hold every product issued so far and none may be in flight: the product of
                         // half-step g - 1 (the other half's latest) is the only one the barrier above does not cover.
                         if (!warp_wait(&pv_done[t * 2 + (hh ^ 1)], ((step - 1) >> 1) & 1)) return false;
@@ -781,9 +785,14 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                 if (lane == 0) mbar_arrive(&p_ready[t * 2 + hh]);  // one arrival per warp
                 return true;
             };
+            int g = 0;
+            if constexpr (kOwnFirst) {
+                if (nh > 0 && !do_step(std::true_type{}, 0)) { failed = true; break; }
+                g = 1;
+            }
 #pragma unroll 1
-            for (int g = 0; g < nh; ++g)
-                if (!do_step(g)) { failed = true; break; }
+            for (; g < nh; ++g)
+                if (!do_step(std::false_type{}, g)) { failed = true; break; }
             if (failed) break;
             if (nh > 0) {
                 pending = true;
@@ -836,14 +845,14 @@ struct TilePlan {
 
 // One tile per item where that leaves no SM with two of them (a lone tile takes a little more than half the time of a pair: 1 x
 // 16 heads x 518 x 80 12.0 -> 10.5 us, 1 x 32/8 x 256 behind 1000 keys 25.0 -> 20.0), else two.
-template <int D>
+template <int D, bool BIAS>
 TilePlan choose_tiles(int B, int Hq, int Hkv, int Sq, int Skv, int mask_kind, int sms) {
     TilePlan t;
     const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, (mask_kind & FORGE_MASK_CAUSAL) != 0, true);
     t.pack = hp.pack; t.head_rows = hp.rows;
     const int q_tiles = (Sq + t.head_rows - 1) / t.head_rows;
     const long long groups = (long long)(Hq / t.pack) * B;
-    t.tiles = groups * q_tiles <= sms ? 1 : 2;
+    t.tiles = (D > 64 || BIAS) && groups * q_tiles <= sms ? 1 : 2;  // (D = 64 without a bias: always many, see many_short_tiles())
     t.two_streams = t.pack == 1 && t.tiles == 2 && AttnSmem<D>::kKVStages >= 8;  // the kernel asks the same
     t.inner = t.two_streams ? (Hq + 1) / 2 : Hq / t.pack;
     t.steps = t.two_streams ? q_tiles : (q_tiles + t.tiles - 1) / t.tiles;
@@ -860,7 +869,7 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
     using L = AttnSmem<D>;
     const int sms = sm_count();
     if (sms <= 0) return FORGE_ERR_CUDA;
-    const TilePlan plan = choose_tiles<D>(B, Hq, Hkv, Sq, Skv, mask_kind, sms);
+    const TilePlan plan = choose_tiles<D, BIAS>(B, Hq, Hkv, Sq, Skv, mask_kind, sms);
     const Strides a = dense_strides(Hq, Sq, head_dim), c = dense_strides(Hkv, Skv, head_dim);
     const Strides sq = strides ? strides[0] : a, sk = strides ? strides[1] : c, sv = strides ? strides[2] : c, so = strides ? strides[3] : a;
     // every tensor as a 4-D map (D, rows, heads, batch): the strides carry the layout
@@ -908,13 +917,37 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
     return finish_launch(1);
 }
 
-// No bias: head sizes up to 64 run on the kernel of attn_narrow.cu, those above 128 on that of attn_wide.cu.  strides: of q, k, v, out,
-// or nullptr for dense tensors.
+// Head sizes up to 64 without a bias.  attn_narrow.cu sets up a CTA for every tile, three per SM: the better way where they all run at once
+// or a tile has steps enough to hide its set-up.  Many short tiles run on this file's kernel, whose CTAs stay and fetch the next item's
+// Q, K and V beside the current one's steps.  Measured, narrow and this one, us: 64 x 16 heads x 64 causal 18.4 and 14.6, x 192 35.4 and
+// 29.9, x 512 (320 keys a tile) 113 and 107, x 384 not causal 85.0 and 85.0; 64 x 32/8 x 128 causal 31.3 and 23.9, padded 31.7 and 27.4.
+// The other way round: 20 x 12 x 384 causal (4.9 tiles per SM; a third round of few long items) 18.2 and 20.0, x 512 (6.5) 26.3 and 26.9;
+// 40 x 15 x 100 (4.1: a third round, nearly empty) 12.1 and 13.1; with a lone tile in every sixth item 26 x 16/4 x 321 22.8 and 24.5, in
+// every second one 64 x 16/4 x 96 padded 13.3 and 15.6; with lengths half of the keys or less 36 x 12 x 444 38.0 and 38.6.
+inline bool many_short_tiles(int B, int Hq, int Hkv, int Sq, int Skv, int mask_kind, int sms) {
+    if ((long long)B * Hq * ((Sq + kBM - 1) / kBM) <= 3LL * sms) return false;  // whatever the packing (a small call's host time counts)
+    const bool causal = (mask_kind & FORGE_MASK_CAUSAL) != 0, padded = (mask_kind & FORGE_MASK_PADDING) != 0;
+    const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, causal, true);
+    const int q_tiles = (Sq + hp.rows - 1) / hp.rows;
+    const long long tiles = (long long)B * (Hq / hp.pack) * q_tiles;
+    if (tiles <= 3LL * sms || (tiles > 4LL * sms && tiles <= 5LL * sms)) return false;
+    const bool lone = hp.pack > 1 && q_tiles % 2;  // the last item of a head group has one tile
+    if (lone && (padded || q_tiles <= 3 || tiles <= 9LL * sms)) return false;
+    const double keys = causal ? Skv - 0.5 * Sq + 0.5 * hp.rows : Skv;  // that a tile is given on average
+    if (tiles > 9LL * sms) return keys <= (padded ? 256 : 320);
+    return keys <= (mask_kind == FORGE_MASK_NONE || (tiles > 6LL * sms && !padded) ? 256 : 128);
+}
+
+// Head sizes above 128 run on the kernel of attn_wide.cu.  strides: of q, k, v, out, or nullptr for dense tensors.
 template <bool F16>
 int attn_by_head_size(const void* q, const void* k, const void* v, void* out, int B, int Hq, int Hkv, int Sq, int Skv, int D,
                       int mask_kind, const int32_t* lens, float scale, cudaStream_t s, const Strides* strides = nullptr) {
     if (D > 64 && D <= 128)
         return launch_attn<128, F16>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, strides);
+    const int sms = sm_count();
+    if (sms <= 0) return FORGE_ERR_CUDA;
+    if (D <= 64 && many_short_tiles(B, Hq, Hkv, Sq, Skv, mask_kind, sms))
+        return launch_attn<64, F16>(q, k, v, out, B, Hq, Hkv, Sq, Skv, D, mask_kind, lens, scale, s, strides);
     const Strides a = dense_strides(Hq, Sq, D), c = dense_strides(Hkv, Skv, D), dense[4] = {a, c, c, a};
     const Strides* t = strides ? strides : dense;
     long long st[4][3];

@@ -1,4 +1,5 @@
-// Fused attention for head sizes up to 64 (Eq. 8 / Eq. 9, the same operator as attn_bf16.cu, without an additive bias).
+// Fused attention for head sizes up to 64 (Eq. 8 / Eq. 9, the same operator as attn_bf16.cu, without an additive bias; many short tiles
+// run there: many_short_tiles()).
 //
 // With 64 columns of output a 64-key step is 256 cycles of tensor core against 512 of the special-function unit's exponentials, and
 // the rest of a step (barriers, tensor-memory round trips, fences) is as long as both.  So the kernel is small and the SM

@@ -24,9 +24,9 @@ def _inputs(B, H, Sq, Skv, D, dtype):
     return mk(Sq), mk(Skv), mk(Skv)
 
 
-def _each_key(D, dtype, Skv, value):
-    """Batch entry b has `value` in key b of head 0; head 1 is left alone.  Two rows of queries, positive ones."""
-    q, k, v = _inputs(Skv, 2, 2, Skv, D, dtype)
+def _each_key(D, dtype, Skv, value, H=2):
+    """Batch entry b has `value` in key b of head 0; the others are left alone.  Two rows of queries, positive ones."""
+    q, k, v = _inputs(Skv, H, 2, Skv, D, dtype)
     q = q.abs() + 0.125
     clean = _run(q, k, v)
     for b in range(Skv):
@@ -42,6 +42,15 @@ def test_a_nan_or_inf_score_makes_the_row_nan_at_every_key(D, dtype, Skv, value)
     lost = [b for b in range(Skv) if not got[b, 0].isnan().all()]
     assert not lost, f"keys whose score was dropped: {lost}"
     assert torch.equal(got[:, 1], clean[:, 1])
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_the_same_in_many_short_tiles(value):
+    """More tiles than run at once: 192 x 8."""
+    *_, clean, got = _each_key(64, torch.bfloat16, 192, value, 8)
+    lost = [b for b in range(192) if not got[b, 0].isnan().all()]
+    assert not lost, f"keys whose score was dropped: {lost}"
+    assert torch.equal(got[:, 1:], clean[:, 1:])
 
 
 @pytest.mark.parametrize("D,dtype", SIZES)

@@ -15,8 +15,16 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,Sq,Skv,D,mask,lens", [
-    (40, 8, 8, 130, 200, 64, 2, [0, 1, 63, 64, 65, 128, 129, 200]),     # private K/V streams, empty items among full ones
-    (24, 15, 15, 100, 70, 64, 3, [70, 1, 0, 64]),                       # odd head count; rows without a visible key
+    (40, 8, 8, 130, 200, 64, 2, [0, 1, 63, 64, 65, 128, 129, 200]),     # a CTA per tile, empty ones among full ones
+    (24, 15, 15, 100, 70, 64, 3, [70, 1, 0, 64]),                       # all tiles at once; rows without a visible key
+    # head sizes up to 64 in many short tiles: pairs of heads with private K/V streams, then grouped heads in pairs of tiles
+    (90, 8, 8, 130, 200, 64, 2, [0, 1, 63, 64, 65, 128, 129, 200]),     # empty items among full ones
+    (64, 15, 15, 100, 70, 64, 3, [70, 1, 0, 64]),                       # odd head count (no second tile); rows without a visible key
+    (100, 9, 9, 20, 129, 40, 1, None),                                  # head size below the kernel's, three half-steps
+    (60, 10, 10, 257, 257, 64, 0, None),                                # a last tile of one row
+    (50, 32, 8, 61, 200, 64, 3, [200, 0, 1, 64, 65, 129]),              # four heads of 32 rows
+    (64, 28, 4, 130, 130, 64, 1, None),                                 # seven heads of 18 rows, two of the 128 out of use
+    (64, 28, 4, 195, 195, 56, 1, None),                                 # an odd number of tiles: the last item has one
     (30, 7, 1, 260, 333, 128, 3, [333, 10, 0, 64, 100]),                # odd group: three tiles of a head in two items
     (50, 8, 2, 40, 300, 128, 2, [300, 0, 1, 65, 257]),                  # one tile per head, pairs of heads
     (64, 12, 12, 128, 128, 64, 1, None),                                # two half-steps each
