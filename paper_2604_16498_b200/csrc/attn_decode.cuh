@@ -523,17 +523,20 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
     // as they are now serves to ask this worker's first blocks into L2, while SMs fall idle one by one at the end of that
     // kernel (addresses only, within the cache whatever lens holds), and to start the first copies right after it.  By the
     // time these land it is known whether the lengths are still the same; if not, the copies are dropped and the schedule is
-    // made again.  (More than 32 sequences: the schedule reads lens several times and is made once, afterwards.)
+    // made again, in the same code: with a second copy of it behind the first the streaming loop of 7 heads of 128 got other registers and was
+    // 6 % slower (16 x 28/4 x 10,442 42.2 -> 40.1 us, 4 x 28/4 x 10,000 22.8 -> 20.1; 24 x 32/8 x 3000 21.0 -> 20.8).
+    // (More than 32 sequences: the schedule reads lens several times and is made once, afterwards.)
     const bool early = B <= 32;
     if (!early) pdl_wait();
-    Schedule sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
-    unsigned first_idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
+    bool waited = !early;
+    Schedule sched;
+    unsigned first_idx;
     auto item_of_round = [&](int r) { return (unsigned)r * (unsigned)workers + first_idx; };
 
     // ---- prefetch cursor: runs kStages blocks ahead of the compute, across item boundaries (a stage is
     // refilled as soon as its fragments are in registers, before the MMAs on them)
     int p_round = 0, p_j0 = 0, p_s1 = 0;
-    unsigned p_idx = item_of_round(0);
+    unsigned p_idx = 0;
     int p_bk = 0;  // batch * Hkv + kv head of the cursor's item
     int p_n = 0;  // blocks issued
     auto p_open = [&]() {  // position the cursor on the first block of the next non-empty item
@@ -568,31 +571,33 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
             if (p_j0 >= p_s1) { p_idx = item_of_round(++p_round); p_open(); }
         }
     };
-    p_open();
-    if (early) {
-        const int row = p_j0 + lane * kBlockKeys;
-        if (p_idx < sched.num_items && lane < kStages && row < p_s1) {
-#pragma unroll
-            for (int cb = 0; cb < D / 64; ++cb) {
-                ptx::tma_prefetch_l2_3d(&tmap_k, cb * 64, row, p_bk);
-                ptx::tma_prefetch_l2_3d(&tmap_v, cb * 64, row, p_bk);
-            }
-        }
-        pdl_wait();
-    }
-    const int len_now = early && lane < B ? first_len(lens, lane, Smax) : 0;
-#pragma unroll
-    for (int i = 0; i < kStages; ++i) issue();
     bool failed = false;
     int n = 0;  // blocks consumed
-    if (early && !__all_sync(0xffffffffu, sched.len0 == len_now)) {
-        for (; n < p_n && !failed; ++n) failed = !ptx::warp_wait(&full[n % kStages], (n / kStages) & 1);
+#pragma unroll 1
+    for (;;) {
         sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
         first_idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
         p_round = 0;
         p_idx = item_of_round(0);
         p_open();
-        for (int i = 0; i < kStages && !failed; ++i) issue();
+        if (!waited) {
+            const int row = p_j0 + lane * kBlockKeys;
+            if (p_idx < sched.num_items && lane < kStages && row < p_s1) {
+#pragma unroll
+                for (int cb = 0; cb < D / 64; ++cb) {
+                    ptx::tma_prefetch_l2_3d(&tmap_k, cb * 64, row, p_bk);
+                    ptx::tma_prefetch_l2_3d(&tmap_v, cb * 64, row, p_bk);
+                }
+            }
+            pdl_wait();
+        }
+        const int len_now = !waited && lane < B ? first_len(lens, lane, Smax) : sched.len0;
+#pragma unroll
+        for (int i = 0; i < kStages; ++i) issue();
+        if (__all_sync(0xffffffffu, sched.len0 == len_now)) break;
+        waited = true;
+        for (; n < p_n && !failed; ++n) failed = !ptx::warp_wait(&full[n % kStages], (n / kStages) & 1);
+        if (failed) break;
     }
     const unsigned num_items = sched.num_items;
     if (MODE == kGrouped && sched.grouped && lane == 0) merge_info[warp][0] = -1;
