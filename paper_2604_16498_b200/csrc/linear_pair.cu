@@ -105,10 +105,17 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         int tile = u, col0 = 0;
         x.width = BNO;
         if (u >= n_whole) { const int v = u - n_whole; tile = n_whole + (v >> 1); col0 = (v & 1) * (BNO / 2); x.width = BNO / 2; }
-        const int row0 = tile / (band_rows * tiles_n) * band_rows, in_band = tile - row0 * tiles_n;
-        const int rows = min(band_rows, tiles_m - row0);
-        const int col = in_band / rows;
-        x.m0 = (row0 + in_band - col * rows) * 2 * kBM;
+        int row, col;
+        if (band_rows == 1) {  // two divisions less before a unit's first copy: 8192 x 3072 x 768 35.1 -> 34.9 us
+            row = tile / tiles_n;
+            col = tile - row * tiles_n;
+        } else {
+            const int row0 = tile / (band_rows * tiles_n) * band_rows, in_band = tile - row0 * tiles_n;
+            const int rows = min(band_rows, tiles_m - row0);
+            col = in_band / rows;
+            row = row0 + in_band - col * rows;
+        }
+        x.m0 = row * 2 * kBM;
         x.n0 = col * BNO + col0;
         return x;
     };
