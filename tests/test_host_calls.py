@@ -1,10 +1,13 @@
 """The native marshalling of the frequent calls (host_calls.cpp): what it takes it does as the general Python way does, and what is
 not plain it leaves to that way, which has the checks and the errors."""
+import os
+import subprocess
+
 import pytest
 import torch
 from torch.overrides import TorchFunctionMode
 
-from paper_2604_16498_b200 import binding
+from paper_2604_16498_b200 import binding, build
 
 NOT_PLAIN = -1
 
@@ -43,6 +46,52 @@ def test_bind_wants_nine_addresses():
     for bad in ((), (1,) * 8, (0,) * 9, ("x",) * 9):
         with pytest.raises((TypeError, ValueError)):
             c.bind(*bad)
+
+
+def _fake_tree(monkeypatch, tmp_path):
+    for name, path in (("HERE", ""), ("CSRC", "csrc"), ("INCLUDE", "include"), ("LIB", "libforge.so"), ("HOST_CALLS", "host_calls.x.so"), ("OBJ_DIR", "obj")):
+        monkeypatch.setattr(build, name, str(tmp_path / path))
+    for name in ("csrc/a.cu", "csrc/host_calls.cpp", "include/forge.h"):
+        (tmp_path / name).parent.mkdir(exist_ok=True)
+        (tmp_path / name).write_text("")
+        os.utime(tmp_path / name, (1e9, 1e9))
+    ran = []
+
+    def run(cmd, **kw):
+        ran.append(os.path.basename(cmd[0]))
+        if "-o" in cmd and not (ran[-1] == "g++" and run.gxx_fails):
+            with open(cmd[cmd.index("-o") + 1], "w") as f:
+                f.write(" ".join(cmd))
+        return subprocess.CompletedProcess(cmd, int(ran[-1] == "g++" and run.gxx_fails), "", "no headers")
+    run.gxx_fails = False
+    monkeypatch.setattr(build.subprocess, "run", run)
+    return ran, run
+
+
+def test_the_library_is_built_where_the_module_cannot_be(monkeypatch, tmp_path, capsys):
+    ran, run = _fake_tree(monkeypatch, tmp_path)
+    run.gxx_fails = True
+    (tmp_path / "host_calls.x.so").write_text("of another torch")
+    os.utime(tmp_path / "host_calls.x.so", (2e9, 2e9))
+    assert build.build() == str(tmp_path / "libforge.so") and (tmp_path / "libforge.so").exists()
+    assert not (tmp_path / "host_calls.x.so").exists() and "no headers" in capsys.readouterr().err
+
+
+def test_each_part_is_rebuilt_for_its_own_reasons(monkeypatch, tmp_path):
+    ran, run = _fake_tree(monkeypatch, tmp_path)
+    build.build()
+    assert sorted(ran) == ["g++", "nvcc", "nvcc"]  # one source, the link
+    ran.clear()
+    build.build()
+    assert ran == []
+    os.utime(tmp_path / "csrc/host_calls.cpp", (3e9, 3e9))
+    build.build()
+    assert ran == ["g++"]
+    ran.clear()
+    os.utime(tmp_path / "csrc/a.cu", (3e9, 3e9))
+    os.utime(tmp_path / "host_calls.x.so", (4e9, 4e9))
+    build.build()
+    assert ran == ["nvcc", "nvcc"]
 
 
 def _attn_args(D=64, dtype=torch.bfloat16):
