@@ -12,6 +12,8 @@ import os
 
 import torch
 
+from .build import host_calls_stamp
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libforge.so")
 
@@ -117,7 +119,10 @@ def _bind_host_calls(lib) -> None:
     global _host_calls
     try:
         from . import host_calls
-    except ImportError:  # built for another torch or Python: the general way
+    except ImportError:  # not built, or for another Python: the general way
+        return
+    # Its symbols may resolve in another torch too, whose tensors it would read wrongly: the general way.
+    if getattr(host_calls, "built_for", None) != host_calls_stamp():
         return
     host_calls.bind(*(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _HOST_CALLS_ENTRIES))
     _host_calls = host_calls

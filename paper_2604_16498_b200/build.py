@@ -2,7 +2,8 @@
 the Python binding, ``host_calls``.
 
 ``python -m paper_2604_16498_b200.build`` or ``build()`` from Python.  nvcc cross-compiles
-without a GPU.  Each is rebuilt when one of its sources or headers is newer than it.  Without what ``host_calls`` needs (torch's and Python's headers, g++) the library is built all the
+without a GPU.  Each is rebuilt when one of its sources or headers is newer than it, ``host_calls`` also when it was
+built for another torch.  Without what ``host_calls`` needs (torch's and Python's headers, g++) the library is built all the
 same: the binding works without it, at a few microseconds more per call.
 """
 from __future__ import annotations
@@ -18,7 +19,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libforge.so")
-HOST_CALLS = os.path.join(HERE, "host_calls.so")
+HOST_CALLS = os.path.join(HERE, "host_calls" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))  # importable by this Python only
 OBJ_DIR = os.path.join(HERE, "_build")
 
 NVCC_FLAGS = [
@@ -30,6 +31,12 @@ NVCC_FLAGS = [
 def _nvcc() -> str:
     cand = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "bin", "nvcc")
     return cand if os.path.exists(cand) else "nvcc"
+
+
+def host_calls_stamp() -> str:
+    """What host_calls is built for: it reads tensors through torch's inline accessors, whose layouts are those of one build of torch."""
+    import torch
+    return f"torch {torch.__version__} {torch.version.git_version} python {sysconfig.get_config_var('EXT_SUFFIX')}"
 
 
 def _older(path: str, deps) -> bool:
@@ -45,7 +52,14 @@ def _stale() -> bool:
 
 
 def _host_calls_stale() -> bool:
-    return _older(HOST_CALLS, [os.path.join(CSRC, "host_calls.cpp"), *_headers()])
+    if _older(HOST_CALLS, [os.path.join(CSRC, "host_calls.cpp"), *_headers()]):
+        return True
+    try:
+        stamp = host_calls_stamp()
+    except ImportError:  # no torch, no binding
+        return False
+    with open(HOST_CALLS, "rb") as f:
+        return stamp.encode() not in f.read()
 
 
 def _build_host_calls() -> None:
@@ -57,7 +71,7 @@ def _build_host_calls() -> None:
            os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
     r = subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
                         f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
-                        *(f"-I{i}" for i in inc),
+                        f'-DFORGE_HOST_CALLS_STAMP="{host_calls_stamp()}"', *(f"-I{i}" for i in inc),
                         os.path.join(CSRC, "host_calls.cpp"), "-o", tmp, "-L" + os.path.join(t, "lib"),
                         "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"], capture_output=True, text=True)
     if r.returncode != 0:
@@ -67,8 +81,9 @@ def _build_host_calls() -> None:
 
 def _try_host_calls() -> None:
     """Builds host_calls, or says why not; one that is out of date does not stay."""
-    if os.path.exists(HOST_CALLS):
-        os.remove(HOST_CALLS)
+    for old in {os.path.join(HERE, "host_calls.so"), HOST_CALLS}:
+        if os.path.exists(old):
+            os.remove(old)
     try:
         _build_host_calls()
     except Exception as e:  # whatever is missing: the library does not depend on it

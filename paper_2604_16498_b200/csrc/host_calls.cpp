@@ -218,4 +218,12 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "host_calls", nullptr, -1, methods,
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit_host_calls() { return PyModule_Create(&module); }
+// built_for: the torch and Python this was compiled against (build.py, host_calls_stamp()); binding.py uses the module with no other.
+PyMODINIT_FUNC PyInit_host_calls() {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", FORGE_HOST_CALLS_STAMP) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

@@ -2,6 +2,7 @@
 not plain it leaves to that way, which has the checks and the errors."""
 import os
 import subprocess
+import types
 
 import pytest
 import torch
@@ -48,6 +49,16 @@ def test_bind_wants_nine_addresses():
             c.bind(*bad)
 
 
+@pytest.mark.parametrize("built_for", [None, "torch 2.10.0 abc python .cpython-312-x86_64-linux-gnu.so"])
+def test_a_module_built_for_another_torch_is_not_used(monkeypatch, built_for):
+    lib = binding.load()
+    fake = types.SimpleNamespace(bind=lambda *a: pytest.fail("bound"), **({} if built_for is None else {"built_for": built_for}))
+    monkeypatch.setattr("paper_2604_16498_b200.host_calls", fake, raising=False)
+    monkeypatch.setattr(binding, "_host_calls", None)
+    binding._bind_host_calls(lib)
+    assert binding._host_calls is None
+
+
 def _fake_tree(monkeypatch, tmp_path):
     for name, path in (("HERE", ""), ("CSRC", "csrc"), ("INCLUDE", "include"), ("LIB", "libforge.so"), ("HOST_CALLS", "host_calls.x.so"), ("OBJ_DIR", "obj")):
         monkeypatch.setattr(build, name, str(tmp_path / path))
@@ -84,6 +95,10 @@ def test_each_part_is_rebuilt_for_its_own_reasons(monkeypatch, tmp_path):
     ran.clear()
     build.build()
     assert ran == []
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    build.build()
+    assert ran == ["g++"]
+    ran.clear()
     os.utime(tmp_path / "csrc/host_calls.cpp", (3e9, 3e9))
     build.build()
     assert ran == ["g++"]
