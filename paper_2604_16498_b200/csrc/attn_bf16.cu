@@ -117,7 +117,7 @@ struct AttnParams {
     FastDiv div_heads;  // by the number of items per query step
     FastDiv div_inner;  // by `inner`
     FastDiv div_group;  // by the query heads per KV head
-    int dynamic;        // more items than SMs
+    int sms, dynamic;   // dynamic: more items than SMs
     int* status;
 };
 
@@ -189,7 +189,9 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     // launch queue, so whoever is done first gets it, whatever the items cost (padding, ragged tiles).  Against a fixed
     // order (item c of every round to CTA c, in alternating direction): 8 x 16/4 heads x 1000 x 1700 with lengths from 300
     // 74 -> 66 us, 2 x 28/4 x 2048 causal 65.6 -> 62.7, 8 x 12 x 1024 causal (an even load) 34.5 -> 34.1.
-    const bool dynamic = p.dynamic != 0;  // else everything runs at once and nothing is left to take
+    // (What the softmax loop gets for registers hangs on where this comes from: without packing a flag from the host costs 3 %, 2 x 16 x
+    // 4000 not causal 247 -> 254 us; with it the comparison does, 1 x 32/8 x 4096 243 -> 250.)
+    const bool dynamic = PACK ? p.dynamic != 0 : p.steps * heads > p.sms;  // else everything runs at once and nothing is left to take
     auto decode = [&](int i) {
         ItemInfo it;
         const int round_q = fast_div(i, p.div_heads);
@@ -908,6 +910,7 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, int B, i
     p.div_heads = make_fastdiv(plan.inner * B);
     p.div_inner = make_fastdiv(plan.inner);
     p.div_group = make_fastdiv(Hq / Hkv);
+    p.sms = sms;
     p.dynamic = plan.items > sms;
     const auto packed = attn_bf16_kernel<D, F16, BIAS, true>, plain = attn_bf16_kernel<D, F16, BIAS, false>;
     const auto kernel = plan.pack > 1 ? packed : plain;
