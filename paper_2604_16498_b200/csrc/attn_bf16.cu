@@ -845,12 +845,44 @@ struct TilePlan {
     long long items;
 };
 
+// When the last item ends, in half-steps of a pair of tiles, if at most a few short items have to wait for an SM; 0 where more do.  A lone
+// tile takes 0.6 of a pair (so do the half-steps that only the later tile of an item has), an item's start and end as long as one.
+inline double end_of_one_round(int pack, int B, int Hq, int Sq, int Skv, bool causal, int sms) {
+    const int rows = 128 / pack, q_tiles = (Sq + rows - 1) / rows, off = Skv - Sq;
+    const long long groups = (long long)(Hq / pack) * B;
+    auto n = [&](int t) {  // half-steps of tile t
+        const long long last = (long long)(t + 1) * rows < Sq ? (t + 1) * rows : Sq, keys = causal && last + off < Skv ? last + off : Skv;
+        return keys > 0 ? (double)((keys + 63) / 64) : 0.;
+    };
+    auto pair = [&](int t) { return 0.6 * n(t) + 0.4 * n(t - 1); };  // tiles t and t - 1
+    if (groups * q_tiles <= sms) return 0.6 * n(q_tiles - 1) + 1;
+    const bool odd = q_tiles % 2 != 0;
+    double longest = odd ? 0.6 * n(q_tiles - 1) : pair(q_tiles - 1);
+    if (odd && q_tiles > 1 && pair(q_tiles - 2) > longest) longest = pair(q_tiles - 2);
+    const long long waiting = groups * ((q_tiles + 1) / 2) - sms;
+    if (waiting <= 0) return longest + 1;
+    // the shortest items of all heads: those that wait start when those that do not have ended, or else the next longer ones
+    if (!causal || q_tiles < 5 || waiting > groups) return 0;
+    const double after = (2 * waiting <= groups ? pair(1) : pair(3)) + pair(1) + 2;
+    return after > longest + 1 ? after : longest + 1;
+}
+
 // One tile per item where that leaves no SM with two of them (a lone tile takes a little more than half the time of a pair: 1 x
 // 16 heads x 518 x 80 12.0 -> 10.5 us, 1 x 32/8 x 256 behind 1000 keys 25.0 -> 20.0), else two.
+// choose_pack() counts scores, which is what many items cost.  Where all run at once the longest one decides, and heads that share a tile
+// do not shorten it: two tiles of 128 rows start 128 keys apart, two of 18 rows see the same, and a tile of several heads takes 4 to 5 %
+// longer.  us, grouped and one head per tile: 2 x 12/4 x 1100 causal 22.1 and 19.7, 1 x 28/4 x 1355 26.7 and 23.6, 2 x 28/4 x 500 13.4 and
+// 12.1, 1 x 32/8 x 512 10.6 and 10.3, 2 x 16/4 x 22 4.95 and 4.49; but with few items left or one tile per item only when grouped
+// 3 x 28/4 x 283 10.1 and 12.7, 2 x 10/2 x 900 15.8 and 18.0; and with a bias, which a CTA's items read once more, 2 x 16/4 x 599 53.6 and 61.3.
 template <int D, bool BIAS>
 TilePlan choose_tiles(int B, int Hq, int Hkv, int Sq, int Skv, int mask_kind, int sms) {
     TilePlan t;
-    const HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, (mask_kind & FORGE_MASK_CAUSAL) != 0, true);
+    const bool causal = (mask_kind & FORGE_MASK_CAUSAL) != 0;
+    HeadPack hp = choose_pack(Hq / Hkv, Sq, Skv, causal, true);
+    if (D > 64 && !BIAS && hp.pack > 1) {
+        const double one_head = end_of_one_round(1, B, Hq, Sq, Skv, causal, sms), grouped = end_of_one_round(hp.pack, B, Hq, Sq, Skv, causal, sms);
+        if (one_head > 0 && (grouped == 0 || one_head <= 1.07 * grouped)) hp = {1, kBM};
+    }
     t.pack = hp.pack; t.head_rows = hp.rows;
     const int q_tiles = (Sq + t.head_rows - 1) / t.head_rows;
     const long long groups = (long long)(Hq / t.pack) * B;

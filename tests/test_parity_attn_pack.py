@@ -41,6 +41,37 @@ def test_rows_around_a_heads_share_of_the_tile(G, rows, D):
         _run(2, 2 * G, 2, Sq, Skv, D, mask)
 
 
+@pytest.mark.parametrize("G,rows", [(2, 64), (3, 42), (4, 32), (5, 25), (6, 21), (7, 18), (8, 16), (12, 10), (15, 8), (16, 8)])
+@pytest.mark.parametrize("D", [64, 128])
+def test_rows_around_a_heads_share_with_many_items(G, rows, D):
+    """Above 64 columns few items, which all run at once, have one head per tile; these do not run at once."""
+    B = 320 // (2 * G) + 1
+    for Sq, Skv, mask in ((rows - 1, 200, 3), (rows + 1, 129, 2), (2 * rows + 3, 2 * rows + 80, 3), (5 * rows + 1, 5 * rows + 1, 1)):
+        w = wl.attention_workload("t", 86, B, 2 * G, 2, Sq, Skv, D, mask, D ** -0.5, "bf16", lens_range=(1, Skv))
+        dl = None
+        if mask & wl.MASK_PADDING:
+            w.lens = np.array(([Skv, 0, 1, 65] * B)[:B], dtype=np.int32)
+            dl = torch.from_numpy(w.lens).cuda()
+        g = Guarded((B, 2 * G, Sq, D), torch.bfloat16)
+        binding.attn_fused(to_device(w.q), to_device(w.k), to_device(w.v), mask, dl, w.scale, out=g.tensor)
+        binding.check_status()
+        pick = np.unique([0, 1, 2, 3, B - 1])  # a period of the lengths and the last entry
+        ref = oracle.attn(w.q.values[pick], w.k.values[pick], w.v.values[pick], mask, w.lens[pick] if dl is not None else None, w.scale)
+        assert_close_bf16(g.tensor[torch.from_numpy(pick).cuda()], ref)
+        assert torch.isfinite(g.tensor.float()).all()
+        g.assert_intact()
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Skv,D,mask", [
+    (1, 28, 4, 1179, 1179, 128, 1),  # pairs of tiles of one head, as many items as SMs or fewer
+    (1, 28, 4, 1355, 1355, 96, 1),   # a few short items wait
+    (2, 10, 2, 900, 900, 128, 1),    # a tile per item with grouped heads only
+    (1, 28, 4, 100, 333, 80, 3),     # a tile per item, one head each
+])
+def test_few_items(B, Hq, Hkv, Sq, Skv, D, mask):
+    _run(B, Hq, Hkv, Sq, Skv, D, mask)
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,Sq,Skv,D,mask", [
     (6, 28, 4, 333, 601, 128, 3),   # more items than SMs, 126 rows in use, empty sequences among full ones
     (40, 16, 4, 130, 130, 80, 1),   # more items than SMs, all rows in use, head size below the kernel's
