@@ -275,7 +275,8 @@ int launch_f32(const float* q, const float* k, const float* v, float* out, int B
     using T = Tile<D, KSPLIT>;
     const dim3 grid((Sq + T::BM - 1) / T::BM, Hq, B);
     // A grid of no more CTAs than SMs takes shared memory for one per SM: launched early, beside the previous kernel's CTAs, two of them would
-    // share an SM that is free already while others fall idle a moment later (1 x 12 x 128 back to back: 8.3 us a call).
+    // share an SM that is free already while others fall idle a moment later.  1 x 12 x 128 without and with it, us: back to back 7.7 and
+    // 5.5, between two linears 6.4 and 5.5, on two streams 8.2 and 7.1 a pair; 1 x 12 x 64 5.1 and 4.9, on two streams 6.1 and 5.1.
     constexpr int kAlone = 116 * 1024;
     const int smem = T::kBytes < kAlone && (long long)grid.x * Hq * B <= sm_count() ? kAlone : T::kBytes;
     FORGE_SET_SMEM_ONCE((attn_f32_kernel<D, KSPLIT>), T::kBytes < kAlone ? kAlone : T::kBytes);
