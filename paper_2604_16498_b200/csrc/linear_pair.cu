@@ -93,12 +93,13 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const int kblocks = (K + kBK - 1) / kBK;
     // Work units.  The tiles of the last, incomplete round of the persistent schedule are cut into two halves of
     // 128 columns (gated: 64 outputs) when that lets them all run at once: the round then takes half as long, which matters
-    // when a pair only gets five or six tiles in all.
+    // when a pair only gets five or six tiles in all.  Gated, whole and halved, us: 320 x 14336 x 4096 (3 tiles a pair and 2 left) 91.5 and
+    // 88.1, 1670 x 8192 x 2048 (6 and 4) 103 and 95, 700 x 4096 x 4096 (1 and 22) 67 and 56.
     const int rem = num_tiles % num_pairs;
     const bool split = rem > 0 && 2 * rem <= num_pairs;
     const int n_whole = split ? num_tiles - rem : num_tiles;
     const int num_units = n_whole + (split ? 2 * rem : 0);
-    // Tiles go down the columns of bands of band_rows row tiles (band_rows_of() has the rule).
+    // Tiles go down the columns of bands of band_rows row tiles (linear_pair_band_rows() has the rule).
     struct Unit { int m0, n0, width; };  // first row and column, columns
     auto unit_of = [&](int u) {
         Unit x;
@@ -331,19 +332,6 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     }
 }
 
-// Row tiles per band of the tile order.  The pairs that run at once should share operands: row by row, the 74 pairs of a round
-// read one row tile of X and 74 column tiles of W, and with N = 14336 (gated: 112 column tiles, 235 MB of W) every row tile reads all of
-// W from HBM again, 7.5 GB a call at 8192 rows.  Down the columns of a band of 16 row tiles a round reads 16 + 5 tiles, and the band's
-// rows of X stay in L2 while W passes once.  Sustained, us, row by row and with bands of 8 / 16 / 24 / 32: 8192 x 14336 x 4096 gated
-// 1665, 1391 / 1352 / 1398 / 1399; 2314 rows 514, 437 / 424 / 427 / 432; 4096 x 14336 x 4096 412, 361 / 357 / 356 / 356; 8192 x 6144 x
-// 4096 323, 317 / 312 / 317 / 337.  A band's rows of X are at most about 48 MB.  Up to 16 column tiles a round of whole rows is nearly
-// square already (8192 x 3072 x 768 37.3, 39.0 with bands of 16; 5027 x 4096 x 4096 130 and 136).
-inline int band_rows_of(int tiles_n, int K) {
-    if (tiles_n <= 16) return 1;
-    const long long fit = (48LL << 20) / (2LL * kBM * 2 * K);
-    return fit < 8 ? 8 : fit > 16 ? 16 : (int)fit;
-}
-
 template <int ACT, bool W_NK, bool F16, bool GATED = false>
 int launch_pair(const void* x, const void* w, const void* b, const void* residual, void* y, int M, int N, int K,
                 cudaStream_t s, const void* w_up = nullptr) {
@@ -391,7 +379,7 @@ int launch_pair(const void* x, const void* w, const void* b, const void* residua
     // the cluster shape is part of the kernel (__cluster_dims__); programmatic stream serialisation as everywhere
     FORGE_CUDA_TRY(launch_pdl(kernel, dim3(2 * pairs), dim3(kThreads), L::kAlloc, s, tmap_x, tmap_w, tmap_w2, tmap_y,
                               static_cast<const uint16_t*>(b), static_cast<const uint16_t*>(residual), M, N, K,
-                              band_rows_of((N + BNO - 1) / BNO, K), status));
+                              linear_pair_band_rows((N + BNO - 1) / BNO, K), status));
     return finish_launch(1);
 }
 
@@ -408,6 +396,21 @@ int dispatch_act(int act, const void* x, const void* w, const void* b, const voi
 }
 
 }  // namespace
+
+// Row tiles per band of the tile order.  The pairs that run at once should share operands: row by row, the 74 pairs of a round
+// read one row tile of X and 74 column tiles of W, and with N = 14336 (gated: 112 column tiles, 235 MB of W) every row tile reads all of
+// W from HBM again, 7.5 GB a call at 8192 rows.  Down the columns of a band of 16 row tiles a round reads 16 + 5 tiles, and the band's
+// rows of X stay in L2 while W passes once.  Sustained, us, row by row and with bands of 8 / 16 / 24 / 32: 8192 x 14336 x 4096 gated
+// 1665, 1391 / 1352 / 1398 / 1399; 2314 rows 514, 437 / 424 / 427 / 432; 4096 x 14336 x 4096 412, 361 / 357 / 356 / 356; 8192 x 6144 x
+// 4096 323, 317 / 312 / 317 / 337.  A band's rows of X take 48 MB at most, but no band has fewer than eight row tiles: above K = 12288,
+// where the 48 MB would allow fewer, us row by row / by the 48 MB / with eight: 8192 x 6144 x 14336 1149 / 1123 / 1083, 4096 x 8192 x 28672
+// 1609 / 1494 / 1453, 4096 x 16384 x 53248 6919 / 6899 / 5481, 4096 x 8192 x 14336 gated 1821 / 1449 / 1435.  Up to 16 column tiles a round
+// of whole rows is nearly square already (8192 x 3072 x 768 37.3, 39.0 with bands of 16; 5027 x 4096 x 4096 130 and 136).
+int linear_pair_band_rows(int tiles_n, int K) {
+    if (tiles_n <= 16) return 1;
+    const long long fit = (48LL << 20) / (2LL * kBM * 2 * K);
+    return fit < 8 ? 8 : fit > 16 ? 16 : (int)fit;
+}
 
 int linear_pair_swiglu(const void* x, const void* w_gate, const void* w_up, void* y, int M, int N, int K, int w_layout,
                        cudaStream_t s) {

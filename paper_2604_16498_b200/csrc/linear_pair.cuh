@@ -9,6 +9,9 @@ namespace forge {
 int linear_pair(bool f16, const void* x, const void* w, const void* b, const void* residual, void* y, int M, int N,
                 int K, int act, int w_layout, cudaStream_t s);
 
+// Row tiles (of 256 rows) in a band of the tile order, for tiles_n column tiles (of 256 columns, gated: 128).
+int linear_pair_band_rows(int tiles_n, int K);
+
 // silu(x Wg) * (x Wu) on CTA pairs (bf16); arguments as forge_linear_swiglu.  Pays whenever M > 128.
 int linear_pair_swiglu(const void* x, const void* w_gate, const void* w_up, void* y, int M, int N, int K, int w_layout,
                        cudaStream_t s);

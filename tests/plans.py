@@ -37,3 +37,16 @@ def split(M, N, K, sms=SMS, gated=False):
         if not f(M, N, K, sms, ctypes.byref(p)):
             return None
     return p.bn, p.split, p.two_per_sm
+
+
+def pair(M, N, K, gated=False, sms=SMS):
+    """The pairs' tiles: (row tiles, column tiles, row tiles of a band, tiles that are cut into halves), or None where the split
+    form is taken."""
+    if M <= 128 or (not gated and split(M, N, K, sms) is not None):
+        return None
+    tiles_m, tiles_n = -(-M // 256), -(-N // (128 if gated else 256))
+    f = binding.load()["_ZN5forge21linear_pair_band_rowsEii"]
+    f.restype, f.argtypes = ctypes.c_int, [ctypes.c_int] * 2
+    pairs = min(tiles_m * tiles_n, sms // 2)
+    rem = tiles_m * tiles_n % pairs
+    return tiles_m, tiles_n, f(tiles_n, K), rem if 2 * rem <= pairs else 0
