@@ -34,8 +34,8 @@ SHAPES = [  # B, Hq, Hkv, Sq, Skv, D, bias heads
     (1, 2, 2, 128, 128, 64, 1),
     (2, 4, 2, 300, 300, 64, 4),     # several tiles, ragged tail, GQA, per-head bias
     (1, 8, 2, 200, 333, 128, 1),    # Skv not a multiple of 4: bias rows off 16-byte boundaries; Sq != Skv
-    (2, 3, 3, 130, 260, 128, 3),    # odd group size at D = 128: consecutive tiles of one head
-    (1, 3, 3, 70, 200, 64, 3),      # odd group size at D = 64: two K/V streams
+    (2, 3, 3, 130, 260, 128, 3),    # odd head count, a ragged second tile
+    (1, 3, 3, 70, 200, 64, 3),      # one tile per head
 ]
 
 

@@ -61,3 +61,32 @@ def test_many_items_with_a_bias():
     binding.check_status()
     ref = oracle.attn_bias(w.q.values[:3], w.k.values[:3], w.v.values[:3], bias[:3].astype(np.float64), wl.MASK_CAUSAL, None, 0.125)
     assert_close_bf16(got[:3], ref)
+
+
+@pytest.mark.parametrize("B,H,Sq,Skv,D,heads", [
+    (24, 15, 100, 200, 64, 1),    # odd head count: the last item of a batch entry has one tile
+    (24, 15, 100, 130, 40, 15),   # a bias per head, head size below the kernel's
+    (10, 9, 130, 70, 64, 1),      # two row tiles per head
+    (11, 16, 90, 261, 56, 16),    # even head count, a ragged last step
+])
+@pytest.mark.parametrize("mask", [wl.MASK_PADDING, wl.MASK_PADDING | wl.MASK_CAUSAL])
+def test_pairs_of_heads_with_a_bias_and_lengths(B, H, Sq, Skv, D, heads, mask):
+    """Up to 64 columns, one head per tile and more tiles than SMs: an item is two heads, each with its own K and V copies.  Unequal
+    streams, empty items among full ones, NaN in the padded rows."""
+    assert B * H * -(-Sq // 128) > 148
+    w = wl.attention_workload("t", 73, B, H, H, Sq, Skv, D, mask, D ** -0.5, "bf16", lens_range=(1, Skv))
+    w.lens = np.array(([Skv, 0, 1, 64, 65, min(128, Skv), 129] * B)[:B], dtype=np.int32).clip(0, Skv)
+    q, k, v = to_device(w.q), to_device(w.k), to_device(w.v)
+    for b in range(B):
+        k[b, :, int(w.lens[b]):] = float("nan")
+        v[b, :, int(w.lens[b]):] = float("nan")
+    bias = wl.normal_tensor(wl.seed_for(73, "b"), (B, heads, Sq, Skv), "f32").values.astype(np.float32)
+    bias[:, :, ::7, 3:60] = -np.inf
+    g = Guarded((B, H, Sq, D), torch.bfloat16)
+    binding.attn_fused_bias(q, k, v, torch.from_numpy(bias).cuda(), mask, torch.from_numpy(w.lens).cuda(), w.scale, out=g.tensor)
+    binding.check_status()
+    pick = np.unique([*range(7), B - 1])
+    ref = oracle.attn_bias(w.q.values[pick], w.k.values[pick], w.v.values[pick], bias[pick].astype(np.float64), mask, w.lens[pick], w.scale)
+    assert_close_bf16(g.tensor[torch.from_numpy(pick).cuda()], ref)
+    assert torch.isfinite(g.tensor.float()).all()
+    g.assert_intact()
