@@ -77,6 +77,10 @@ constexpr int kPiecesPerLane = 1;          // no merge walks through more than 3
 enum { kShort = 0, kGrouped = 1, kTwoLevel = 2 };
 template <int D, int G>
 constexpr int kUpTo32Pieces = D == 128 && G >= 7 ? kTwoLevel : kShort;
+// Whether more than 32 sequences have an instance of their own (LATE below).  With 7 or 8 heads of 128 the shared one is as good or better
+// (40 x 28/4 x 1000 18.9 and 18.9 us, 33 x 32/4 x 3000 30.8 and 31.5).
+template <int D, int G>
+constexpr bool kOwnLate = !(D == 128 && G >= 7);
 constexpr int kMaxGroupedPieces = 20 * kWarps;
 
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
@@ -483,7 +487,10 @@ __device__ __noinline__ void merge_cta(const float* __restrict__ rings, const in
 //                   probabilities exactly where the first MMA left them.
 // Workspace: counters[B * Hkv] and counters of the groups of sixteen pieces [B * Hkv][16] (zero between calls), then ws_o[(b, head, piece)][D] and ws_ml[(b, head, piece)][2]
 // with num_splits piece slots per (batch, head).
-template <int D, int G, bool F16, int MODE>
+// LATE: no look at the lengths before the previous kernel has completed, for more than 32 sequences (see `early`).  An instance of its own, for
+// up to 32 pieces: as a run-time choice the streaming loop got other registers and lost what there is nothing to gain for (us, run-time choice
+// and own instance: 33 x 12/12 x 10,591 of 64 135.3 and 127.2, 40 x 12/12 x 1000 of 64 26.1 and 25.0, 64 x 12/12 x 300 of 64 19.3 and 18.6).
+template <int D, int G, bool F16, int MODE, bool LATE>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
                     const uint16_t* __restrict__ q, const int32_t* __restrict__ lens, uint16_t* __restrict__ out,
@@ -526,7 +533,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
     // made again, in the same code: with a second copy of it behind the first the streaming loop of 7 heads of 128 got other registers and was
     // 6 % slower (16 x 28/4 x 10,442 42.2 -> 40.1 us, 4 x 28/4 x 10,000 22.8 -> 20.1; 24 x 32/8 x 3000 21.0 -> 20.8).
     // (More than 32 sequences: the schedule reads lens several times and is made once, afterwards.)
-    const bool early = B <= 32;
+    const bool early = !LATE && B <= 32;
     if (!early) pdl_wait();
     bool waited = !early;
     Schedule sched;
@@ -573,31 +580,40 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
     };
     bool failed = false;
     int n = 0;  // blocks consumed
-#pragma unroll 1
-    for (;;) {
+    if constexpr (LATE) {
         sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
-        first_idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
-        p_round = 0;
+        first_idx = (unsigned)worker;
         p_idx = item_of_round(0);
         p_open();
-        if (!waited) {
-            const int row = p_j0 + lane * kBlockKeys;
-            if (p_idx < sched.num_items && lane < kStages && row < p_s1) {
-#pragma unroll
-                for (int cb = 0; cb < D / 64; ++cb) {
-                    ptx::tma_prefetch_l2_3d(&tmap_k, cb * 64, row, p_bk);
-                    ptx::tma_prefetch_l2_3d(&tmap_v, cb * 64, row, p_bk);
-                }
-            }
-            pdl_wait();
-        }
-        const int len_now = !waited && lane < B ? first_len(lens, lane, Smax) : sched.len0;
 #pragma unroll
         for (int i = 0; i < kStages; ++i) issue();
-        if (__all_sync(0xffffffffu, sched.len0 == len_now)) break;
-        waited = true;
-        for (; n < p_n && !failed; ++n) failed = !ptx::warp_wait(&full[n % kStages], (n / kStages) & 1);
-        if (failed) break;
+    } else {
+#pragma unroll 1
+        for (;;) {
+            sched = make_schedule<MODE>(lens, B, Hkv, Smax, num_splits, workers, lane);
+            first_idx = MODE == kGrouped && sched.grouped ? blockIdx.x * kWarps + warp : (unsigned)worker;
+            p_round = 0;
+            p_idx = item_of_round(0);
+            p_open();
+            if (!waited) {
+                const int row = p_j0 + lane * kBlockKeys;
+                if (p_idx < sched.num_items && lane < kStages && row < p_s1) {
+#pragma unroll
+                    for (int cb = 0; cb < D / 64; ++cb) {
+                        ptx::tma_prefetch_l2_3d(&tmap_k, cb * 64, row, p_bk);
+                        ptx::tma_prefetch_l2_3d(&tmap_v, cb * 64, row, p_bk);
+                    }
+                }
+                pdl_wait();
+            }
+            const int len_now = !waited && lane < B ? first_len(lens, lane, Smax) : sched.len0;
+#pragma unroll
+            for (int i = 0; i < kStages; ++i) issue();
+            if (__all_sync(0xffffffffu, sched.len0 == len_now)) break;
+            waited = true;
+            for (; n < p_n && !failed; ++n) failed = !ptx::warp_wait(&full[n % kStages], (n / kStages) & 1);
+            if (failed) break;
+        }
     }
     const unsigned num_items = sched.num_items;
     if (MODE == kGrouped && sched.grouped && lane == 0) merge_info[warp][0] = -1;
@@ -847,7 +863,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
     }
 }
 
-template <int D, int G, bool F16, int MODE>
+template <int D, int G, bool F16, int MODE, bool LATE = false>
 int launch_split(const void* q, const void* kc, const void* vc, const int32_t* lens, void* out, unsigned int* counters,
                  float* ws_o, float* ws_ml, int B, int Hq, int Hkv, int Smax, int head_dim, int num_splits,
                  float scale_log2, cudaStream_t s) {
@@ -863,7 +879,7 @@ int launch_split(const void* q, const void* kc, const void* vc, const int32_t* l
         if (!encode_tmap_bf16_sw128(&tk, kc, 3, dims, strides, box)) return FORGE_ERR_CUDA;
         if (!encode_tmap_bf16_sw128(&tv, vc, 3, dims, strides, box)) return FORGE_ERR_CUDA;
     }
-    auto kernel = decode_split_kernel<D, G, F16, MODE>;
+    auto kernel = decode_split_kernel<D, G, F16, MODE, LATE>;
     FORGE_SET_SMEM_ONCE(kernel, kSmem);
     const int sms = sm_count();
     if (sms <= 0) return FORGE_ERR_CUDA;
@@ -884,11 +900,12 @@ int dispatch_g(int G, const void* q, const void* kc, const void* vc, const int32
                int num_splits, float scale_log2, cudaStream_t s) {
     // no more pieces than this can exist, whatever lens holds
     const long long blocks_max = (Smax + kBlockKeys - 1) / kBlockKeys, most = blocks_max < num_splits ? blocks_max : num_splits;
-    const bool few = most <= kSingleLevelPieces;
+    const bool few = most <= kSingleLevelPieces, late = B > 32;
     const bool grouped = most <= kMaxGroupedPieces && most * B * Hkv <= (long long)sm_count() * kWarps;
 #define FORGE_DECODE_CASE(g)                                                                                     \
     case g:                                                                                                      \
-        return few       ? launch_split<D, g, F16, kUpTo32Pieces<D, g>>(FORGE_DECODE_ARGS)                       \
+        return few       ? late ? launch_split<D, g, F16, kUpTo32Pieces<D, g>, kOwnLate<D, g>>(FORGE_DECODE_ARGS) \
+                                : launch_split<D, g, F16, kUpTo32Pieces<D, g>>(FORGE_DECODE_ARGS)                \
                : grouped ? launch_split<D, g, F16, kGrouped>(FORGE_DECODE_ARGS)                                  \
                          : launch_split<D, g, F16, kTwoLevel>(FORGE_DECODE_ARGS)
 #define FORGE_DECODE_ARGS \
