@@ -67,8 +67,9 @@ def test_rows_around_a_heads_share_with_many_items(G, rows, D):
     (1, 28, 4, 1355, 1355, 96, 1),   # a few short items wait
     (2, 10, 2, 900, 900, 128, 1),    # a tile per item with grouped heads only
     (1, 28, 4, 100, 333, 80, 3),     # a tile per item, one head each
+    (6, 28, 4, 250, 300, 80, 2),     # more items than SMs, as many tiles as with grouped heads
 ])
-def test_few_items(B, Hq, Hkv, Sq, Skv, D, mask):
+def test_one_head_per_tile_or_more(B, Hq, Hkv, Sq, Skv, D, mask):
     _run(B, Hq, Hkv, Sq, Skv, D, mask)
 
 
