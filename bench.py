@@ -52,7 +52,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 NOMINAL_PEAKS = {"hbm_gbs": 8000.0, "bf16_tflops": 2250.0}
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised under
 # profiles/ (None once the kernel has changed since the capture).
-NCU_TRAFFIC_BYTES = {"attention": None, "linear": 19230000, "decode": None}
+NCU_TRAFFIC_BYTES = {"attention": 133615104, "linear": 19230000, "decode": 146330000}
 
 
 def load_peaks():

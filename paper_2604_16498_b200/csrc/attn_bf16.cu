@@ -33,7 +33,8 @@
 // The CTA's last output is stored by the softmax warps, each its own rows, without the way through warp 11: with one item
 // per CTA that is 0.4 us (6 x 12 heads x 385 causal, D = 128, 12.56 -> 12.15).
 // Reading the output only after the next item's first half-step gained nothing more and cost short items their overlap
-// (64 x 16/4 x 64: 16.7 -> 21.3 us).  At D = 128 long runs are at the power limit: fewer cycles, lower clock.
+// (64 x 16/4 x 64: 16.7 -> 21.3 us).  At D = 128 a run of seconds is at the power limit (4 x 32/8 x 2048 130 us at 1965 MHz in a few calls,
+// 150 at 1620 MHz later on): there fewer cycles are a lower clock.
 #include <type_traits>
 
 #include "attn_math.cuh"
