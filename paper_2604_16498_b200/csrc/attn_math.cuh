@@ -49,7 +49,8 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
 
 // 2^x for two values on the FMA and integer pipes instead of the special-function unit (which is the
 // narrowest pipe of the softmax): x = n + f with n = round(x), f in [-0.5, 0.5]; 2^f by a cubic with a
-// relative error of 7.6e-5 (far below the bf16 rounding of P); n is added to the exponent field.
+// relative error of 7.6e-5 (far below the bf16 rounding of P); n is added to the exponent field.  The coefficients, here and below, are
+// the polynomial's with the least largest relative error on that range (it swings between plus and minus that error).
 // Inputs below -125, -infinity and NaN give 2^-125, so this is used only where no score is masked or NaN and the row's reference is finite.
 __device__ __forceinline__ float2 ex2_fma2(float2 x) {
     const float kMagic = 12582912.f;  // 1.5 * 2^23: adding it leaves round(x) in the low mantissa bits
