@@ -250,8 +250,9 @@ attn_wide_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         // ------------------------------------------------------------------ softmax / rescale / epilogue
         const int row = warp * 32 + lane;
         // head and query row within the tile; a row that is not in use goes along as the last head's first with Q = 0
-        const bool live = row < pack * head_rows;
-        const int row_h = min(row / head_rows, pack - 1), row_q = live ? row - row_h * head_rows : 0;
+        // (without packing both are known at compile time: 30 x 16 x 100 not causal 32.5 -> 32.0 us, 18 x 12 x 17 causal 9.9 -> 9.7)
+        const bool live = !PACK || row < pack * head_rows;
+        const int row_h = PACK ? min(row / head_rows, pack - 1) : 0, row_q = !PACK ? row : live ? row - row_h * head_rows : 0;
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
         const float sl2 = p.scale_log2;
         int steps[2] = {0, 0};  // steps done so far per parity (phases of s_full, pv_done)
