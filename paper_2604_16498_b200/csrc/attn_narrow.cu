@@ -391,13 +391,14 @@ int launch_narrow(const void* q, const void* k, const void* v, void* out, int B,
     const long long tiles = (long long)B * (Hq / hp.pack) * ((Sq + hp.rows - 1) / hp.rows);
     if (tiles > 2147483647LL) return FORGE_ERR_UNSUPPORTED;
     // Launched early, beside the previous kernel's, three CTAs would share an SM that is free already while others fall idle a moment
-    // later.  So a grid of up to two CTAs per SM takes shared memory for two, and one that leaves half of the SMs to others for one.  (One
-    // each for up to all SMs would keep a second stream's grid out until the first has ended: two streams of 12 x 12 heads x 128,
-    // us a pair: three per SM 6.0, two 5.7, one 10.0; 6 x 12 x 256 7.6, 7.1, 11.3.)  The same call in a chain, three / two / one per SM:
-    // 12 x 12 x 128 6.1 / 5.4 / 5.1, 4 x 12 x 128 4.7 / 4.6 / 4.5, 2 x 12 x 512 9.6 / 9.6 / 8.8.  GPT-2-small layers, 1 x 512 42.5 / 40.2 /
-    // 39.1, 2 x 256 38.3 / 37.1 / 36.5, 2 x 128 31.2 / 31.7 / 31.6; layers of 32/8 heads of 64, width 2048, 2 x 128 56.7 / 56.7 / 58.6 (its
-    // CTA of 116 KB sets up only when the projection's has left), 2 x 256 79.4 / 81.1 / 81.0.
-    const int sms = sm_count(), smem = 2 * tiles <= sms ? kAlone : tiles <= 2LL * sms ? kTwo : L::kAlloc;
+    // later.  So a grid of up to two CTAs per SM takes shared memory for two, and one that leaves a quarter of the SMs to others for one.
+    // (One each for up to all SMs keeps a second stream's grid out until the first has ended.)  Three / two / one per SM, us.  Two streams, a
+    // pair of calls: 8 x 12 heads x 128 (96 tiles) 5.8 / 5.2 / 6.9, 3 x 12 x 384 (108) 8.7 / 8.5 / 9.6, 12 x 12 x 128 (144) 6.0 / 5.7 / 10.0,
+    // 6 x 12 x 256 (144) 7.6 / 7.1 / 11.3; the kernel before this one took 6.7, 10.5, 7.1 and 9.0.  The same call in a chain: 8 x 12 x 128
+    // 5.5 / 5.1 / 4.8, 3 x 12 x 384 9.0 / 8.0 / 7.4, 12 x 12 x 128 6.1 / 5.4 / 5.1, 6 x 12 x 256 7.9 / 7.0 / 6.0.  GPT-2-small layers, 1 x 512
+    // 42.5 / 40.2 / 39.1, 2 x 256 38.3 / 37.1 / 36.5, 2 x 128 31.2 / 31.7 / 31.6; layers of 32/8 heads of 64, width 2048, 2 x 128 56.7 / 56.7 /
+    // 58.6 (its CTA of 116 KB sets up only when the projection's has left), 2 x 256 79.4 / 81.1 / 81.0.
+    const int sms = sm_count(), smem = 4 * tiles <= 3LL * sms ? kAlone : tiles <= 2LL * sms ? kTwo : L::kAlloc;
     FORGE_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)tiles), dim3(kThreads), smem, s, tq, tk, tv, to, p));
     return finish_launch(1);
 }
